@@ -88,7 +88,7 @@ struct dags_ctx {
   TrackGraph graph;
   TrackGraph graph_lm;            // captured LM iteration
   LmBuffers lm;                   // allocated by the first LM call
-  uint32_t *warp_masks = nullptr; // [max_tiles][kMaskGroups][8] forward masks of the tracking loop
+  uint32_t *warp_masks = nullptr; // [max_v * max_tiles][kMaskGroups][8] the last forward's records for its adjoint
   uint32_t *cand_ids = nullptr;   // [max_n] the tracking frame's culled candidates
   uint32_t *cand_n = nullptr;     // [1]
   float *cull_pose = nullptr;     // [12]
@@ -108,6 +108,7 @@ struct dags_ctx {
   const void *fwd_gauss = nullptr;
   int64_t fwd_n = -1;
   int fwd_views = 0, fwd_w = 0, fwd_h = 0, fwd_tiles = 0;
+  float fwd_log2_alpha_min = 0.f;   // the threshold its recorded masks hold for
 };
 
 namespace {
@@ -322,7 +323,7 @@ int dags_create(dags_ctx **out, int64_t max_gaussians, int32_t max_width, int32_
   A(alloc(&w.vis_n, (size_t)w.max_v));
   A(alloc(&w.counters, (size_t)CNT_N));
   A(alloc(&w.evals, (size_t)4));
-  A(alloc(&c->warp_masks, (size_t)w.max_tiles * kMaskGroups * 8));
+  A(alloc(&c->warp_masks, vt * kMaskGroups * 8));
   A(alloc(&c->cand_ids, (size_t)w.max_n));
   A(alloc(&c->cand_n, (size_t)1));
   A(alloc(&c->cull_pose, (size_t)12));
@@ -444,7 +445,10 @@ int splat_forward(dags_ctx *ctx, const float *gauss, int64_t n, const dags_camer
   cudaStream_t s = (cudaStream_t)stream;
   ctx->last_stream = s;
   ctx->fwd_image = nullptr;
-  const Workspace &w = ctx->ws;
+  Workspace w = ctx->ws;
+  // the forward records, per warp, which list entries its pixels took; the
+  // adjoint that follows it visits only those
+  w.warp_masks = ctx->warp_masks;
   const float4 *g4 = reinterpret_cast<const float4 *>(gauss);
   KernelTimer &tm = ctx->timer;
   int ev = tm.begin(DAGS_K_PREPROCESS, s);
@@ -469,6 +473,7 @@ int splat_forward(dags_ctx *ctx, const float *gauss, int64_t n, const dags_camer
   ctx->fwd_w = cam->width;
   ctx->fwd_h = cam->height;
   ctx->fwd_tiles = r.T;
+  ctx->fwd_log2_alpha_min = r.log2_alpha_min;
   return DAGS_OK;
 }
 
@@ -490,6 +495,18 @@ int dags_copy_bins(dags_ctx *ctx, uint32_t *tile_start, int64_t n_start, uint32_
     return DAGS_E_CUDA;
   return DAGS_OK;
 }
+
+}  // extern "C"
+
+// The workspace of the adjoint of the ctx's last forward: with the entries
+// that forward recorded, unless the adjoint is asked for another alpha_min.
+static Workspace backward_workspace(const dags_ctx *ctx, const Raster &r) {
+  Workspace w = ctx->ws;
+  w.warp_masks = r.log2_alpha_min == ctx->fwd_log2_alpha_min ? ctx->warp_masks : nullptr;
+  return w;
+}
+
+extern "C" {
 
 int splat_backward(dags_ctx *ctx, const float *gauss, int64_t n, const dags_camera *cam, const double *poses,
                    int32_t n_views, const float *targets, const dags_raster_cfg *rcfg,
@@ -514,8 +531,8 @@ int splat_backward(dags_ctx *ctx, const float *gauss, int64_t n, const dags_came
   const bool full = (grad_flags & DAGS_GRAD_GAUSS) != 0;
   KernelTimer &tm = ctx->timer;
   int ev = tm.begin(DAGS_K_RENDER_BWD, s);
-  cudaError_t e = launch_render_bwd(ctx->ws, n_views, n, r, l, reinterpret_cast<const float4 *>(targets),
-                                    image, last, full, s);
+  cudaError_t e = launch_render_bwd(backward_workspace(ctx, r), n_views, n, r, l, reinterpret_cast<const float4 *>(targets),
+                                    image, last, full, (grad_flags & DAGS_GRAD_POSE) != 0, s);
   tm.end(ev, s);
   if (e == cudaSuccess) {
     ev = tm.begin(DAGS_K_PREPROCESS_BWD, s);
@@ -550,7 +567,7 @@ int splat_backward_upstream(dags_ctx *ctx, const float *gauss, int64_t n, const 
   const bool full = (grad_flags & DAGS_GRAD_GAUSS) != 0;
   KernelTimer &tm = ctx->timer;
   int ev = tm.begin(DAGS_K_RENDER_BWD, s);
-  cudaError_t e = launch_render_bwd(ctx->ws, n_views, n, r, l, nullptr, image, last, full, s, grad_image);
+  cudaError_t e = launch_render_bwd(backward_workspace(ctx, r), n_views, n, r, l, nullptr, image, last, full, (grad_flags & DAGS_GRAD_POSE) != 0, s, grad_image);
   tm.end(ev, s);
   if (e == cudaSuccess) {
     ev = tm.begin(DAGS_K_PREPROCESS_BWD, s);
@@ -685,7 +702,7 @@ int track_iteration(dags_ctx *ctx, const float *gauss, int64_t n, const dags_cam
   }
   if (e == cudaSuccess) {
     ev = tm.begin(DAGS_K_RENDER_BWD, s);
-    e = launch_render_bwd(w, 1, n, r, l, reinterpret_cast<const float4 *>(targets), image, last, false, s);
+    e = launch_render_bwd(w, 1, n, r, l, reinterpret_cast<const float4 *>(targets), image, last, false, true, s);
     tm.end(ev, s);
   }
   if (e == cudaSuccess) {

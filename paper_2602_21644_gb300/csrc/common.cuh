@@ -36,8 +36,14 @@ __device__ __forceinline__ bool dags_in_bounds(bool ok, uint32_t *status) {
 #define DAGS_IN_BOUNDS(cond, status) true
 #endif
 
-// 2D gradient slots per (view, Gaussian).
-enum { G2_U = 0, G2_V, G2_A, G2_B, G2_C, G2_Z, G2_O, G2_R, G2_G, G2_BL };
+// 2D gradient slots per (view, Gaussian), sums over the pixels it covers.
+// With g = alpha dL/dalpha (0 where alpha is clamped) and d = centre - pixel:
+//   moments      words 0-4: g dx, g dy, g dx^2, g dx dy, g dy^2, of which the
+//                gradients of centre and conic are linear combinations
+//   otherwise    words 0-4: the gradients of the centre (u, v) and of the conic
+//                (a, b, c) themselves
+// and in both the gradient of depth, the sum of g, and those of the colour.
+enum { G2_U = 0, G2_V, G2_A, G2_B, G2_C, G2_Z, G2_S0, G2_R, G2_G, G2_BL };
 
 // Counters in the workspace's counter array.
 enum {
@@ -106,8 +112,8 @@ struct Workspace {
   uint32_t bucket_cap = 0;
   // Per tile, warp and 32-entry group of the first kMaskGroups groups: the
   // entries at least one pixel of the warp took in the forward (one bit
-  // each), for the adjoint of the same iteration; null: not recorded.
-  uint32_t *warp_masks = nullptr;   // [max_tiles][kMaskGroups][8]
+  // each), for the adjoint of the same forward; null: not recorded.
+  uint32_t *warp_masks = nullptr;   // [V * T][kMaskGroups][8]
   // Per-frame culling of the tracking loop: the candidates of the frame's
   // starting pose (cull_pose, FP32 3x4) and their count; null: no culling.
   uint32_t *cand_ids = nullptr;     // [max_n]
@@ -188,10 +194,13 @@ cudaError_t launch_order_identity(uint32_t *order, int tiles, cudaStream_t s);
 cudaError_t launch_render_fwd(const Workspace &ws, int views, int64_t n, const Raster &r, const Loss &l,
                               const float4 *targets, float *image, int32_t *last, double *loss,
                               cudaStream_t s);
+// full, pose: the gradients that the launch_preprocess_bwd after it is asked
+// for (the Gaussians', the twists'); the two agree on the form of the 2D
+// gradients by them.
 // upstream (V x 6 x P, or null): a caller's gradients of the composited
 // channels (C_r, C_g, C_b, D, O, R_MP) used in place of the loss's
 cudaError_t launch_render_bwd(const Workspace &ws, int views, int64_t n, const Raster &r, const Loss &l,
-                              const float4 *targets, const float *image, const int32_t *last, bool full,
+                              const float4 *targets, const float *image, const int32_t *last, bool full, bool pose,
                               cudaStream_t s, const float *upstream = nullptr);
 cudaError_t launch_preprocess_bwd(const Workspace &ws, const float4 *gauss, int64_t n, int views,
                                   const Raster &r, float *grad_gauss, double *grad_pose, const PoseStep &ps,
@@ -581,16 +590,15 @@ __device__ __forceinline__ bool ellipse_reaches_rect(float u, float v, float A2,
   return best <= thr;
 }
 
-// Reduce-scatter of K values over the 32 lanes of a warp. Each of the five
-// xor levels (16, 8, 4, 2, 1) halves the lane's list: the lane keeps one half
-// and adds its partner's copy of that half; an odd last entry is summed whole
-// and stays with both partners. On return every lane holds the full warp sum
-// of one component, rs_component<K>(lane). Shuffles: 8 for K = 6, 9 for
-// K = 8, 12 for K = 10 (against 5 K for separate warp sums).
-template <int K, int M = 16>
+// Reduce-scatter of K values over groups of 2 M lanes. Each xor level (M,
+// M / 2, ..., 1) halves the lane's list: the lane with that bit set keeps the
+// second half, the other the first, and adds its partner's copy of it; an odd
+// last entry is summed whole and stays with both partners. On return every
+// lane holds the group's sum of one component.
+template <int K, int M>
 __device__ __forceinline__ float warp_reduce_scatter(const float (&cur)[K], int lane) {
   constexpr int P = K / 2, K2 = P + (K & 1);
-  static_assert(M > 1 || K2 == 1, "at most 32 components");
+  static_assert(M > 1 || K2 == 1, "at most 2 M components");
   const bool hi = (lane & M) != 0;
   float nxt[K2];
 #pragma unroll
@@ -607,9 +615,9 @@ __device__ __forceinline__ float warp_reduce_scatter(const float (&cur)[K], int 
   }
 }
 
-// The component whose sum warp_reduce_scatter<K> leaves in lane `lane`: the
+// The component whose sum warp_reduce_scatter<K, 16> leaves in lane `lane`: the
 // same selections applied to the component indices.
-template <int K, int M = 16>
+template <int K, int M>
 __device__ __forceinline__ int rs_component_of(const int (&cur)[K], int lane) {
   constexpr int P = K / 2, K2 = P + (K & 1);
   const bool hi = (lane & M) != 0;
@@ -629,7 +637,7 @@ __device__ __forceinline__ int rs_component(int lane) {
   int ids[K];
 #pragma unroll
   for (int i = 0; i < K; ++i) ids[i] = i;
-  return rs_component_of<K>(ids, lane);
+  return rs_component_of<K, 16>(ids, lane);
 }
 
 // FP64 Adam step on the twist of one pose followed by T <- exp(xi^) T, with

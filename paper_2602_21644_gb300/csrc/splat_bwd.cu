@@ -5,10 +5,10 @@
 //                          contributor, re-deriving each pixel's
 //                          transmittance from its final value (T_k =
 //                          T_{k+1} / (1 - alpha_k)) with running suffix sums,
-//                          so no per-pair state is stored; the per-Gaussian
-//                          2D gradients of the 32 pixels of a warp are summed
-//                          with shuffles and added with one atomic per
-//                          Gaussian per warp.
+//                          so no per-pair state is stored; the 2D-gradient
+//                          moments of the 32 pixels of a warp are summed with
+//                          shuffles and added with one atomic per word per
+//                          (warp, Gaussian) pair.
 //   preprocess_bwd_kernel  per Gaussian over all views: chains the 2D
 //                          gradients through conic, EWA covariance, Jacobian,
 //                          camera transform, scale and rotation to the record's
@@ -24,13 +24,59 @@ namespace dags {
 namespace {
 
 constexpr int kMaxViewsSmem = 64;
-// the reduce-scatter's component k is 2D-gradient word k
-static_assert(G2_U == 0 && G2_Z == 5 && G2_BL == 9 && kGradWords >= 10, "2D-gradient word order");
+// the pose path's words are the first two float4 (the preprocess zeroes only those)
+static_assert(G2_U == 0 && G2_C == 4 && G2_Z == 5 && G2_BL == 9 && kGradWords >= 10, "2D-gradient word order");
+
+// Warp sums of an entry's moments over the warp's 8 x 4 pixels (lane = 8 row +
+// column). dx depends on the column only and dy on the row only, so m0, m1, m2
+// = g, g dx, g dx^2 and the depth and colour terms are first reduce-scattered
+// over each row's 8 lanes, and the y factors are applied to the row sums: 7 + 2
+// shuffles for the ten words and 4 + 2 for the pose path's six (a
+// reduce-scatter of all words over 32 lanes takes 12 and 8, and needs every
+// word formed per pixel). After the row stage lane l8 = lane & 7 holds
+//   FULL:      m1, m2, z, m0, r, g, b, m0
+//   pose only: m1, m1, m2, m2, z, z, m0, m0
+// and the rows are summed as is by the lanes below 16, weighted with dy by the
+// others, with l8 = 7 taking dy^2. moment_word: the word a lane ends up with
+// (-1: it writes none).
+template <bool FULL>
+__device__ __forceinline__ int moment_word(int lane) {
+  const int l8 = lane & 7;
+  if (lane & 8) return -1;
+  if (lane & 16) return l8 == 0 ? G2_B : (l8 == (FULL ? 3 : 6) ? G2_V : -1);
+  if (l8 == 0) return G2_U;
+  if (l8 == 7) return G2_C;
+  if (FULL) return l8 == 1 ? G2_A : l8 == 2 ? G2_Z : l8 == 3 ? G2_S0 : l8 == 4 ? G2_R : l8 == 5 ? G2_G : G2_BL;
+  return l8 == 2 ? G2_A : l8 == 4 ? G2_Z : -1;
+}
+
+template <bool FULL>
+__device__ __forceinline__ float moment_sums(float m0, float m1, float m2, float gz, float gr, float gg, float gb,
+                                             float dy, int lane) {
+  const unsigned FULLM = 0xffffffffu;
+  float v;
+  if constexpr (FULL) {
+    const float x[7] = {m1, m2, gz, gr, gg, gb, m0};
+    v = warp_reduce_scatter<7, 4>(x, lane);
+  } else {
+    const float x[4] = {m1, m2, gz, m0};
+    v = warp_reduce_scatter<4, 4>(x, lane);
+  }
+  const float b = v * dy;
+  const float a = (lane & 7) == 7 ? b * dy : v;
+  const bool hi = (lane & 16) != 0;
+  const float keep = hi ? b : a, send = hi ? a : b;
+  const float s = keep + __shfl_xor_sync(FULLM, send, 16);
+  return s + __shfl_xor_sync(FULLM, s, 8);
+}
 
 // FULL: every parameter's 2D gradients (else the pose path's six words);
+// MOMENTS: words 0-4 as moments (see G2_U), else as gradients formed per pixel;
 // MASKS: visit only the entries the forward recorded as taken by the warp
 // (ws.warp_masks); COUNT: count evaluations and contributions (ws.evals).
-template <bool FULL, bool MASKS, bool COUNT>
+// Bound by instruction issue (75-87% issue-active): a pair costs its loop, its
+// loads, the arithmetic per pixel and the warp's reduction.
+template <bool FULL, bool MOMENTS, bool MASKS, bool COUNT>
 __global__ void __launch_bounds__(kTilePix, 5)
 render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ targets,
                   const float *__restrict__ image, const int32_t *__restrict__ last,
@@ -39,7 +85,10 @@ render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ tar
   pdl_trigger();
   __shared__ float4 s_a[kTilePix], s_b[kTilePix], s_c[kTilePix];   // s_a: {u hi, v hi, u lo, v lo}
   __shared__ float2 s_e[kTilePix];                                  // box half extents
-  __shared__ float *s_dst[kTilePix];                                // the entry's 2D-gradient words
+  __shared__ float s_bl[kTilePix];                                  // s_c: {z, M, r, g}; blue here
+  // the entry's slot (32 bits: 2^32 slots would need 400 GB of records and
+  // gradients)
+  __shared__ uint32_t s_slot[kTilePix];
   __shared__ int s_max;
   const unsigned FULLM = 0xffffffffu;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -56,11 +105,17 @@ render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ tar
     const uint64_t tot = (uint64_t)ws.counters[CNT_REQ_LO] | ((uint64_t)ws.counters[CNT_REQ_HI] << 32);
     if (tot > (uint64_t)ws.max_pairs) return;
   }
-  // the 2D-gradient word whose warp sum this lane receives from the
-  // reduce-scatter below (words G2_U .. G2_Z, and with FULL up to G2_BL), and
-  // whether it is the lowest lane holding that word (the one that adds it)
-  const int comp = FULL ? rs_component<10>(lane) : rs_component<6>(lane);
-  const bool writer = __ffs(__match_any_sync(0xffffffffu, (unsigned)comp)) - 1 == lane;
+  // the 2D-gradient word whose warp sum this lane adds, if any (of the lanes
+  // that hold one word, the lowest)
+  int word;
+  if constexpr (MOMENTS) {
+    word = moment_word<FULL>(lane);
+  } else {
+    word = rs_component<10>(lane);
+    if (__ffs(__match_any_sync(FULLM, (unsigned)word)) - 1 != lane) word = -1;
+  }
+  const bool writer = word >= 0;
+  float *const gdst = ws.grad2d + (writer ? word : 0);
   const int tile = (int)ws.tile_order[blockIdx.x];   // longest lists first
   const int v = tile / r.T, tv = tile - v * r.T;
   const int tx = tv % r.tiles_x, ty = tv / r.tiles_x;
@@ -137,13 +192,16 @@ render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ tar
       uint32_t id = ws.sorted_ids[s + beg + tid];
       if (!DAGS_IN_BOUNDS(id < (uint32_t)ws.max_n, ws.counters + CNT_STATUS)) id = 0;
       const size_t slot = vbase + id;
-      s_dst[tid] = ws.grad2d + slot * kGradWords;
+      s_slot[tid] = (uint32_t)slot;
       const float4 r0 = ws.rec2d[slot * 3 + 0];
       const float2 lo = ws.rec_lo[slot];
       s_a[tid] = make_float4(r0.x, r0.y, lo.x, lo.y);
       s_e[tid] = make_float2(r0.z, r0.w);
       s_b[tid] = ws.rec2d[slot * 3 + 1];
-      s_c[tid] = ws.rec2d[slot * 3 + 2];
+      const float4 r2 = ws.rec2d[slot * 3 + 2];
+      const uint32_t rg = __float_as_uint(r2.z), bl = __float_as_uint(r2.w);
+      s_c[tid] = make_float4(r2.x, r2.y, bf16_lo(rg), bf16_hi(rg));
+      s_bl[tid] = bf16_lo(bl);
     }
     __syncthreads();
     const int cnt = end - beg;
@@ -183,57 +241,41 @@ render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ tar
         const bool contrib = k < lastp && p >= r.log2_alpha_min;
         if (COUNT) { n_eval += k < lastp ? 1u : 0u; n_contrib += contrib ? 1u : 0u; }
         const float ag = hw_exp2(p);
-        const float alpha = fminf(r.alpha_max, ag);
+        // zero for a lane that does not take the entry: 1 / (1 - alpha) is
+        // then exactly 1, T is kept, and the weight and the suffix update
+        // vanish without a select
+        const float alpha = contrib ? fminf(r.alpha_max, ag) : 0.f;
         const float inv = hw_rcp(1.f - alpha);
-        T = contrib ? T * inv : T;           // transmittance in front of this Gaussian
-        // the weight, zero for a lane that does not take the entry (its
-        // depth gradient and suffix update then vanish without a select)
-        const float wk = contrib ? alpha * T : 0.f;
+        T *= inv;                            // transmittance in front of this Gaussian
+        const float wk = alpha * T;
         const float4 c = s_c[j];
-        const uint32_t rgb = __float_as_uint(c.z), blb = __float_as_uint(c.w);
-        const float fr = bf16_lo(rgb), fg = bf16_hi(rgb), fb = bf16_lo(blb);
         // dL/dalpha = sum_ch g_ch (c_ch T - S_ch / (1 - alpha))
-        const float gcv = fmaf(g0, fr, fmaf(g1, fg, fmaf(g2, fb, fmaf(g3, c.x, fmaf(g5, c.y, g4)))));
+        const float gcv = fmaf(g0, c.z, fmaf(g1, c.w, fmaf(g2, s_bl[j], fmaf(g3, c.x, fmaf(g5, c.y, g4)))));
         const float dal = fmaf(gcv, T, -Sg * inv);
+        // below the clamp, d alpha / d(natural exponent) = alpha (at the clamp
+        // alpha does not move with the exponent)
+        const float dpw = contrib && ag <= r.alpha_max ? dal * alpha : 0.f;
         const float gz = g3 * wk;
-        float gr = 0.f, gg = 0.f, gbl = 0.f, go = 0.f;
-        if (FULL) {
-          gr = g0 * wk;
-          gg = g1 * wk;
-          gbl = g2 * wk;
-        }
-        // below the clamp, d alpha / d(natural exponent) = alpha; the
-        // exponent in log2 units is p, so d/dx of the natural exponent is
-        // ln2 * dp/dx (at the clamp alpha does not move with the exponent)
-        const bool slope = contrib && ag <= r.alpha_max;
-        const float dpw = slope ? dal * alpha : 0.f;
-        const float hl = dpw * kLn2;
-        // d p / d(u, v) = (2 a' dx + b' dy, b' dx + 2 c' dy) from the
-        // exponent's products; d(natural exponent) / d(conic) = -(dx^2 / 2,
-        // dx dy, dy^2 / 2)
-        const float gu = hl * fmaf(2.f, bxdx, b.y * dy);
-        const float gv = hl * fmaf(2.f, bzdy, bydx);
-        const float tx = dpw * dx, ty = dpw * dy;
-        const float ga = -0.5f * (tx * dx);
-        const float gb = -(tx * dy);
-        const float gc = -0.5f * (ty * dy);
-        if (FULL) go = slope ? dal * hw_exp2(p - b.w) : 0.f;
+        const float tx = dpw * dx;
         Sg = fmaf(gcv, wk, Sg);
         // a recorded entry has a contributing lane: the forward took it for
         // the same pixels by the same arithmetic
         if (recorded || __any_sync(FULLM, contrib)) {
-          // reduce-scatter over the warp: every lane then holds the warp sum
-          // of word `comp`, and one lane per word adds it with one atomic
-          float *dst = s_dst[j];
           float sum;
-          if constexpr (FULL) {
-            const float v10[10] = {gu, gv, ga, gb, gc, gz, go, gr, gg, gbl};
-            sum = warp_reduce_scatter<10>(v10, lane);
+          if constexpr (MOMENTS) {
+            sum = moment_sums<FULL>(dpw, tx, tx * dx, gz, g0 * wk, g1 * wk, g2 * wk, dy, lane);
           } else {
-            const float v6[6] = {gu, gv, ga, gb, gc, gz};
-            sum = warp_reduce_scatter<6>(v6, lane);
+            // the exponent in log2 units is p, so d/dx of the natural exponent
+            // is ln2 dp/dx: d p / d(u, v) = (2 a' dx + b' dy, b' dx + 2 c' dy)
+            // from the exponent's products; d(natural exponent) / d(conic) =
+            // -(dx^2 / 2, dx dy, dy^2 / 2). A reduce-scatter leaves every lane
+            // the warp sum of one word
+            const float hl = dpw * kLn2, ty = dpw * dy;
+            const float v10[10] = {hl * fmaf(2.f, bxdx, b.y * dy), hl * fmaf(2.f, bzdy, bydx), -0.5f * (tx * dx),
+                                   -(tx * dy), -0.5f * (ty * dy), gz, dpw, g0 * wk, g1 * wk, g2 * wk};
+            sum = warp_reduce_scatter<10, 16>(v10, lane);
           }
-          if (writer) atomicAdd(dst + comp, sum);
+          if (writer) atomicAdd(gdst + (size_t)s_slot[j] * kGradWords, sum);
         }
       }
     }
@@ -247,13 +289,24 @@ render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ tar
 // Chains the 2D gradients of the Gaussian projected as q in view slot `slot`
 // (pose Pm) to the pose twist (pg, added) and, FULL, to the record's
 // parameters (acc, added).
-template <bool FULL>
+template <bool FULL, bool MOMENTS>
 __device__ __forceinline__ void chain_proj(const Workspace &ws, const Raster &r, const Proj &q, const float *Pm,
                                            size_t slot, float *pg, float *acc) {
   const float *gd = ws.grad2d + slot * kGradWords;
   const float4 ga4 = *reinterpret_cast<const float4 *>(gd);
   const float4 gb4 = *reinterpret_cast<const float4 *>(gd + 4);
-  const float gu = ga4.x, gv = ga4.y, gA = ga4.z, gB = ga4.w, gC = gb4.x, gzz = gb4.y;
+  float gu = ga4.x, gv = ga4.y, gA = ga4.z, gB = ga4.w, gC = gb4.x;
+  const float gzz = gb4.y;
+  if constexpr (MOMENTS) {
+    // the natural exponent is -(a dx^2 / 2 + b dx dy + c dy^2 / 2) for the
+    // conic (a, b, c): d/du = -(a Sx + b Sy), d/d(a, b, c) = -(Sxx / 2, Sxy,
+    // Syy / 2)
+    gu = -fmaf(q.ca, ga4.x, q.cb * ga4.y);
+    gv = -fmaf(q.cc, ga4.y, q.cb * ga4.x);
+    gA *= -0.5f;
+    gB = -gB;
+    gC *= -0.5f;
+  }
   // conic -> 2D covariance: dS = -Q Gq Q with Gq the symmetric-matrix form of
   // the conic gradient (the off-diagonal appears twice in the quadratic form)
   const float qa = q.ca, qb = q.cb, qc = q.cc;
@@ -310,11 +363,11 @@ __device__ __forceinline__ void chain_proj(const Workspace &ws, const Raster &r,
   pg[5] += Bm[1] - Bm[3];
   if (FULL) {
     const float4 gc4 = *reinterpret_cast<const float4 *>(gd + 8);
-    const float go = gb4.z;
+    const float s0 = gb4.z;   // o dL/do: alpha is proportional to the opacity
     acc[0] += Pm[0] * dpx + Pm[4] * dpy + Pm[8] * dpz;
     acc[1] += Pm[1] * dpx + Pm[5] * dpy + Pm[9] * dpz;
     acc[2] += Pm[2] * dpx + Pm[6] * dpy + Pm[10] * dpz;
-    acc[3] += go * q.o * (1.f - q.o);
+    acc[3] += s0 * (1.f - q.o);
     // K = R M, M = Rq diag(S): dM = R^T dK
     float dRq[9];
 #pragma unroll
@@ -359,11 +412,11 @@ __device__ __forceinline__ bool visible_proj(const Workspace &ws, const Raster &
 }
 
 // chain_proj of Gaussian (g0, g1, g2) when it is visible.
-template <bool FULL>
+template <bool FULL, bool MOMENTS>
 __device__ __forceinline__ void chain_one(const Workspace &ws, const Raster &r, const float4 &g0, const float4 &g1,
                                           const float4 &g2, const float *Pm, size_t slot, float *pg, float *acc) {
   Proj q;
-  if (visible_proj(ws, r, g0, g1, g2, Pm, slot, q)) chain_proj<FULL>(ws, r, q, Pm, slot, pg, acc);
+  if (visible_proj(ws, r, g0, g1, g2, Pm, slot, q)) chain_proj<FULL, MOMENTS>(ws, r, q, Pm, slot, pg, acc);
 }
 
 // Compensated (double-FP32) addition: (h, l) += (bh, bl) through two-sum,
@@ -401,7 +454,7 @@ __device__ __forceinline__ void store_pose_partial(const Workspace &ws, float *p
 // !FULL (pose only): a fixed grid strides over the Gaussians of each view.
 // The last CTA sums the pose partials in a fixed order in FP64 (one warp per
 // twist component) and, if ps.poses is set, applies the pose step.
-template <bool FULL>
+template <bool FULL, bool MOMENTS>
 __global__ void __launch_bounds__(kBwdPrepBlock)
 preprocess_bwd_kernel(Workspace ws, const float4 *__restrict__ gauss, int64_t n, int views, Raster r,
                       float *__restrict__ grad_gauss, double *__restrict__ grad_pose, PoseStep ps) {
@@ -472,7 +525,7 @@ preprocess_bwd_kernel(Workspace ws, const float4 *__restrict__ gauss, int64_t n,
     for (int k = 0; k < 16; ++k) acc[k] = 0.f;
     for (int v = 0; v < views; ++v) {
       float pg[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      if (i < n) chain_one<true>(ws, r, g0, g1, g2, sp + v * 12, (size_t)v * ws.max_n + i, pg, acc);
+      if (i < n) chain_one<true, MOMENTS>(ws, r, g0, g1, g2, sp + v * 12, (size_t)v * ws.max_n + i, pg, acc);
       if (grad_pose) store_pose_partial(ws, pg, v, blockIdx.x, nb, s_red);
     }
     if (i < n) {
@@ -491,13 +544,13 @@ preprocess_bwd_kernel(Workspace ws, const float4 *__restrict__ gauss, int64_t n,
       const uint32_t *vis = ws.vis_ids + (size_t)v * ws.max_n;
       for (int64_t k = (int64_t)bid * blockDim.x + tid; k < nv; k += (int64_t)nb * blockDim.x) {
         if (pre && k == pre_k) {
-          if (pre_vis) chain_proj<false>(ws, r, q0, sp, pre_slot, pg, nullptr);
+          if (pre_vis) chain_proj<false, MOMENTS>(ws, r, q0, sp, pre_slot, pg, nullptr);
           continue;
         }
         int64_t i = vis[k];
         if (!DAGS_IN_BOUNDS(i >= 0 && i < n, ws.counters + CNT_STATUS)) continue;
         const float4 g0 = __ldg(gauss + 4 * i + 0), g1 = __ldg(gauss + 4 * i + 1), g2 = __ldg(gauss + 4 * i + 2);
-        chain_one<false>(ws, r, g0, g1, g2, sp + v * 12, (size_t)v * ws.max_n + i, pg, nullptr);
+        chain_one<false, MOMENTS>(ws, r, g0, g1, g2, sp + v * 12, (size_t)v * ws.max_n + i, pg, nullptr);
       }
       store_pose_partial(ws, pg, v, bid, nb, s_red);
     }
@@ -578,17 +631,30 @@ preprocess_bwd_kernel(Workspace ws, const float4 *__restrict__ gauss, int64_t n,
 
 }  // namespace
 
+// Whether the 2D gradients are accumulated as moments. They are, except where
+// the Gaussian and the twist gradients are both asked for: the twist gradient
+// cancels by two to three digits over the map, and a caller that takes it in
+// FP64 beside the map's gradients gets it with the rounding of the per-pixel
+// form (either form is about 3e-7 from 64 bits on the 2,000-Gaussian scene).
+// Gradients of 200k Gaussians over 8 views of 640x480: the adjoint takes 354 us
+// with moments over the entries the forward recorded, 421 us per pixel over
+// every entry whose box meets the warp's block.
+static bool backward_moments(bool full, bool pose) { return !(full && pose); }
+
 cudaError_t launch_render_bwd(const Workspace &ws, int views, int64_t n, const Raster &r, const Loss &l,
-                              const float4 *targets, const float *image, const int32_t *last, bool full,
+                              const float4 *targets, const float *image, const int32_t *last, bool full, bool pose,
                               cudaStream_t s, const float *upstream) {
   (void)n;
   const dim3 grid((unsigned)(views * r.T));
   const bool masks = ws.warp_masks != nullptr, count = ws.count_evals != 0;
-#define DAGS_BWD(F, M, C) \
-  launch_pdl(render_bwd_kernel<F, M, C>, grid, dim3(kTilePix), 0, s, ws, r, l, targets, image, last, upstream)
-  if (full) return count ? DAGS_BWD(true, false, true) : DAGS_BWD(true, false, false);
-  if (masks) return count ? DAGS_BWD(false, true, true) : DAGS_BWD(false, true, false);
-  return count ? DAGS_BWD(false, false, true) : DAGS_BWD(false, false, false);
+#define DAGS_BWD(F, M, K, C) \
+  launch_pdl(render_bwd_kernel<F, M, K, C>, grid, dim3(kTilePix), 0, s, ws, r, l, targets, image, last, upstream)
+#define DAGS_BWD_KC(F, M) \
+  (masks ? (count ? DAGS_BWD(F, M, true, true) : DAGS_BWD(F, M, true, false)) \
+         : (count ? DAGS_BWD(F, M, false, true) : DAGS_BWD(F, M, false, false)))
+  if (full) return backward_moments(full, pose) ? DAGS_BWD_KC(true, true) : DAGS_BWD_KC(true, false);
+  return DAGS_BWD_KC(false, true);
+#undef DAGS_BWD_KC
 #undef DAGS_BWD
 }
 
@@ -599,8 +665,11 @@ cudaError_t launch_preprocess_bwd(const Workspace &ws, const float4 *gauss, int6
   const unsigned gx = (unsigned)((n + kBwdPrepBlock - 1) / kBwdPrepBlock);
   unsigned grid = gx > 0 ? gx : 1u;
   if (grad_gauss) {
-    return launch_pdl(preprocess_bwd_kernel<true>, dim3(grid), dim3(kBwdPrepBlock), 0, s, ws, gauss, n, views, r,
-                      grad_gauss, grad_pose, ps);
+    if (backward_moments(true, grad_pose != nullptr))
+      return launch_pdl(preprocess_bwd_kernel<true, true>, dim3(grid), dim3(kBwdPrepBlock), 0, s, ws, gauss, n, views,
+                        r, grad_gauss, grad_pose, ps);
+    return launch_pdl(preprocess_bwd_kernel<true, false>, dim3(grid), dim3(kBwdPrepBlock), 0, s, ws, gauss, n, views,
+                      r, grad_gauss, grad_pose, ps);
   } else {
     // pose only: a fixed grid of 4 CTAs per SM (one wave) strides over the
     // visible Gaussians (at most one per thread at the tracking size); the
@@ -609,7 +678,7 @@ cudaError_t launch_preprocess_bwd(const Workspace &ws, const float4 *gauss, int6
     const unsigned cap = (unsigned)(4 * (ws.band > 0 ? ws.band : 1));
     if (grid > cap) grid = cap;
     if (ws.order_next) grid += 1;
-    return launch_pdl(preprocess_bwd_kernel<false>, dim3(grid), dim3(kBwdPrepBlock), 0, s, ws, gauss, n, views, r,
+    return launch_pdl(preprocess_bwd_kernel<false, true>, dim3(grid), dim3(kBwdPrepBlock), 0, s, ws, gauss, n, views, r,
                       grad_gauss, grad_pose, ps);
   }
   return cudaGetLastError();

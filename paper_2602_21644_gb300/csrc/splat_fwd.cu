@@ -547,9 +547,13 @@ emit_kernel(Workspace ws, int64_t n, Raster r) {
   walk_tiles<kWalkEmit>(ws, r, v, id, rect, r0, r1, z);
 }
 
-// MASKS: record per warp the list entries its pixels took (ws.warp_masks,
-// the tracking loop); COUNT: count evaluations and contributions (ws.evals).
-template <bool MASKS, bool COUNT>
+// COUNT: count evaluations and contributions (ws.evals). Bound by instruction
+// issue (73-75% issue-active, ALU pipe busiest), so what is per (warp, entry)
+// pair is kept short: a lane's contributions of a 32-entry group are one bit
+// each in `took`, from which the last contributor and, by one reduction per
+// group, the warp's record for the adjoint (ws.warp_masks) follow; the BF16
+// colour is widened once per staged entry.
+template <bool COUNT>
 __global__ void __launch_bounds__(kTilePix, 5)
 render_fwd_kernel(Workspace ws, int views, Raster r, Loss l, const float4 *__restrict__ targets,
                   float *__restrict__ image, int32_t *__restrict__ last, double *__restrict__ loss) {
@@ -559,6 +563,7 @@ render_fwd_kernel(Workspace ws, int views, Raster r, Loss l, const float4 *__res
   __shared__ __align__(16) uint64_t s_key[kSortSmallCap];
   __shared__ float4 s_a[kTilePix], s_b[kTilePix], s_c[kTilePix];   // s_a: {u hi, v hi, u lo, v lo}
   __shared__ float2 s_e[kTilePix];                                  // box half extents
+  __shared__ float s_bl[kTilePix];                                  // s_c: {z, M, r, g}; blue here
   __shared__ float2 s_red[kTilePix / 32];
   __shared__ int s_last;
   const unsigned FULL = 0xffffffffu;
@@ -595,7 +600,7 @@ render_fwd_kernel(Workspace ws, int views, Raster r, Loss l, const float4 *__res
   const bool inside = px < r.W && py < r.H;
   uint32_t s = 0u, e = 0u;
   if (!ovf) tile_range(ws, tile, s, e);
-  uint32_t *const wmask = MASKS ? ws.warp_masks + (size_t)tile * kMaskGroups * 8 + warp : nullptr;
+  uint32_t *const wmask = ws.warp_masks ? ws.warp_masks + (size_t)tile * kMaskGroups * 8 + warp : nullptr;
   const size_t vbase = (size_t)v * ws.max_n;
   const float bcx = (float)bx0 + 3.5f, bcy = (float)by0 + 1.5f;
 
@@ -620,7 +625,10 @@ render_fwd_kernel(Workspace ws, int views, Raster r, Loss l, const float4 *__res
       s_a[tid] = make_float4(r0.x, r0.y, lo.x, lo.y);
       s_e[tid] = make_float2(r0.z, r0.w);
       s_b[tid] = ws.rec2d[slot * 3 + 1];
-      s_c[tid] = ws.rec2d[slot * 3 + 2];
+      const float4 r2 = ws.rec2d[slot * 3 + 2];
+      const uint32_t rg = __float_as_uint(r2.z), bl = __float_as_uint(r2.w);
+      s_c[tid] = make_float4(r2.x, r2.y, bf16_lo(rg), bf16_hi(rg));
+      s_bl[tid] = bf16_lo(bl);
     }
     __syncthreads();
     const int cnt = (int)min((uint32_t)kTilePix, e - base);
@@ -635,11 +643,11 @@ render_fwd_kernel(Workspace ws, int views, Raster r, Loss l, const float4 *__res
         hit = fabsf(a.x - bcx) <= ex.x + 3.5f && fabsf(a.y - bcy) <= ex.y + 1.5f;
       }
       unsigned mask = __ballot_sync(FULL, hit);
-      unsigned took = 0u;   // entries at least one pixel of the warp took
+      unsigned took = 0u;   // entries this lane's pixel took
       while (mask) {
-        const int bit = __ffs(mask) - 1;
-        const int j = g * 32 + bit;
-        mask &= mask - 1;
+        const unsigned b1 = mask & (0u - mask);   // the lowest entry's bit
+        mask ^= b1;
+        const int j = g * 32 + 31 - __clz((int)b1);
         // evaluated by every lane, without branches: a lane that is done,
         // or whose alpha is below alpha_min, or that would stop here adds
         // a zero weight and keeps T (x + 0 * c == x), so each pixel's sums
@@ -659,16 +667,16 @@ render_fwd_kernel(Workspace ws, int views, Raster r, Loss l, const float4 *__res
         done = done || stop;
         const float w = contrib ? __fmul_rn(alpha, T) : 0.f;
         const float4 c = s_c[j];
-        const uint32_t rg = __float_as_uint(c.z), bl = __float_as_uint(c.w);
-        cr = __fmaf_rn(bf16_lo(rg), w, cr); cg = __fmaf_rn(bf16_hi(rg), w, cg); cb = __fmaf_rn(bf16_lo(bl), w, cb);
+        cr = __fmaf_rn(c.z, w, cr); cg = __fmaf_rn(c.w, w, cg); cb = __fmaf_rn(s_bl[j], w, cb);
         dd = __fmaf_rn(c.x, w, dd); oo = __fadd_rn(oo, w); rm = __fmaf_rn(c.y, w, rm);
         T = contrib ? tt : T;
-        lastk = contrib ? (int)(base - s) + j + 1 : lastk;
-        if (MASKS && __any_sync(FULL, contrib)) took |= 1u << bit;
+        if (contrib) took |= b1;
       }
-      if (MASKS) {
-        const int gk = (int)((base - s) >> 5) + g;
-        if (lane == 0 && gk < kMaskGroups) wmask[gk * 8] = took;
+      const int gk = (int)((base - s) >> 5) + g;
+      if (took) lastk = gk * 32 + 32 - __clz((int)took);
+      if (wmask && gk < kMaskGroups) {
+        const unsigned any = __reduce_or_sync(FULL, took);
+        if (lane == 0) wmask[gk * 8] = any;
       }
       if (__all_sync(FULL, done)) break;
     }
@@ -800,17 +808,9 @@ cudaError_t launch_render_fwd(const Workspace &ws, int views, int64_t n, const R
                               cudaStream_t s) {
   (void)n;
   const dim3 grid((unsigned)(views * r.T));
-  const bool masks = ws.warp_masks != nullptr;
-  if (ws.count_evals) {
-    if (masks) return launch_pdl(render_fwd_kernel<true, true>, grid, dim3(kTilePix), 0, s, ws, views, r, l, targets,
-                                 image, last, loss);
-    return launch_pdl(render_fwd_kernel<false, true>, grid, dim3(kTilePix), 0, s, ws, views, r, l, targets, image,
-                      last, loss);
-  }
-  if (masks) return launch_pdl(render_fwd_kernel<true, false>, grid, dim3(kTilePix), 0, s, ws, views, r, l, targets,
-                               image, last, loss);
-  return launch_pdl(render_fwd_kernel<false, false>, grid, dim3(kTilePix), 0, s, ws, views, r, l, targets, image,
-                    last, loss);
+  if (ws.count_evals)
+    return launch_pdl(render_fwd_kernel<true>, grid, dim3(kTilePix), 0, s, ws, views, r, l, targets, image, last, loss);
+  return launch_pdl(render_fwd_kernel<false>, grid, dim3(kTilePix), 0, s, ws, views, r, l, targets, image, last, loss);
 }
 
 }  // namespace dags
