@@ -119,7 +119,7 @@ cudaError_t alloc(T **p, size_t count) {
 }
 
 void free_ws(Workspace &w) {
-  void *ptrs[] = {w.rec2d, w.rec_lo, w.rect, w.grad2d, w.tile_count, w.tile_start, w.tile_cursor, w.keys,
+  void *ptrs[] = {w.rec2d, w.rect, w.grad2d, w.tile_count, w.tile_start, w.tile_cursor, w.keys,
                   w.keys_tmp, w.sorted_ids, w.tile_order, w.loss_partial, w.pose_partial, w.pose32,
                   w.vis_ids, w.vis_append, w.vis_n, w.counters, w.evals};
   for (void *p : ptrs)
@@ -304,8 +304,7 @@ int dags_create(dags_ctx **out, int64_t max_gaussians, int32_t max_width, int32_
   const size_t vt = (size_t)w.max_v * (size_t)w.max_tiles;
   cudaError_t e = cudaSuccess;
   auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-  A(alloc(&w.rec2d, vn * 3));
-  A(alloc(&w.rec_lo, vn));
+  A(alloc(&w.rec2d, vn * 4));
   A(alloc(&w.rect, vn));
   A(alloc(&w.grad2d, vn * kGradWords));
   A(alloc(&w.tile_count, vt));
@@ -1367,8 +1366,7 @@ constexpr size_t kOffLossPartial = kOffOrder + al256(kStaticTiles * 4);
 constexpr size_t kOffVisN = kOffLossPartial + al256(kStaticTiles * 8);
 constexpr size_t kOffPose32 = kOffVisN + al256(4);
 constexpr size_t kOffRec2d = kOffPose32 + al256(12 * 4);
-constexpr size_t kOffRecLo = kOffRec2d + al256(kStaticMaxN * 3 * 16);
-constexpr size_t kOffRect = kOffRecLo + al256(kStaticMaxN * 8);
+constexpr size_t kOffRect = kOffRec2d + al256(kStaticMaxN * 4 * 16);
 constexpr size_t kOffGrad2d = kOffRect + al256(kStaticMaxN * 8);
 constexpr size_t kOffVisIds = kOffGrad2d + al256(kStaticMaxN * kGradWords * 4);
 constexpr size_t kOffKeys = kOffVisIds + al256(kStaticMaxN * 4);
@@ -1482,7 +1480,6 @@ extern "C" int splat_forward_static(const float *gauss, int64_t n, const dags_ca
   w.vis_n = reinterpret_cast<uint32_t *>(base + kOffVisN);
   w.pose32 = reinterpret_cast<float *>(base + kOffPose32);
   w.rec2d = reinterpret_cast<float4 *>(base + kOffRec2d);
-  w.rec_lo = reinterpret_cast<float2 *>(base + kOffRecLo);
   w.rect = reinterpret_cast<uint2 *>(base + kOffRect);
   w.grad2d = reinterpret_cast<float *>(base + kOffGrad2d);
   w.vis_ids = reinterpret_cast<uint32_t *>(base + kOffVisIds);

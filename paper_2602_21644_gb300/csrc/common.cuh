@@ -59,20 +59,20 @@ enum {
   CNT_N
 };
 
-// Projected Gaussian, 3 float4 per (view, Gaussian):
-//   r0 = {u, v, ex, ey}      centre (px) and half extents of the bounding box
-//                            of the alpha >= alpha_min ellipse
+// Projected Gaussian, one 64-byte line of 4 float4 per (view, Gaussian), as the
+// compositing kernels stage it:
+//   r0 = {u, v, u_lo, v_lo}  centre (px), with FP32 remainders
 //   r1 = {a', b', c', lo}    exponent p(d) = a' dx^2 + b' dx dy + c' dy^2 + lo
 //                            in log2 units: alpha = min(alpha_max, 2^p),
 //                            a' = -a log2(e) / 2, b' = -b log2(e),
 //                            c' = -c log2(e) / 2 for the conic (a, b, c), and
 //                            lo = log2(opacity)
-//   r2 = {z, M, rg, bl}      depth, motion probability, colour as the
-//                            record's BF16 bit patterns
-// The centre (u, v) is computed in FP64 from the FP64 pose and stored as
-// u = r0.x + lo.x, v = r0.y + lo.y with the FP32 remainders in rec_lo, so
-// that a pixel offset (u - px) = (r0.x - px) + lo.x carries a relative
-// rounding of 2^-24 of the offset rather than an absolute ulp(u).
+//   r2 = {z, M, r, g}        depth, motion probability, the record's BF16 colour
+//   r3 = {b, ex, ey, id}     blue, half extents of the bounding box of the
+//                            alpha >= alpha_min ellipse, Gaussian id (its bits)
+// The centre is computed from the FP64 pose and stored as u = r0.x + r0.z,
+// v = r0.y + r0.w, so that a pixel offset (u - px) = (r0.x - px) + r0.z carries
+// a relative rounding of 2^-24 of the offset rather than an absolute ulp(u).
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -82,8 +82,7 @@ struct Workspace {
   int64_t max_pairs = 0;
   int bwd_prep_blocks = 0;
   int band = 1;                   // CTAs per dispatch round of the renders (the SM count)
-  float4 *rec2d = nullptr;        // [V][N][3], see above
-  float2 *rec_lo = nullptr;       // [V][N] FP32 remainders of the FP64 centre
+  float4 *rec2d = nullptr;        // [V][N][4], see above
   uint2 *rect = nullptr;          // [V][N]: {x0 | x1 << 16, y0 | y1 << 16}, candidate tiles [x0, x1) x [y0, y1)
   float *grad2d = nullptr;        // [V][N][kGradWords]
   uint32_t *tile_count = nullptr; // [V * T]

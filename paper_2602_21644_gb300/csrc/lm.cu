@@ -238,6 +238,7 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
   __shared__ __align__(16) uint64_t s_key[kSortSmallCap];
   __shared__ float4 s_a[kJacBatch], s_b[kJacBatch], s_c[kJacBatch];   // s_a: {u hi, v hi, u lo, v lo}
   __shared__ float2 s_e[kJacBatch];                                   // box half extents
+  __shared__ float s_bl[kJacBatch];                                   // blue
   extern __shared__ float4 s_t[];   // kJacBatch * kTan4
   __shared__ float s_red[kTilePix / 32][kNormal];
   __shared__ int s_last;
@@ -293,12 +294,12 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
       if (!DAGS_IN_BOUNDS(id < (uint32_t)ws.max_n, ws.counters + CNT_STATUS)) id = 0;
       const float4 *tg = tan + (size_t)id * kTan4;
       float4 *st = s_t + q * kTan4;
-      const float4 r0 = ws.rec2d[(size_t)id * 3 + 0];
-      const float2 lo = ws.rec_lo[id];
-      s_a[q] = make_float4(r0.x, r0.y, lo.x, lo.y);
-      s_e[q] = make_float2(r0.z, r0.w);
-      s_b[q] = ws.rec2d[(size_t)id * 3 + 1];
-      s_c[q] = ws.rec2d[(size_t)id * 3 + 2];
+      const float4 r3 = ws.rec2d[(size_t)id * 4 + 3];
+      s_a[q] = ws.rec2d[(size_t)id * 4 + 0];
+      s_b[q] = ws.rec2d[(size_t)id * 4 + 1];
+      s_c[q] = ws.rec2d[(size_t)id * 4 + 2];
+      s_e[q] = make_float2(r3.y, r3.z);
+      s_bl[q] = r3.x;
 #pragma unroll
       for (int w = 0; w < kTan4; ++w) st[w] = tg[w];
     }
@@ -328,8 +329,7 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
         if (tt < r.t_min) { done = true; continue; }
         const float w = alpha * T;
         const float4 c = s_c[j];
-        const uint32_t rg = __float_as_uint(c.z), bl = __float_as_uint(c.w);
-        const float cR = bf16_lo(rg), cG = bf16_hi(rg), cB = bf16_lo(bl);
+        const float cR = c.z, cG = c.w, cB = s_bl[j];
         cr += cR * w; cg += cG * w; cb += cB * w;
         dd += c.x * w; oo += w; rm += c.y * w;
         // tangents: p' = da' dx^2 + db' dx dy + dc' dy^2 + dp/du du + dp/dv dv,

@@ -1,6 +1,6 @@
 // Backward half of the MP-aware splatting path (sm_103a).
 //
-//   render_bwd_kernel      one CTA per 16x16 tile: walks the tile's sorted
+//   render_bwd_kernel      one warp per 8x4 pixel block: walks its tile's sorted
 //                          list back to front from the furthest recorded
 //                          contributor, re-deriving each pixel's
 //                          transmittance from its final value (T_k =
@@ -33,7 +33,9 @@ static_assert(G2_U == 0 && G2_C == 4 && G2_Z == 5 && G2_BL == 9 && kGradWords >=
 // over each row's 8 lanes, and the y factors are applied to the row sums: 7 + 2
 // shuffles for the ten words and 4 + 2 for the pose path's six (a
 // reduce-scatter of all words over 32 lanes takes 12 and 8, and needs every
-// word formed per pixel). After the row stage lane l8 = lane & 7 holds
+// word formed per pixel). The terms are given as x = (m1, m2, z, r, g, b, m0),
+// or (m1, m2, z, m0) for the pose path; after the row stage lane l8 = lane & 7
+// holds
 //   FULL:      m1, m2, z, m0, r, g, b, m0
 //   pose only: m1, m1, m2, m2, z, z, m0, m0
 // and the rows are summed as is by the lanes below 16, weighted with dy by the
@@ -50,18 +52,10 @@ __device__ __forceinline__ int moment_word(int lane) {
   return l8 == 2 ? G2_A : l8 == 4 ? G2_Z : -1;
 }
 
-template <bool FULL>
-__device__ __forceinline__ float moment_sums(float m0, float m1, float m2, float gz, float gr, float gg, float gb,
-                                             float dy, int lane) {
+template <int K>
+__device__ __forceinline__ float moment_sums(const float (&x)[K], float dy, int lane) {
   const unsigned FULLM = 0xffffffffu;
-  float v;
-  if constexpr (FULL) {
-    const float x[7] = {m1, m2, gz, gr, gg, gb, m0};
-    v = warp_reduce_scatter<7, 4>(x, lane);
-  } else {
-    const float x[4] = {m1, m2, gz, m0};
-    v = warp_reduce_scatter<4, 4>(x, lane);
-  }
+  const float v = warp_reduce_scatter<K, 4>(x, lane);
   const float b = v * dy;
   const float a = (lane & 7) == 7 ? b * dy : v;
   const bool hi = (lane & 16) != 0;
@@ -74,34 +68,36 @@ __device__ __forceinline__ float moment_sums(float m0, float m1, float m2, float
 // MOMENTS: words 0-4 as moments (see G2_U), else as gradients formed per pixel;
 // MASKS: visit only the entries the forward recorded as taken by the warp
 // (ws.warp_masks); COUNT: count evaluations and contributions (ws.evals).
-// Bound by instruction issue (75-87% issue-active): a pair costs its loop, its
-// loads, the arithmetic per pixel and the warp's reduction.
+// One warp, and one CTA, per 8 x 4 pixel block: no barrier joins the blocks of a
+// tile, a block with few entries leaves its slot at once, and the short blocks
+// launched last even out the SMs (with a CTA of 8 warps per tile, a frame's
+// 1,200 CTAs kept the SMs busy for 77% of the kernel and half of a busy SM's
+// warp slots). The warp stages the taken entries of a 32-entry group with
+// cp.async while it works on the group before, and works on two entries at a
+// time. 300k Gaussians, 640x480, pose only: 67 us per CTA of 8 warps, 58 and 54
+// per warp in CTAs of two and one, 52 with two entries at a time; all
+// gradients: 74 -> 66 us; 2,000 Gaussians, 160x120: 60 -> 42 us.
+constexpr int kBlocks = kTilePix / 32;   // pixel blocks per tile
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
 template <bool FULL, bool MOMENTS, bool MASKS, bool COUNT>
-__global__ void __launch_bounds__(kTilePix, 5)
+__global__ void __launch_bounds__(32, 32)
 render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ targets,
                   const float *__restrict__ image, const int32_t *__restrict__ last,
                   const float *__restrict__ upstream) {
   pdl_wait();
   pdl_trigger();
-  __shared__ float4 s_a[kTilePix], s_b[kTilePix], s_c[kTilePix];   // s_a: {u hi, v hi, u lo, v lo}
-  __shared__ float2 s_e[kTilePix];                                  // box half extents
-  __shared__ float s_bl[kTilePix];                                  // s_c: {z, M, r, g}; blue here
-  // the entry's slot (32 bits: 2^32 slots would need 400 GB of records and
-  // gradients)
-  __shared__ uint32_t s_slot[kTilePix];
-  __shared__ int s_max;
+  __shared__ float4 s_rec[2][4][32];   // projected records, double-buffered
   const unsigned FULLM = 0xffffffffu;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (ws.bucket_cap) {
-    // fixed-bucket layout: an overflowed tile is skipped (its count is
-    // cleared for the next preprocess all the same)
-    const int t = (int)ws.tile_order[blockIdx.x];
-    if (ws.tile_count[t] > ws.bucket_cap) {
-      __syncthreads();
-      if (tid == 0) ws.tile_count[t] = 0u;
-      return;
-    }
-  } else {
+  const int lane = threadIdx.x;
+  const int warp = (int)(blockIdx.x % kBlocks);   // the tile's pixel block
+  // an overflow of the packed layout leaves every tile out; in the
+  // fixed-bucket layout a tile that overflowed has no contributors
+  if (!ws.bucket_cap) {
     const uint64_t tot = (uint64_t)ws.counters[CNT_REQ_LO] | ((uint64_t)ws.counters[CNT_REQ_HI] << 32);
     if (tot > (uint64_t)ws.max_pairs) return;
   }
@@ -115,19 +111,18 @@ render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ tar
     if (__ffs(__match_any_sync(FULLM, (unsigned)word)) - 1 != lane) word = -1;
   }
   const bool writer = word >= 0;
-  float *const gdst = ws.grad2d + (writer ? word : 0);
-  const int tile = (int)ws.tile_order[blockIdx.x];   // longest lists first
+  const int tile = (int)ws.tile_order[blockIdx.x / kBlocks];   // longest lists first
   const int v = tile / r.T, tv = tile - v * r.T;
   const int tx = tv % r.tiles_x, ty = tv / r.tiles_x;
   const int bx0 = tx * kTile + (warp & 1) * 8, by0 = ty * kTile + (warp >> 1) * 4;
   const int px = bx0 + (lane & 7), py = by0 + (lane >> 3);
   const bool inside = px < r.W && py < r.H;
-  uint32_t s, e_unused;
-  tile_range(ws, tile, s, e_unused);
+  const uint32_t s = ws.bucket_cap ? (uint32_t)tile * ws.bucket_cap : ws.tile_start[tile];
   // the forward's record of the entries this warp's pixels took (groups of
   // 32 entries; later groups fall back to the box test)
   const uint32_t *const wmask = MASKS ? ws.warp_masks + (size_t)tile * kMaskGroups * 8 + warp : nullptr;
-  const size_t vbase = (size_t)v * ws.max_n;
+  const float4 *const recs = ws.rec2d + (size_t)v * ws.max_n * 4;
+  float *const gdst = ws.grad2d + (size_t)v * ws.max_n * kGradWords + (writer ? word : 0);
   const size_t P = (size_t)r.W * r.H;
   const float bcx = (float)bx0 + 3.5f, bcy = (float)by0 + 1.5f;
 
@@ -170,120 +165,146 @@ render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ tar
       }
     }
   }
-  if (tid == 0) s_max = 0;
-  __syncthreads();
   const int wmax = (int)__reduce_max_sync(FULLM, (unsigned)lastp);
-  if (lane == 0) atomicMax(&s_max, wmax);
-  __syncthreads();
-  const int kmax = s_max;
 
   // Sg = sum over channels of g_ch * S_ch, S_ch the channel's composited sum
   // behind the current Gaussian: dL/dalpha needs only this contraction
   float Sg = 0.f;
   unsigned n_eval = 0, n_contrib = 0;
   const float fpx = (float)px, fpy = (float)py;
-  // batches of kTilePix entries aligned as the forward's (the recorded
-  // masks address entries by their 32-entry group in the tile's list); the
-  // first batch walked is the one holding the last contributor
-  for (int end = kmax, beg; end > 0; end = beg) {
-    beg = ((end - 1) / kTilePix) * kTilePix;
-    __syncthreads();
-    if (beg + tid < end && DAGS_IN_BOUNDS((uint64_t)s + beg + tid < (uint64_t)ws.max_pairs, ws.counters + CNT_STATUS)) {
-      uint32_t id = ws.sorted_ids[s + beg + tid];
-      if (!DAGS_IN_BOUNDS(id < (uint32_t)ws.max_n, ws.counters + CNT_STATUS)) id = 0;
-      const size_t slot = vbase + id;
-      s_slot[tid] = (uint32_t)slot;
-      const float4 r0 = ws.rec2d[slot * 3 + 0];
-      const float2 lo = ws.rec_lo[slot];
-      s_a[tid] = make_float4(r0.x, r0.y, lo.x, lo.y);
-      s_e[tid] = make_float2(r0.z, r0.w);
-      s_b[tid] = ws.rec2d[slot * 3 + 1];
-      const float4 r2 = ws.rec2d[slot * 3 + 2];
-      const uint32_t rg = __float_as_uint(r2.z), bl = __float_as_uint(r2.w);
-      s_c[tid] = make_float4(r2.x, r2.y, bf16_lo(rg), bf16_hi(rg));
-      s_bl[tid] = bf16_lo(bl);
+  // this lane's entry of group g, and the group's entries to visit: those the
+  // forward recorded, or all up to the last contributor
+  auto group = [&](int g, uint32_t &id, unsigned &mask) {
+    const int k = g * 32 + lane;
+    id = 0u;
+    if (k < wmax && DAGS_IN_BOUNDS((uint64_t)s + k < (uint64_t)ws.max_pairs, ws.counters + CNT_STATUS)) {
+      id = __ldg(ws.sorted_ids + s + k);
+      if (!DAGS_IN_BOUNDS(id < (uint32_t)ws.max_n, ws.counters + CNT_STATUS)) id = 0u;
     }
-    __syncthreads();
-    const int cnt = end - beg;
-    if (wmax <= beg) continue;               // no pixel of this warp reaches this batch
-    const int top = min(cnt, wmax - beg);    // entries [beg, beg + top) may matter to this warp
-    for (int g = (top - 1) >> 5; g >= 0; --g) {
-      const int gk = (beg >> 5) + g;
-      unsigned mask;
-      const bool recorded = MASKS && gk < kMaskGroups;
-      if (recorded) {
-        mask = __ldg(wmask + gk * 8);
-      } else {
-        const int jj = g * 32 + lane;
-        bool hit = false;
-        if (jj < cnt) {
-          const float4 a = s_a[jj];
-          const float2 ex = s_e[jj];
-          hit = fabsf(a.x - bcx) <= ex.x + 3.5f && fabsf(a.y - bcy) <= ex.y + 1.5f;
-        }
-        mask = __ballot_sync(FULLM, hit);
+    mask = MASKS && g < kMaskGroups ? __ldg(wmask + g * 8) : FULLM;
+    const int lim = wmax - g * 32;
+    if (lim < 32) mask &= (1u << lim) - 1u;
+  };
+  auto stage = [&](int b, uint32_t id, unsigned mask) {
+    if ((mask >> lane) & 1u) {
+      const float4 *src = recs + (size_t)id * 4;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) cp_async16(&s_rec[b][w][lane], src + w);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  // One entry: advances T and Sg and gives the terms x of its 2D gradient for
+  // this lane's pixel; whether any lane takes it (a recorded entry has one: the
+  // forward took it for the same pixels by the same arithmetic).
+  constexpr int kTerms = !FULL ? 4 : MOMENTS ? 7 : 10;
+  auto entry = [&](const float4 (*rec)[32], int j, int k, bool recorded, float (&x)[kTerms], float &dy, uint32_t &id) {
+    // evaluated by every lane, without branches: a lane past its last
+    // contributor or below alpha_min keeps T and Sg and carries zero
+    // gradients, so each contributing lane's values are those of the
+    // branching form, operation for operation
+    const float4 a = rec[0][j], b = rec[1][j];
+    const float dx = (a.x - fpx) + a.z;
+    dy = (a.y - fpy) + a.w;
+    const float bxdx = b.x * dx, bydx = b.y * dx, bzdy = b.z * dy;
+    const float p = fmaf(bxdx, dx, fmaf(bydx, dy, fmaf(bzdy, dy, b.w)));
+    const bool contrib = k < lastp && p >= r.log2_alpha_min;
+    if (COUNT) { n_eval += k < lastp ? 1u : 0u; n_contrib += contrib ? 1u : 0u; }
+    const float ag = hw_exp2(p);
+    // zero for a lane that does not take the entry: 1 / (1 - alpha) is
+    // then exactly 1, T is kept, and the weight and the suffix update
+    // vanish without a select
+    const float alpha = contrib ? fminf(r.alpha_max, ag) : 0.f;
+    const float inv = hw_rcp(1.f - alpha);
+    T *= inv;                            // transmittance in front of this Gaussian
+    const float wk = alpha * T;
+    const float4 c = rec[2][j], d = rec[3][j];
+    // dL/dalpha = sum_ch g_ch (c_ch T - S_ch / (1 - alpha))
+    const float gcv = fmaf(g0, c.z, fmaf(g1, c.w, fmaf(g2, d.x, fmaf(g3, c.x, fmaf(g5, c.y, g4)))));
+    const float dal = fmaf(gcv, T, -Sg * inv);
+    // below the clamp, d alpha / d(natural exponent) = alpha (at the clamp
+    // alpha does not move with the exponent)
+    const float dpw = contrib && ag <= r.alpha_max ? dal * alpha : 0.f;
+    const float gz = g3 * wk;
+    const float tx = dpw * dx;
+    Sg = fmaf(gcv, wk, Sg);
+    id = __float_as_uint(d.w);
+    if constexpr (MOMENTS && FULL) {
+      x[0] = tx; x[1] = tx * dx; x[2] = gz; x[3] = g0 * wk; x[4] = g1 * wk; x[5] = g2 * wk; x[6] = dpw;
+    } else if constexpr (MOMENTS) {
+      x[0] = tx; x[1] = tx * dx; x[2] = gz; x[3] = dpw;
+    } else {
+      // the exponent in log2 units is p, so d/dx of the natural exponent is
+      // ln2 dp/dx: d p / d(u, v) = (2 a' dx + b' dy, b' dx + 2 c' dy) from the
+      // exponent's products; d(natural exponent) / d(conic) = -(dx^2 / 2,
+      // dx dy, dy^2 / 2)
+      const float hl = dpw * kLn2, ty = dpw * dy;
+      x[0] = hl * fmaf(2.f, bxdx, b.y * dy); x[1] = hl * fmaf(2.f, bzdy, bydx); x[2] = -0.5f * (tx * dx);
+      x[3] = -(tx * dy); x[4] = -0.5f * (ty * dy); x[5] = gz; x[6] = dpw; x[7] = g0 * wk; x[8] = g1 * wk;
+      x[9] = g2 * wk;
+    }
+    return recorded || __any_sync(FULLM, contrib);
+  };
+  // the warp sum of this lane's word
+  auto sums = [&](const float (&x)[kTerms], float dy) {
+    if constexpr (MOMENTS) return moment_sums<kTerms>(x, dy, lane);
+    else return warp_reduce_scatter<kTerms, 16>(x, lane);
+  };
+  // groups from the last contributor's down; the ids of the group after next
+  // and the records of the next are in flight while a group is worked on
+  int g = wmax > 0 ? (wmax - 1) >> 5 : -1, cur = 0;
+  uint32_t id_next = 0u;
+  unsigned mask_cur = 0u, mask_next = 0u;
+  if (g >= 0) {
+    uint32_t id;
+    group(g, id, mask_cur);
+    if (g > 0) group(g - 1, id_next, mask_next);
+    stage(0, id, mask_cur);
+  }
+  for (; g >= 0; --g, cur ^= 1) {
+    stage(cur ^ 1, id_next, mask_next);      // (nothing when g is 0)
+    unsigned mask = mask_cur;
+    mask_cur = mask_next;
+    mask_next = 0u;
+    if (g > 1) group(g - 2, id_next, mask_next);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp();
+    const float4(*const rec)[32] = s_rec[cur];
+    const bool recorded = MASKS && g < kMaskGroups;
+    if (!recorded) {
+      // later groups, or no record: the entries whose box meets the block
+      bool hit = false;
+      if ((mask >> lane) & 1u) {
+        const float4 a = rec[0][lane], d = rec[3][lane];
+        hit = fabsf(a.x - bcx) <= d.y + 3.5f && fabsf(a.y - bcy) <= d.z + 1.5f;
       }
-      const int lim = top - g * 32;
-      if (lim < 32) mask &= (1u << lim) - 1u;
-      while (mask) {
-        const int bit = 31 - __clz(mask);
-        mask &= ~(1u << bit);
-        const int j = g * 32 + bit;
-        const int k = beg + j;
-        // evaluated by every lane, without branches: a lane past its last
-        // contributor or below alpha_min keeps T and Sg and carries zero
-        // gradients, so each contributing lane's values are those of the
-        // branching form, operation for operation
-        const float4 a = s_a[j], b = s_b[j];
-        const float dx = (a.x - fpx) + a.z, dy = (a.y - fpy) + a.w;
-        const float bxdx = b.x * dx, bydx = b.y * dx, bzdy = b.z * dy;
-        const float p = fmaf(bxdx, dx, fmaf(bydx, dy, fmaf(bzdy, dy, b.w)));
-        const bool contrib = k < lastp && p >= r.log2_alpha_min;
-        if (COUNT) { n_eval += k < lastp ? 1u : 0u; n_contrib += contrib ? 1u : 0u; }
-        const float ag = hw_exp2(p);
-        // zero for a lane that does not take the entry: 1 / (1 - alpha) is
-        // then exactly 1, T is kept, and the weight and the suffix update
-        // vanish without a select
-        const float alpha = contrib ? fminf(r.alpha_max, ag) : 0.f;
-        const float inv = hw_rcp(1.f - alpha);
-        T *= inv;                            // transmittance in front of this Gaussian
-        const float wk = alpha * T;
-        const float4 c = s_c[j];
-        // dL/dalpha = sum_ch g_ch (c_ch T - S_ch / (1 - alpha))
-        const float gcv = fmaf(g0, c.z, fmaf(g1, c.w, fmaf(g2, s_bl[j], fmaf(g3, c.x, fmaf(g5, c.y, g4)))));
-        const float dal = fmaf(gcv, T, -Sg * inv);
-        // below the clamp, d alpha / d(natural exponent) = alpha (at the clamp
-        // alpha does not move with the exponent)
-        const float dpw = contrib && ag <= r.alpha_max ? dal * alpha : 0.f;
-        const float gz = g3 * wk;
-        const float tx = dpw * dx;
-        Sg = fmaf(gcv, wk, Sg);
-        // a recorded entry has a contributing lane: the forward took it for
-        // the same pixels by the same arithmetic
-        if (recorded || __any_sync(FULLM, contrib)) {
-          float sum;
-          if constexpr (MOMENTS) {
-            sum = moment_sums<FULL>(dpw, tx, tx * dx, gz, g0 * wk, g1 * wk, g2 * wk, dy, lane);
-          } else {
-            // the exponent in log2 units is p, so d/dx of the natural exponent
-            // is ln2 dp/dx: d p / d(u, v) = (2 a' dx + b' dy, b' dx + 2 c' dy)
-            // from the exponent's products; d(natural exponent) / d(conic) =
-            // -(dx^2 / 2, dx dy, dy^2 / 2). A reduce-scatter leaves every lane
-            // the warp sum of one word
-            const float hl = dpw * kLn2, ty = dpw * dy;
-            const float v10[10] = {hl * fmaf(2.f, bxdx, b.y * dy), hl * fmaf(2.f, bzdy, bydx), -0.5f * (tx * dx),
-                                   -(tx * dy), -0.5f * (ty * dy), gz, dpw, g0 * wk, g1 * wk, g2 * wk};
-            sum = warp_reduce_scatter<10, 16>(v10, lane);
-          }
-          if (writer) atomicAdd(gdst + (size_t)s_slot[j] * kGradWords, sum);
-        }
+      mask = __ballot_sync(FULLM, hit);
+    }
+    // two entries at a time: the second's arithmetic and reduction fill the
+    // latencies of the first's
+    while (mask) {
+      float x0[kTerms], x1[kTerms], dy0, dy1;
+      uint32_t id0, id1;
+      const int j0 = 31 - __clz((int)mask);
+      mask &= ~(1u << j0);
+      const bool any0 = entry(rec, j0, g * 32 + j0, recorded, x0, dy0, id0);
+      if (mask) {
+        const int j1 = 31 - __clz((int)mask);
+        mask &= ~(1u << j1);
+        const bool any1 = entry(rec, j1, g * 32 + j1, recorded, x1, dy1, id1);
+        const float s0 = sums(x0, dy0), s1 = sums(x1, dy1);
+        if (any0 && writer) atomicAdd(gdst + (size_t)id0 * kGradWords, s0);
+        if (any1 && writer) atomicAdd(gdst + (size_t)id1 * kGradWords, s1);
+      } else if (any0) {
+        const float s0 = sums(x0, dy0);
+        if (writer) atomicAdd(gdst + (size_t)id0 * kGradWords, s0);
       }
     }
+    __syncwarp();   // the group's buffer is staged again in the next round
   }
   if (COUNT) add_eval_counts(ws, 1, n_eval, n_contrib);
   // the fixed-bucket layout's counts start at zero for the next preprocess
   // (the adjoint is the last reader of the tile's range)
-  if (ws.bucket_cap && tid == 0) ws.tile_count[tile] = 0u;
+  if (ws.bucket_cap && warp == 0 && lane == 0) ws.tile_count[tile] = 0u;
 }
 
 // Chains the 2D gradients of the Gaussian projected as q in view slot `slot`
@@ -636,7 +657,7 @@ preprocess_bwd_kernel(Workspace ws, const float4 *__restrict__ gauss, int64_t n,
 // cancels by two to three digits over the map, and a caller that takes it in
 // FP64 beside the map's gradients gets it with the rounding of the per-pixel
 // form (either form is about 3e-7 from 64 bits on the 2,000-Gaussian scene).
-// Gradients of 200k Gaussians over 8 views of 640x480: the adjoint takes 354 us
+// Gradients of 200k Gaussians over 8 views of 640x480: the adjoint takes 333 us
 // with moments over the entries the forward recorded, 421 us per pixel over
 // every entry whose box meets the warp's block.
 static bool backward_moments(bool full, bool pose) { return !(full && pose); }
@@ -645,10 +666,10 @@ cudaError_t launch_render_bwd(const Workspace &ws, int views, int64_t n, const R
                               const float4 *targets, const float *image, const int32_t *last, bool full, bool pose,
                               cudaStream_t s, const float *upstream) {
   (void)n;
-  const dim3 grid((unsigned)(views * r.T));
+  const dim3 grid((unsigned)(views * r.T) * kBlocks);
   const bool masks = ws.warp_masks != nullptr, count = ws.count_evals != 0;
 #define DAGS_BWD(F, M, K, C) \
-  launch_pdl(render_bwd_kernel<F, M, K, C>, grid, dim3(kTilePix), 0, s, ws, r, l, targets, image, last, upstream)
+  launch_pdl(render_bwd_kernel<F, M, K, C>, grid, dim3(32), 0, s, ws, r, l, targets, image, last, upstream)
 #define DAGS_BWD_KC(F, M) \
   (masks ? (count ? DAGS_BWD(F, M, true, true) : DAGS_BWD(F, M, true, false)) \
          : (count ? DAGS_BWD(F, M, false, true) : DAGS_BWD(F, M, false, false)))

@@ -277,7 +277,7 @@ __device__ __forceinline__ void preprocess_one(const Workspace &ws, const Rec &r
     const float *P = sp + v * 12;
     const size_t slot = (size_t)v * ws.max_n + i;
 
-    float4 o0 = make_float4(0.f, 0.f, 0.f, 0.f), o1 = o0, o2 = o0;
+    float4 o0 = make_float4(0.f, 0.f, 0.f, 0.f), o1 = o0, o2 = o0, o3 = o0;
     float2 ulo = make_float2(0.f, 0.f);
     uint2 rect = make_uint2(0u, 0u);
     Proj q;
@@ -303,19 +303,21 @@ __device__ __forceinline__ void preprocess_one(const Workspace &ws, const Rec &r
       const int x1 = clampi(floorf((q.u + ex) * inv_tile) + 1.f, 0, r.tiles_x);
       const int y1 = clampi(floorf((q.v + ey) * inv_tile) + 1.f, 0, r.tiles_y);
       if (thr > 0.f && x1 > x0 && y1 > y0 && isfinite(q.u) && isfinite(q.v)) {
-        o0 = make_float4(q.u, q.v, ex, ey);
+        const uint32_t rg = __float_as_uint(g3.x), bl = __float_as_uint(g3.y);
+        o0 = make_float4(q.u, q.v, ulo.x, ulo.y);
         o1 = make_float4(-0.5f * kLog2e * q.ca, -kLog2e * q.cb, -0.5f * kLog2e * q.cc, lo);
-        o2 = make_float4(q.z, g2.w, g3.x, g3.y);
+        o2 = make_float4(q.z, g2.w, bf16_lo(rg), bf16_hi(rg));
+        o3 = make_float4(bf16_lo(bl), ex, ey, __uint_as_float((uint32_t)i));
         rect = make_uint2((uint32_t)x0 | ((uint32_t)x1 << 16), (uint32_t)y0 | ((uint32_t)y1 << 16));
       }
     }
     // invisible Gaussians only need their empty rect: nothing reads their
     // projected record or 2D gradient
     if ((rect.x >> 16) > (rect.x & 0xFFFF)) {
-      ws.rec2d[slot * 3 + 0] = o0;
-      ws.rec2d[slot * 3 + 1] = o1;
-      ws.rec2d[slot * 3 + 2] = o2;
-      ws.rec_lo[slot] = ulo;
+      ws.rec2d[slot * 4 + 0] = o0;
+      ws.rec2d[slot * 4 + 1] = o1;
+      ws.rec2d[slot * 4 + 2] = o2;
+      ws.rec2d[slot * 4 + 3] = o3;
       float4 *gz = reinterpret_cast<float4 *>(ws.grad2d + slot * kGradWords);
       for (int w = 0; w < zero_words / 4; ++w) gz[w] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
@@ -538,9 +540,9 @@ emit_kernel(Workspace ws, int64_t n, Raster r) {
   if (i < nv) {
     const size_t slot = (size_t)v * ws.max_n + min(id, (uint32_t)(n - 1));
     rect = ws.rect[slot];
-    r0 = ws.rec2d[slot * 3 + 0];
-    r1 = ws.rec2d[slot * 3 + 1];
-    z = ws.rec2d[slot * 3 + 2].x;
+    r0 = ws.rec2d[slot * 4 + 0];
+    r1 = ws.rec2d[slot * 4 + 1];
+    z = ws.rec2d[slot * 4 + 2].x;
   } else {
     id = 0;
   }
@@ -551,8 +553,7 @@ emit_kernel(Workspace ws, int64_t n, Raster r) {
 // issue (73-75% issue-active, ALU pipe busiest), so what is per (warp, entry)
 // pair is kept short: a lane's contributions of a 32-entry group are one bit
 // each in `took`, from which the last contributor and, by one reduction per
-// group, the warp's record for the adjoint (ws.warp_masks) follow; the BF16
-// colour is widened once per staged entry.
+// group, the warp's record for the adjoint (ws.warp_masks) follow.
 template <bool COUNT>
 __global__ void __launch_bounds__(kTilePix, 5)
 render_fwd_kernel(Workspace ws, int views, Raster r, Loss l, const float4 *__restrict__ targets,
@@ -620,15 +621,12 @@ render_fwd_kernel(Workspace ws, int views, Raster r, Loss l, const float4 *__res
     const uint32_t id = k < e ? (own_sort ? (uint32_t)s_key[k - s] : ws.sorted_ids[k]) : 0u;
     if (k < e && DAGS_IN_BOUNDS(id < (uint32_t)ws.max_n && k < (uint64_t)ws.max_pairs, ws.counters + CNT_STATUS)) {
       const size_t slot = vbase + id;
-      const float4 r0 = ws.rec2d[slot * 3 + 0];
-      const float2 lo = ws.rec_lo[slot];
-      s_a[tid] = make_float4(r0.x, r0.y, lo.x, lo.y);
-      s_e[tid] = make_float2(r0.z, r0.w);
-      s_b[tid] = ws.rec2d[slot * 3 + 1];
-      const float4 r2 = ws.rec2d[slot * 3 + 2];
-      const uint32_t rg = __float_as_uint(r2.z), bl = __float_as_uint(r2.w);
-      s_c[tid] = make_float4(r2.x, r2.y, bf16_lo(rg), bf16_hi(rg));
-      s_bl[tid] = bf16_lo(bl);
+      const float4 r3 = ws.rec2d[slot * 4 + 3];
+      s_a[tid] = ws.rec2d[slot * 4 + 0];
+      s_b[tid] = ws.rec2d[slot * 4 + 1];
+      s_c[tid] = ws.rec2d[slot * 4 + 2];
+      s_e[tid] = make_float2(r3.y, r3.z);
+      s_bl[tid] = r3.x;
     }
     __syncthreads();
     const int cnt = (int)min((uint32_t)kTilePix, e - base);
