@@ -135,7 +135,7 @@ void free_mp(MpBuffers &b) {
 }
 
 void free_lm(LmBuffers &b) {
-  void *ptrs[] = {b.tan, b.partial, b.normal, b.pose_try};
+  void *ptrs[] = {b.tan, b.block_partial, b.partial, b.group_partial, b.done, b.normal, b.pose_try};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   b = LmBuffers();
@@ -834,10 +834,16 @@ int ensure_lm(dags_ctx *ctx) {
   cudaError_t e = cudaSuccess;
   auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
   A(alloc(&b.tan, (size_t)ctx->ws.max_n * 9));
-  A(alloc(&b.partial, (size_t)ctx->ws.max_tiles * DAGS_LM_NORMAL));
+  const size_t tiles = (size_t)ctx->ws.max_tiles, groups = (tiles + kLmTileGroup - 1) / kLmTileGroup;
+  A(alloc(&b.block_partial, tiles * (kTilePix / 32) * DAGS_LM_NORMAL));
+  A(alloc(&b.partial, tiles * DAGS_LM_NORMAL));
+  A(alloc(&b.group_partial, groups * DAGS_LM_NORMAL));
+  A(alloc(&b.done, tiles + groups + 1));
   A(alloc(&b.normal, (size_t)DAGS_LM_NORMAL));
   A(alloc(&b.pose_try, (size_t)12));
-  A(lm_kernel_setup());
+  // (synchronous: the first call's kernels may be on any stream)
+  if (e == cudaSuccess) e = cudaMemset(b.done, 0, (tiles + groups + 1) * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     cudaGetLastError();
     free_lm(b);
@@ -887,8 +893,8 @@ int normal_core(dags_ctx *ctx, const float *gauss, int64_t n, const dags_camera 
   }
   if (e == cudaSuccess) {
     ev = tm.begin(DAGS_K_RENDER_JAC, s);
-    e = launch_render_jac(w, r, l, delta, reinterpret_cast<const float4 *>(targets), ctx->lm.tan, ctx->lm.partial,
-                          normal, jac, image, last, fuse, s);
+    e = launch_render_jac(w, r, l, delta, reinterpret_cast<const float4 *>(targets), ctx->lm, normal, jac, image, last,
+                          fuse, s);
     tm.end(ev, s);
   }
   (void)cam;
@@ -898,7 +904,7 @@ int normal_core(dags_ctx *ctx, const float *gauss, int64_t n, const dags_camera 
 int lm_iteration(dags_ctx *ctx, const float *gauss, int64_t n, const dags_camera *cam, double *pose,
                  const float *targets, const Raster &r, const Loss &l, const dags_lm_cfg &c, double *state,
                  bool follows_iteration, cudaStream_t s) {
-  // the LM step runs in the last CTA of the Jacobian render
+  // the LM step runs in the last warp of the Jacobian render
   LmFuse fuse;
   fuse.state = state;
   fuse.pose_try = ctx->lm.pose_try;

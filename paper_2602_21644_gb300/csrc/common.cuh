@@ -214,16 +214,19 @@ cudaError_t launch_gauss_adam(float *gauss, float *colour, float *m, float *v, c
                               int64_t step, const dags_gauss_adam_cfg &c, cudaStream_t s);
 
 // Levenberg-Marquardt pose refinement (lm.cu).
+constexpr int kLmTileGroup = 32;   // tiles per group of the normal equations' FP64 sums
 struct LmBuffers {
   float4 *tan = nullptr;      // [max_n][9] twist tangents of the projected records (view 0)
-  float *partial = nullptr;   // [max_tiles][28] tile partials of the normal equations
+  float *block_partial = nullptr;   // [max_tiles][8][28] pixel blocks' sums of the normal equations
+  float *partial = nullptr;         // [max_tiles][28] tiles' sums
+  double *group_partial = nullptr;  // [groups of max_tiles][28] tile groups' sums
+  uint32_t *done = nullptr;   // [max_tiles + groups + 1] arrivals of a render (zero between renders)
   double *normal = nullptr;   // [28] the loop's normal equations
   double *pose_try = nullptr; // [12] the loop's linearisation point
 };
-cudaError_t lm_kernel_setup();
 cudaError_t launch_pose_tangents(const Workspace &ws, const float4 *gauss, int64_t n, const Raster &r, float4 *tan,
                                  int num_sms, cudaStream_t s);
-// Optional LM step fused into the last CTA of the Jacobian render.
+// Optional LM step fused into the last warp of the Jacobian render.
 struct LmFuse {
   double *state = nullptr;      // nullptr: no step
   double *pose_try = nullptr;
@@ -231,8 +234,8 @@ struct LmFuse {
   dags_lm_cfg cfg;
 };
 cudaError_t launch_render_jac(const Workspace &ws, const Raster &r, const Loss &l, float delta,
-                              const float4 *targets, const float4 *tan, float *partial, double *normal, float *jac,
-                              float *image, int32_t *last, const LmFuse &fuse, cudaStream_t s);
+                              const float4 *targets, const LmBuffers &buf, double *normal, float *jac, float *image,
+                              int32_t *last, const LmFuse &fuse, cudaStream_t s);
 cudaError_t launch_lm_init(const double *pose, double *state, double *pose_try, double mu0, cudaStream_t s);
 cudaError_t launch_lm_step(const double *normal, double *state, double *pose_try, double *pose_best,
                            const dags_lm_cfg &c, cudaStream_t s);
@@ -384,6 +387,30 @@ __device__ __forceinline__ float hw_rcp(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+
+// Two FP32 values in a register pair and the packed operations of sm_100-class
+// GPUs: each half is rounded as the scalar operation rounds it; one instruction
+// issues where two would (the FMA pipe takes two cycles for it).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ f32x2 dup2(float x) { return pack2(x, x); }
+__device__ __forceinline__ void unpack2(f32x2 a, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
 }
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
@@ -712,6 +739,46 @@ __device__ inline void pose_adam_exp(double *T, const double *grad, double *st, 
   se3_exp_left(T, xi);
 }
 
+// exp(xi^) T spread over threads: thread 0 forms the scalar series (sc:
+// sin(t)/t, (1 - cos t)/t^2, (t - sin t)/t^3 of the angle t) and, once they are
+// visible, thread e = 0..11 one entry of the new 3x4 pose.
+__device__ inline void se3_exp_coeffs(const double *xi, double *sc, int thread) {
+  if (thread != 0) return;
+  const double t2 = xi[3] * xi[3] + xi[4] * xi[4] + xi[5] * xi[5];
+  double a, b, c;
+  if (t2 < 0.0625) {
+    a = 1.0 + t2 * (-1.0 / 6 + t2 * (1.0 / 120 + t2 * (-1.0 / 5040 + t2 * (1.0 / 362880 + t2 * (-1.0 / 39916800 +
+        t2 * (1.0 / 6227020800.0))))));
+    b = 0.5 + t2 * (-1.0 / 24 + t2 * (1.0 / 720 + t2 * (-1.0 / 40320 + t2 * (1.0 / 3628800 + t2 * (-1.0 / 479001600 +
+        t2 * (1.0 / 87178291200.0))))));
+    c = 1.0 / 6 + t2 * (-1.0 / 120 + t2 * (1.0 / 5040 + t2 * (-1.0 / 362880 + t2 * (1.0 / 39916800 +
+        t2 * (-1.0 / 6227020800.0 + t2 * (1.0 / 1307674368000.0))))));
+  } else {
+    const double th = sqrt(t2);
+    a = sin(th) / th;
+    b = (1.0 - cos(th)) / t2;
+    c = (th - sin(th)) / (t2 * th);
+  }
+  sc[0] = a; sc[1] = b; sc[2] = c;
+}
+
+__device__ inline double se3_exp_entry(const double *T, const double *xi, const double *sc, int e) {
+  const int i = e >> 2, j = e & 3;
+  const double px = xi[3], py = xi[4], pz = xi[5];
+  const double Kh[9] = {0.0, -pz, py, pz, 0.0, -px, -py, px, 0.0};
+  double Re[3], V[3];
+#pragma unroll
+  for (int kk = 0; kk < 3; ++kk) {
+    const double K2 = Kh[3 * i] * Kh[kk] + Kh[3 * i + 1] * Kh[3 + kk] + Kh[3 * i + 2] * Kh[6 + kk];
+    const double I = (i == kk) ? 1.0 : 0.0;
+    Re[kk] = I + sc[0] * Kh[3 * i + kk] + sc[1] * K2;
+    V[kk] = I + sc[1] * Kh[3 * i + kk] + sc[2] * K2;
+  }
+  double out = Re[0] * T[j] + Re[1] * T[4 + j] + Re[2] * T[8 + j];
+  if (j == 3) out += V[0] * xi[0] + V[1] * xi[1] + V[2] * xi[2];
+  return out;
+}
+
 // The same pose step spread over the first 12 threads of a CTA (dependent
 // FP64 chains are what costs on GB300): threads 0-5 update one twist
 // component's Adam moments each, thread 0 the scalar series, threads 0-11
@@ -749,42 +816,10 @@ __device__ inline void pose_adam_exp_cta(double *T, const double *grad, double *
   __syncthreads();
   if (t < 6) xi_s[t] = -cfg.lr[t] * (m * sc_s[0]) / (rs * sc_s[1] + cfg.eps);
   __syncthreads();
-  if (t == 0) {
-    st[12] = k;
-    const double t2 = xi_s[3] * xi_s[3] + xi_s[4] * xi_s[4] + xi_s[5] * xi_s[5];
-    double a, b, c;
-    if (t2 < 0.0625) {
-      a = 1.0 + t2 * (-1.0 / 6 + t2 * (1.0 / 120 + t2 * (-1.0 / 5040 + t2 * (1.0 / 362880 + t2 * (-1.0 / 39916800 +
-          t2 * (1.0 / 6227020800.0))))));
-      b = 0.5 + t2 * (-1.0 / 24 + t2 * (1.0 / 720 + t2 * (-1.0 / 40320 + t2 * (1.0 / 3628800 + t2 * (-1.0 / 479001600 +
-          t2 * (1.0 / 87178291200.0))))));
-      c = 1.0 / 6 + t2 * (-1.0 / 120 + t2 * (1.0 / 5040 + t2 * (-1.0 / 362880 + t2 * (1.0 / 39916800 +
-          t2 * (-1.0 / 6227020800.0 + t2 * (1.0 / 1307674368000.0))))));
-    } else {
-      const double th = sqrt(t2);
-      a = sin(th) / th;
-      b = (1.0 - cos(th)) / t2;
-      c = (th - sin(th)) / (t2 * th);
-    }
-    sc_s[0] = a; sc_s[1] = b; sc_s[2] = c;
-  }
+  if (t == 0) st[12] = k;
+  se3_exp_coeffs(xi_s, sc_s, t);
   __syncthreads();
-  double out = 0.0;
-  if (t < 12) {
-    const int i = t >> 2, j = t & 3;
-    const double px = xi_s[3], py = xi_s[4], pz = xi_s[5];
-    const double Kh[9] = {0.0, -pz, py, pz, 0.0, -px, -py, px, 0.0};
-    double Re[3], V[3];
-#pragma unroll
-    for (int kk = 0; kk < 3; ++kk) {
-      const double K2 = Kh[3 * i] * Kh[kk] + Kh[3 * i + 1] * Kh[3 + kk] + Kh[3 * i + 2] * Kh[6 + kk];
-      const double I = (i == kk) ? 1.0 : 0.0;
-      Re[kk] = I + sc_s[0] * Kh[3 * i + kk] + sc_s[1] * K2;
-      V[kk] = I + sc_s[1] * Kh[3 * i + kk] + sc_s[2] * K2;
-    }
-    out = Re[0] * T[j] + Re[1] * T[4 + j] + Re[2] * T[8 + j];
-    if (j == 3) out += V[0] * xi_s[0] + V[1] * xi_s[1] + V[2] * xi_s[2];
-  }
+  const double out = t < 12 ? se3_exp_entry(T, xi_s, sc_s, t) : 0.0;
   __syncthreads();
   if (t < 12) T[t] = out;
 }

@@ -11,19 +11,20 @@
 //   pose_tangent_kernel   per visible Gaussian, the derivative of its 2D
 //                         record (centre, conic in log2 units, depth) along
 //                         the six twist directions xi = (rho, phi) of the
-//                         left perturbation T <- exp(xi^) T
-//   render_jac_kernel     one CTA per 16x16 tile: the forward compositing
+//                         left perturbation T <- exp(xi^) T; beside it, one CTA
+//                         per tile depth-sorts the tile's bucket
+//   render_jac_kernel     one warp per 8x4 pixel block: the forward compositing
 //                         with forward-mode tangents (the derivative of alpha,
 //                         of the transmittance and of the composited colour
 //                         and depth, 30 accumulators per pixel), then per
-//                         pixel the loss and W J J^T, W r J; tile partials in
-//                         FP32, the last CTA sums them in FP64 in a fixed order
-//                         into (L, H, g)
+//                         pixel the loss and W J J^T, W r J; summed per block
+//                         and tile in FP32 and over tiles in FP64, each in a
+//                         fixed order, into (L, H, g)
 //   LM step               FP64, one thread on shared-memory copies: accept the
 //                         linearisation point if its loss is lower, adapt the
 //                         damping, solve the damped 6x6 system by Cholesky and
 //                         step the pose; inside the tracking loop it runs in
-//                         the last CTA of render_jac_kernel, on its own as
+//                         the last warp of render_jac_kernel, on its own as
 //                         lm_step_kernel
 //
 // The kernels use programmatic dependent launch like the other splatting
@@ -35,29 +36,48 @@ namespace dags {
 
 namespace {
 
-constexpr int kJacBatch = kTilePix;   // list entries staged in shared memory per round (one per thread)
-constexpr int kJacTanBytes = kJacBatch * 9 * 16;   // their tangent records (dynamic shared memory)
+constexpr int kJacChunk = 8;    // entries a warp stages at a time
 constexpr int kTan4 = 9;         // float4 per Gaussian tangent record (36 floats)
 constexpr int kNormal = 28;      // L, the upper triangle of H (21), g (6)
+constexpr int kTanBlock = kTilePix;      // threads per CTA of the tangents and the sort
+constexpr int kBlocks = kTilePix / 32;   // pixel blocks per tile
+constexpr int kTileGroup = kLmTileGroup; // tiles whose partials one warp sums in FP64
 
 // Tangent record of a visible Gaussian: for twist direction k = 0..5 the six
-// floats (du, dv, da', db', dc', dz) at offset 6k, where (a', b', c') are the
-// exponent coefficients of the projected record (log2 units).
-__global__ void __launch_bounds__(kPrepBlock, 6)
+// floats (du, dv, da', db', dc', dz), where (a', b', c') are the exponent
+// coefficients of the projected record (log2 units). Directions 2p and 2p + 1
+// are interleaved, so that a component of both is one aligned register pair.
+__host__ __device__ constexpr int tan_at(int k, int c) { return (k >> 1) * 12 + 2 * c + (k & 1); }
+
+// The grid: (tracking loop) one CTA that ranks the tiles by the previous
+// Jacobian render's counts into this iteration's render order, dispatched
+// first; one CTA per tile that sorts its bucket (an overflowed one is left);
+// CTAs that stride over the visible Gaussians. The sort needs nothing of the
+// tangents, so it fills the SMs beside them, and the render after it runs
+// without a CTA per tile.
+__global__ void __launch_bounds__(kTanBlock, 3)
 pose_tangent_kernel(Workspace ws, const float4 *__restrict__ gauss, int64_t n, Raster r,
                     float4 *__restrict__ tan) {
   pdl_wait();
-  // the tracking loop's bucket layout: the grid's first CTA (dispatched
-  // first, so that it runs beside the first wave) ranks the tiles by the
-  // previous Jacobian render's counts into this iteration's render order,
-  // and the visible list is still the preprocess's append cursor
-  const bool ordering = ws.order_next != nullptr;
+  const int ordering = ws.order_next != nullptr ? 1 : 0;
   if (ordering && blockIdx.x == 0) {
     rank_tiles(ws.prev_count, r.T, ws.order_next, ws.band);
     return;
   }
-  const int64_t nb = (int64_t)gridDim.x - (ordering ? 1 : 0);
-  const int64_t bid = (int64_t)blockIdx.x - (ordering ? 1 : 0);
+  const int64_t lead = ordering + (int64_t)r.T;
+  if ((int64_t)blockIdx.x < lead) {
+    __shared__ __align__(16) uint64_t s_key[kSortSmallCap];
+    const int tile = (int)blockIdx.x - ordering;
+    if (ws.bucket_cap ? ws.tile_count[tile] > ws.bucket_cap : pairs_overflow_ws(ws)) return;
+    uint32_t s, e;
+    tile_range(ws, tile, s, e);
+    sort_tile_bucket(ws, s, (int)(e - s), s_key);
+    return;
+  }
+  const int64_t nb = (int64_t)gridDim.x - lead;
+  const int64_t bid = (int64_t)blockIdx.x - lead;
+  // the tracking loop's bucket layout: the visible list is still the
+  // preprocess's append cursor
   const uint32_t nv = ws.bucket_cap ? ws.vis_append[0] : ws.vis_n[0];
   float P[12];
 #pragma unroll
@@ -117,12 +137,12 @@ pose_tangent_kernel(Workspace ws, const float4 *__restrict__ gauss, int64_t n, R
         const float dca = (dC - q.ca * ddet) * idet;
         const float dcb = (-dB - q.cb * ddet) * idet;
         const float dcc = (dA - q.cc * ddet) * idet;
-        out[6 * k + 0] = r.fx * (dp[0] * z - x * dp[2]) * iz2;
-        out[6 * k + 1] = r.fy * (dp[1] * z - y * dp[2]) * iz2;
-        out[6 * k + 2] = -0.5f * kLog2e * dca;
-        out[6 * k + 3] = -kLog2e * dcb;
-        out[6 * k + 4] = -0.5f * kLog2e * dcc;
-        out[6 * k + 5] = dp[2];
+        out[tan_at(k, 0)] = r.fx * (dp[0] * z - x * dp[2]) * iz2;
+        out[tan_at(k, 1)] = r.fy * (dp[1] * z - y * dp[2]) * iz2;
+        out[tan_at(k, 2)] = -0.5f * kLog2e * dca;
+        out[tan_at(k, 3)] = -kLog2e * dcb;
+        out[tan_at(k, 4)] = -0.5f * kLog2e * dcc;
+        out[tan_at(k, 5)] = dp[2];
       }
     }
     float4 *o = tan + (size_t)id * kTan4;
@@ -139,111 +159,132 @@ __host__ __device__ constexpr int tri(int a, int b) { return a * 6 - a * (a - 1)
 enum { ST_T = 0, ST_L = 12, ST_MU = 13, ST_H = 14, ST_G = 35, ST_ACC = 41, ST_IT = 42, ST_LAST_L = 43,
        ST_LAST_A = 44 };
 
-// One LM decision and damped step by one thread, on shared-memory copies:
-// n the normal equations at p (the linearisation point), st the state; on
-// return st is updated and p holds the next linearisation point.
-__device__ void lm_decide_solve(const double *n, double *st, double *p, const dags_lm_cfg &c) {
-  const double L = n[0];
-  double mu = st[ST_MU];
-  const bool accept = L < st[ST_L];
+// The LM step by one warp (all lanes must call it): decide, solve the damped
+// system and step the pose, on shared-memory copies of the normal equations at
+// the linearisation point, the state and the pose. FP64 instructions are what
+// it costs (each occupies the pipe as long for one lane as for 32, and they
+// depend on one another), so the factorisation, the solves and the exponential
+// are spread over the lanes: 7 us against 10 for one lane.
+__device__ void lm_step_warp(const double *nrm, double *state, double *pose_try, double *pose_best,
+                             const dags_lm_cfg &c) {
+  __shared__ double s_st[DAGS_LM_STATE], s_A[6][6], s_x[6], s_sc[3];
+  const unsigned FULL = 0xffffffffu;
+  const int t = threadIdx.x & 31;
+  const bool accept = nrm[0] < state[ST_L];
+  double mu = state[ST_MU];
+  mu = accept ? fmax(mu * c.down, c.mu_min) : fmin(mu * c.up, c.mu_max);
+  for (int k = t; k < DAGS_LM_STATE; k += 32) s_st[k] = state[k];
+  __syncwarp();
   if (accept) {
-    for (int k = 0; k < 12; ++k) st[ST_T + k] = p[k];
-    st[ST_L] = L;
-    for (int k = 0; k < 21; ++k) st[ST_H + k] = n[1 + k];
-    for (int k = 0; k < 6; ++k) st[ST_G + k] = n[22 + k];
-    mu = fmax(mu * c.down, c.mu_min);
-    st[ST_ACC] += 1.0;
-  } else {
-    mu = fmin(mu * c.up, c.mu_max);
+    if (t < 12) s_st[ST_T + t] = pose_try[t];
+    if (t < 21) s_st[ST_H + t] = nrm[1 + t];
+    if (t < 6) s_st[ST_G + t] = nrm[22 + t];
   }
-  st[ST_MU] = mu;
-  st[ST_IT] += 1.0;
-  st[ST_LAST_L] = L;
-  st[ST_LAST_A] = accept ? 1.0 : 0.0;
-  // (H + mu diag(H) + floor tr(H)/6 I) delta = -g by Cholesky
-  double A[6][6], d[6];
+  if (t == 0) {
+    if (accept) {
+      s_st[ST_L] = nrm[0];
+      s_st[ST_ACC] += 1.0;
+    }
+    s_st[ST_MU] = mu;
+    s_st[ST_IT] += 1.0;
+    s_st[ST_LAST_L] = nrm[0];
+    s_st[ST_LAST_A] = accept ? 1.0 : 0.0;
+  }
+  __syncwarp();
+  // (H + mu diag(H) + floor tr(H)/6 I) delta = -g by Cholesky: lane (i, j) of
+  // the lower triangle holds A[i][j]; column k's lanes are scaled by the
+  // reciprocal square root of the pivot, then every lane to their right
+  // subtracts its product (the diagonal holds 1 / l_jj)
   double tr = 0.0;
-  for (int a = 0; a < 6; ++a) tr += st[ST_H + tri(a, a)];
+  for (int a = 0; a < 6; ++a) tr += s_st[ST_H + tri(a, a)];
   bool ok = tr > 0.0;
-  if (ok) {
-    for (int a = 0; a < 6; ++a)
-      for (int b = a; b < 6; ++b) A[a][b] = A[b][a] = st[ST_H + tri(a, b)];
-    for (int a = 0; a < 6; ++a) A[a][a] += mu * A[a][a] + c.floor * (tr / 6.0);
-    for (int j = 0; j < 6 && ok; ++j) {
-      double sjj = A[j][j];
-      for (int k = 0; k < j; ++k) sjj -= A[j][k] * A[j][k];
-      if (!(sjj > 0.0)) { ok = false; break; }
-      // the diagonal holds 1 / l_jj: one reciprocal square root per pivot and
-      // multiplications elsewhere (dependent FP64 divisions are what costs)
-      const double inv = rsqrt(sjj);
-      A[j][j] = inv;
-      for (int i = j + 1; i < 6; ++i) {
-        double sij = A[i][j];
-        for (int k = 0; k < j; ++k) sij -= A[i][k] * A[j][k];
-        A[i][j] = sij * inv;
-      }
-    }
+  int i = 0, j = t;                 // lane t < 21: row i, column j <= i
+  while (i < 5 && j > i) { j -= i + 1; ++i; }
+  const bool mine = t < 21;
+  double v = 0.0;
+  if (mine) {
+    v = s_st[ST_H + tri(j, i)];
+    if (i == j) v += mu * v + c.floor * (tr / 6.0);
   }
-  if (ok) {
-    double y[6];
-    for (int i = 0; i < 6; ++i) {
-      double t = -st[ST_G + i];
-      for (int k = 0; k < i; ++k) t -= A[i][k] * y[k];
-      y[i] = t * A[i][i];
+  for (int k = 0; k < 6; ++k) {
+    const int diag = k * (k + 1) / 2 + k;   // lane of A[k][k]
+    const double piv = __shfl_sync(FULL, v, diag);
+    if (!(piv > 0.0)) ok = false;
+    const double inv = rsqrt(piv);
+    if (mine && j == k) {
+      v = i == k ? inv : v * inv;
+      s_A[i][k] = v;
     }
-    for (int i = 5; i >= 0; --i) {
-      double t = y[i];
-      for (int k = i + 1; k < 6; ++k) t -= A[k][i] * d[k];
-      d[i] = t * A[i][i];
-    }
-  } else {
-    for (int i = 0; i < 6; ++i) d[i] = 0.0;
+    __syncwarp();
+    if (mine && j > k) v -= s_A[i][k] * s_A[j][k];
   }
-  double T[12];
-  for (int k = 0; k < 12; ++k) T[k] = st[ST_T + k];
-  se3_exp_left(T, d);
-  for (int k = 0; k < 12; ++k) p[k] = T[k];
-}
-
-// The LM step by a CTA of at least 48 threads (all must call it): the inputs
-// are staged in shared memory by parallel loads, one thread decides and
-// solves, and the results are written back in parallel.
-__device__ void lm_step_cta(const double *nrm, double *state, double *pose_try, double *pose_best,
-                            const dags_lm_cfg &c) {
-  __shared__ double s_n[kNormal], s_st[DAGS_LM_STATE], s_p[12];
-  const int t = threadIdx.x;
-  if (t < kNormal) s_n[t] = nrm[t];
-  if (t < DAGS_LM_STATE) s_st[t] = state[t];
-  if (t < 12) s_p[t] = pose_try[t];
-  __syncthreads();
-  if (t == 0) lm_decide_solve(s_n, s_st, s_p, c);
-  __syncthreads();
-  if (t < DAGS_LM_STATE) state[t] = s_st[t];
+  // forward and back substitution: lane i holds row i's running sum
+  double x = t < 6 ? -s_st[ST_G + t] : 0.0;
+  for (int k = 0; k < 6; ++k) {
+    const double y = __shfl_sync(FULL, x, k) * s_A[k][k];
+    if (t == k) x = y;
+    else if (t > k && t < 6) x -= s_A[t][k] * y;
+  }
+  for (int k = 5; k >= 0; --k) {
+    const double d = __shfl_sync(FULL, x, k) * s_A[k][k];
+    if (t == k) x = d;
+    else if (t < k) x -= s_A[k][t] * d;
+  }
+  if (t < 6) s_x[t] = ok ? x : 0.0;
+  __syncwarp();
+  // T <- exp(delta^) T, an entry to a lane
+  se3_exp_coeffs(s_x, s_sc, t);
+  __syncwarp();
+  const double out = t < 12 ? se3_exp_entry(s_st + ST_T, s_x, s_sc, t) : 0.0;
+  for (int k = t; k < DAGS_LM_STATE; k += 32) state[k] = s_st[k];
   if (t < 12) {
-    pose_try[t] = s_p[t];
+    pose_try[t] = out;
     pose_best[t] = s_st[ST_T + t];
   }
 }
 
-// Three CTAs per SM (a budget of 80 registers, 30 tangent accumulators per
-// pixel, some of them spilled to L1): the kernel is bound by instruction
-// issue, and six warps per scheduler hide more latency than the four that
-// the unspilled 118 registers allowed (146 against 160 us per launch at the
-// tracking size; four CTAs per SM spill more and take 154).
-__global__ void __launch_bounds__(kTilePix, 3)
+// One warp arrives at `counter`; true for the last of `count`, which then sees
+// what the others wrote before they arrived, and leaves the counter at zero.
+__device__ __forceinline__ bool arrive_last(uint32_t *counter, uint32_t count) {
+  __syncwarp();
+  uint32_t t = 0;
+  if ((threadIdx.x & 31) == 0) {
+    __threadfence();
+    t = atomicAdd(counter, 1u);
+    if (t == count - 1u) {
+      *counter = 0u;
+      __threadfence();
+    }
+  }
+  return __shfl_sync(0xffffffffu, t, 0) == count - 1u;
+}
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+// One warp, and one CTA, per 8 x 4 pixel block, as in the adjoint of the
+// first-order loop: bound by the latency of a warp's own chain (59% of the
+// issue slots used, FP32 pipe next) and by the number of warps that 30 tangent
+// accumulators per pixel leave room for (20 per SM at 96 registers; 24 spill
+// and are slower, as are 16 and 18). The six twist directions run in pairs on
+// the packed FP32 operations, so a pair's 84 operations issue as 42. 300k
+// Gaussians, 640x480, per launch: 146 us with a CTA of 8 warps per tile that
+// sorts its bucket, scalar (93M warp instructions) or packed (77M, the same
+// time: the tile's CTAs wait on one another); 129 us with a warp per block and
+// the sort beside the tangents (60M); 125 with the sums and the step spread
+// over warps and lanes; 121 without branches, the next entry read ahead.
+__global__ void __launch_bounds__(32, 20)
 render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__restrict__ targets,
-                  const float4 *__restrict__ tan, float *__restrict__ partial, double *__restrict__ normal,
+                  const float4 *__restrict__ tan, LmBuffers buf, double *__restrict__ normal,
                   float *__restrict__ jac, float *__restrict__ image, int32_t *__restrict__ last, LmFuse fuse) {
   pdl_wait();
-  __shared__ __align__(16) uint64_t s_key[kSortSmallCap];
-  __shared__ float4 s_a[kJacBatch], s_b[kJacBatch], s_c[kJacBatch];   // s_a: {u hi, v hi, u lo, v lo}
-  __shared__ float2 s_e[kJacBatch];                                   // box half extents
-  __shared__ float s_bl[kJacBatch];                                   // blue
-  extern __shared__ float4 s_t[];   // kJacBatch * kTan4
-  __shared__ float s_red[kTilePix / 32][kNormal];
-  __shared__ int s_last;
+  // records and tangent records of a chunk's entries, double-buffered
+  __shared__ float4 s_rec[2][4 + kTan4][kJacChunk];
   const unsigned FULL = 0xffffffffu;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int lane = threadIdx.x;
+  const int warp = (int)(blockIdx.x % kBlocks);   // the tile's pixel block
   // the tracking loop's fixed-capacity buckets: a tile whose list overflowed
   // its bucket is skipped and reported, and the render publishes the counts
   // and the visible count as the forward of the first-order loop does;
@@ -251,10 +292,10 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
   bool ovf;
   int tile;
   if (ws.bucket_cap) {
-    tile = (int)ws.tile_order[blockIdx.x];
+    tile = (int)ws.tile_order[blockIdx.x / kBlocks];
     const uint32_t c = ws.tile_count[tile];
     ovf = c > ws.bucket_cap;
-    if (tid == 0) {
+    if (warp == 0 && lane == 0) {
       ws.prev_count[tile] = c;
       atomicMax(reinterpret_cast<unsigned long long *>(ws.counters + CNT_REQ_LO), (unsigned long long)c * r.T);
       if (ovf) atomicOr(ws.counters + CNT_STATUS, kStatusCapacity);
@@ -265,7 +306,7 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
     }
   } else {
     ovf = pairs_overflow_ws(ws);
-    tile = ovf ? (int)blockIdx.x : (int)ws.tile_order[blockIdx.x];
+    tile = (int)(ovf ? blockIdx.x / kBlocks : ws.tile_order[blockIdx.x / kBlocks]);
   }
   const int tx = tile % r.tiles_x, ty = tile / r.tiles_x;
   const int bx0 = tx * kTile + (warp & 1) * 8, by0 = ty * kTile + (warp >> 1) * 4;
@@ -274,96 +315,139 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
   uint32_t s = 0u, e = 0u;
   if (!ovf) tile_range(ws, tile, s, e);
   const float bcx = (float)bx0 + 3.5f, bcy = (float)by0 + 1.5f;
-  const bool own_sort = sort_tile_bucket(ws, s, (int)(e - s), s_key);
+  const int len = (int)(e - s);
 
   float T = 1.f, cr = 0.f, cg = 0.f, cb = 0.f, dd = 0.f, oo = 0.f, rm = 0.f;
-  float dT[6], jr[6], jg[6], jb[6], jd[6];
+  // tangents of T and of the composited channels, directions in pairs
+  f32x2 dT2[3], jr2[3], jg2[3], jb2[3], jd2[3];
 #pragma unroll
-  for (int k = 0; k < 6; ++k) { dT[k] = 0.f; jr[k] = 0.f; jg[k] = 0.f; jb[k] = 0.f; jd[k] = 0.f; }
+  for (int k = 0; k < 3; ++k) dT2[k] = jr2[k] = jg2[k] = jb2[k] = jd2[k] = 0ull;
+  const f32x2 minus1 = dup2(-1.f);
   int lastk = 0;
   bool done = !inside;
   const float fpx = (float)px, fpy = (float)py;
-  for (uint32_t base = s; base < e; base += kJacBatch) {
-    if (__syncthreads_count(!done) == 0) break;
-    const int cnt = (int)min((uint32_t)kJacBatch, e - base);
-    // thread q stages entry q: its record and its tangent record
-    const int q = tid;
-    if (q < cnt) {
-      const uint32_t k = base + q;
-      uint32_t id = own_sort ? (uint32_t)s_key[k - s] : ws.sorted_ids[k];
-      if (!DAGS_IN_BOUNDS(id < (uint32_t)ws.max_n, ws.counters + CNT_STATUS)) id = 0;
-      const float4 *tg = tan + (size_t)id * kTan4;
-      float4 *st = s_t + q * kTan4;
-      const float4 r3 = ws.rec2d[(size_t)id * 4 + 3];
-      s_a[q] = ws.rec2d[(size_t)id * 4 + 0];
-      s_b[q] = ws.rec2d[(size_t)id * 4 + 1];
-      s_c[q] = ws.rec2d[(size_t)id * 4 + 2];
-      s_e[q] = make_float2(r3.y, r3.z);
-      s_bl[q] = r3.x;
-#pragma unroll
-      for (int w = 0; w < kTan4; ++w) st[w] = tg[w];
+  // The list in groups of 32 entries, in depth order; of a group, the entries
+  // whose box meets the block, in chunks of up to kJacChunk. While a chunk is
+  // worked on, the records and tangents of the next are on their way to shared
+  // memory; the boxes of the next group and the ids of the one after are on
+  // their way to registers.
+  auto load_id = [&](int g) -> uint32_t {
+    const int k = g * 32 + lane;
+    if (k >= len) return 0u;
+    const uint32_t id = __ldg(ws.sorted_ids + s + k);
+    return DAGS_IN_BOUNDS(id < (uint32_t)ws.max_n, ws.counters + CNT_STATUS) ? id : 0u;
+  };
+  auto load_box = [&](uint32_t id) {   // {u, v, ex, ey}
+    const float4 r0 = __ldg(ws.rec2d + (size_t)id * 4), r3 = __ldg(ws.rec2d + (size_t)id * 4 + 3);
+    return make_float4(r0.x, r0.y, r3.y, r3.z);
+  };
+  const int groups = (len + 31) >> 5;
+  int pg = -1;                     // the group being staged
+  unsigned pend = 0u;              // its entries that are still to be staged
+  uint32_t pid = 0u, nid = load_id(0), nnid = load_id(1);
+  float4 nbox = load_box(nid);
+  // stages the next chunk; its entries as bits of group pg (0: the list's end)
+  auto stage = [&](int b) -> unsigned {
+    while (pend == 0u && pg + 1 < groups) {
+      ++pg;
+      pid = nid;
+      const float4 box = nbox;
+      nid = nnid;
+      nnid = load_id(pg + 2);
+      nbox = load_box(nid);
+      pend = __ballot_sync(FULL, pg * 32 + lane < len && fabsf(box.x - bcx) <= box.z + 3.5f &&
+                                     fabsf(box.y - bcy) <= box.w + 1.5f);
     }
-    __syncthreads();
-    if (__all_sync(FULL, done)) continue;
-    for (int g = 0; g < kJacBatch / 32 && g * 32 < cnt; ++g) {
-      const int jj = g * 32 + lane;
-      bool hit = false;
-      if (jj < cnt) {
-        const float4 a = s_a[jj];
-        const float2 ex = s_e[jj];
-        hit = fabsf(a.x - bcx) <= ex.x + 3.5f && fabsf(a.y - bcy) <= ex.y + 1.5f;
-      }
-      unsigned mask = __ballot_sync(FULL, hit);
-      while (mask) {
-        const int j = g * 32 + __ffs(mask) - 1;
-        mask &= mask - 1;
-        if (done) continue;
-        const float4 a = s_a[j], b = s_b[j];
-        const float dx = (a.x - fpx) + a.z, dy = (a.y - fpy) + a.w;
-        const float p = fmaf(b.x * dx, dx, fmaf(b.y * dx, dy, fmaf(b.z * dy, dy, b.w)));
-        if (p < r.log2_alpha_min) continue;
-        const float ag = hw_exp2(p);
-        const bool clamped = ag > r.alpha_max;
-        const float alpha = clamped ? r.alpha_max : ag;
-        const float tt = T * (1.f - alpha);
-        if (tt < r.t_min) { done = true; continue; }
-        const float w = alpha * T;
-        const float4 c = s_c[j];
-        const float cR = c.z, cG = c.w, cB = s_bl[j];
-        cr += cR * w; cg += cG * w; cb += cB * w;
-        dd += c.x * w; oo += w; rm += c.y * w;
-        // tangents: p' = da' dx^2 + db' dx dy + dc' dy^2 + dp/du du + dp/dv dv,
-        // alpha' = alpha ln2 p' (0 where clamped), weight' = alpha' T + alpha T';
-        // the next entry's T = T - weight, so its T' = T' - weight'
-        const float gx = fmaf(2.f * b.x, dx, b.y * dy), gy = fmaf(b.y, dx, 2.f * b.z * dy);
-        const float dx2 = dx * dx, dxy = dx * dy, dy2 = dy * dy;
-        const float aln = clamped ? 0.f : alpha * kLn2;
-        const float4 *t4 = s_t + j * kTan4;
-        float tv[36];
+    const int rank = __popc(pend & ((1u << lane) - 1u));
+    const bool take = ((pend >> lane) & 1u) != 0u && rank < kJacChunk;
+    if (take) {
+      const float4 *rec = ws.rec2d + (size_t)pid * 4, *tg = tan + (size_t)pid * kTan4;
 #pragma unroll
-        for (int q = 0; q < kTan4; ++q) {
-          const float4 v4 = t4[q];
-          tv[4 * q] = v4.x; tv[4 * q + 1] = v4.y; tv[4 * q + 2] = v4.z; tv[4 * q + 3] = v4.w;
-        }
+      for (int w = 0; w < 4; ++w) cp_async16(&s_rec[b][w][rank], rec + w);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
-          const float *t = tv + 6 * k;
-          const float dp = fmaf(t[2], dx2, fmaf(t[3], dxy, fmaf(t[4], dy2, fmaf(gx, t[0], gy * t[1]))));
-          const float da = aln * dp;
-          const float dw = fmaf(da, T, alpha * dT[k]);
-          jr[k] = fmaf(cR, dw, jr[k]);
-          jg[k] = fmaf(cG, dw, jg[k]);
-          jb[k] = fmaf(cB, dw, jb[k]);
-          jd[k] = fmaf(c.x, dw, fmaf(w, t[5], jd[k]));
-          dT[k] -= dw;
-        }
-        T = tt;
-        lastk = (int)(base - s) + j + 1;
-      }
-      if (__all_sync(FULL, done)) break;
+      for (int w = 0; w < kTan4; ++w) cp_async16(&s_rec[b][4 + w][rank], tg + w);
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const unsigned chunk = __ballot_sync(FULL, take);
+    pend ^= chunk;
+    return chunk;
+  };
+  unsigned mask_next = groups > 0 ? stage(0) : 0u;
+  for (int cur = 0; mask_next; cur ^= 1) {
+    unsigned mask = mask_next;
+    const int kbase = pg * 32 + 1;
+    mask_next = stage(cur ^ 1);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp();
+    const float4(*const rec)[kJacChunk] = s_rec[cur];
+    float4 a = rec[0][0], b = rec[1][0];
+    for (int j = 0; mask; ++j) {
+      const int bit = __ffs((int)mask) - 1;
+      mask &= mask - 1;
+      // evaluated by every lane, without branches: a lane that is done, or
+      // whose alpha is below alpha_min, or that would stop here carries zero
+      // weights (x + 0 * c == x), so each pixel's sums are those of the
+      // branching form, operation for operation
+      const float dx = (a.x - fpx) + a.z, dy = (a.y - fpy) + a.w;
+      const float p = fmaf(b.x * dx, dx, fmaf(b.y * dx, dy, fmaf(b.z * dy, dy, b.w)));
+      const bool live = !done && p >= r.log2_alpha_min;
+      const float ag = hw_exp2(p);
+      const bool clamped = ag > r.alpha_max;
+      const float alpha = clamped ? r.alpha_max : ag;
+      const float tt = T * (1.f - alpha);
+      const bool stop = live && tt < r.t_min;
+      const bool contrib = live && !stop;
+      done = done || stop;
+      const float gxs = fmaf(2.f * b.x, dx, b.y * dy), gys = fmaf(b.y, dx, 2.f * b.z * dy);
+      // the next entry's centre and conic (past the chunk's last, stale values
+      // of the staging buffer that nothing uses)
+      a = rec[0][j + 1];
+      b = rec[1][j + 1];
+      if (!__any_sync(FULL, contrib)) continue;
+      const float w = contrib ? alpha * T : 0.f;
+      const float4 c = rec[2][j];
+      const float blue = rec[3][j].x;
+      cr += c.z * w; cg += c.w * w; cb += blue * w;
+      dd += c.x * w; oo += w; rm += c.y * w;
+      // tangents: p' = da' dx^2 + db' dx dy + dc' dy^2 + dp/du du + dp/dv dv,
+      // alpha' = alpha ln2 p' (0 where clamped), weight' = alpha' T + alpha T';
+      // the next entry's T = T - weight, so its T' = T' - weight'
+      const f32x2 gx = dup2(gxs), gy = dup2(gys);
+      const f32x2 pdx = dup2(dx), pdy = dup2(dy);
+      const f32x2 dx2 = mul2(pdx, pdx), dxy = mul2(pdx, pdy), dy2 = mul2(pdy, pdy);
+      const f32x2 aln = dup2(contrib && !clamped ? alpha * kLn2 : 0.f), al2 = dup2(contrib ? alpha : 0.f);
+      const f32x2 T2 = dup2(T), w2 = dup2(w);
+      const f32x2 cz2 = dup2(c.x), cr2 = dup2(c.z), cg2 = dup2(c.w), cb2 = dup2(blue);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const ulonglong2 uv = *reinterpret_cast<const ulonglong2 *>(&rec[4 + 3 * k][j]);
+        const ulonglong2 ab = *reinterpret_cast<const ulonglong2 *>(&rec[5 + 3 * k][j]);
+        const ulonglong2 cz = *reinterpret_cast<const ulonglong2 *>(&rec[6 + 3 * k][j]);
+        const f32x2 dp = fma2(ab.x, dx2, fma2(ab.y, dxy, fma2(cz.x, dy2, fma2(gx, uv.x, mul2(gy, uv.y)))));
+        const f32x2 da = mul2(aln, dp);
+        const f32x2 dw = fma2(da, T2, mul2(al2, dT2[k]));
+        jr2[k] = fma2(cr2, dw, jr2[k]);
+        jg2[k] = fma2(cg2, dw, jg2[k]);
+        jb2[k] = fma2(cb2, dw, jb2[k]);
+        jd2[k] = fma2(cz2, dw, fma2(w2, cz.y, jd2[k]));
+        dT2[k] = fma2(dw, minus1, dT2[k]);
+      }
+      T = contrib ? tt : T;
+      lastk = contrib ? kbase + bit : lastk;
+    }
+    __syncwarp();   // the chunk's buffer is staged again in the next round
+    if (__all_sync(FULL, done)) break;
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");   // no copy outlives the warp
 
+  float jr[6], jg[6], jb[6], jd[6];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    unpack2(jr2[k], jr[2 * k], jr[2 * k + 1]);
+    unpack2(jg2[k], jg[2 * k], jg[2 * k + 1]);
+    unpack2(jb2[k], jb[2 * k], jb[2 * k + 1]);
+    unpack2(jd2[k], jd[2 * k], jd[2 * k + 1]);
+  }
   float acc[kNormal];
 #pragma unroll
   for (int k = 0; k < kNormal; ++k) acc[k] = 0.f;
@@ -410,45 +494,36 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
     }
     if (last) last[pix] = lastk;
   }
-  // tile partials: warp sums, then the 8 warps in a fixed order
-#pragma unroll
-  for (int k = 0; k < kNormal; ++k) {
-    const float v = warp_sum(acc[k]);
-    if (lane == 0) s_red[warp][k] = v;
+  // block sums, the tile's eight in order, a group's tiles and the groups: the
+  // last warp to arrive at each level sums the level below in a fixed order
+  // (FP64 additions run at two per cycle and SM, so they are spread over the
+  // groups' last warps)
+  {
+    const float v = warp_reduce_scatter<kNormal, 16>(acc, lane);
+    const int comp = rs_component<kNormal>(lane);
+    if (__ffs(__match_any_sync(FULL, (unsigned)comp)) - 1 == lane)
+      buf.block_partial[((size_t)tile * kBlocks + warp) * kNormal + comp] = v;
   }
-  __syncthreads();
-  if (tid < kNormal) {
+  if (!arrive_last(buf.done + tile, kBlocks)) return;
+  if (lane < kNormal) {
     float t = 0.f;
 #pragma unroll
-    for (int w = 0; w < kTilePix / 32; ++w) t += s_red[w][tid];
-    // by tile, so that the final sum's order does not depend on the launch order
-    partial[(size_t)tile * kNormal + tid] = t;
+    for (int w = 0; w < kBlocks; ++w) t += __ldcg(buf.block_partial + ((size_t)tile * kBlocks + w) * kNormal + lane);
+    buf.partial[(size_t)tile * kNormal + lane] = t;
   }
-  __syncthreads();
-  if (tid == 0) {
-    // the bucket is empty again for the next iteration's binning (its list
-    // was read before the compositing)
-    if (ws.bucket_cap) ws.tile_count[tile] = 0u;
-    __threadfence();
-    const unsigned int done_ctas = atomicAdd(ws.counters + CNT_DONE_RENDER, 1u);
-    s_last = (done_ctas == gridDim.x - 1);
-    if (s_last) __threadfence();
-  }
-  __syncthreads();
-  if (!s_last) return;
-  // FP64 sum of the tile partials: column c by 8 threads with a fixed stride,
-  // then those 8 in order
-  __shared__ double s_d[kNormal * 8];
-  if (tid < kNormal * 8) {
-    const int c = tid >> 3, part = tid & 7;
-    // four independent accumulators per thread (dependent FP64 additions
-    // are slow on GB300), combined in a fixed order
+  // the bucket is empty again for the next iteration's binning (the tile's
+  // warps have read its range)
+  if (ws.bucket_cap && lane == 0) ws.tile_count[tile] = 0u;
+  const int group = tile / kTileGroup, ngroups = (r.T + kTileGroup - 1) / kTileGroup;
+  const int first = group * kTileGroup, in_group = min(kTileGroup, r.T - first);
+  if (!arrive_last(buf.done + r.T + group, (uint32_t)in_group)) return;
+  if (lane < kNormal) {
     double a4[4] = {0.0, 0.0, 0.0, 0.0};
-    int j = 0;
-    for (int k = part; k < (int)gridDim.x; k += 8, ++j) a4[j & 3] += (double)__ldcg(partial + (size_t)k * kNormal + c);
-    s_d[tid] = (a4[0] + a4[1]) + (a4[2] + a4[3]);
+#pragma unroll 4
+    for (int k = 0; k < in_group; ++k) a4[k & 3] += (double)__ldcg(buf.partial + (size_t)(first + k) * kNormal + lane);
+    buf.group_partial[(size_t)group * kNormal + lane] = (a4[0] + a4[1]) + (a4[2] + a4[3]);
   }
-  __syncthreads();
+  if (!arrive_last(buf.done + r.T + ngroups, (uint32_t)ngroups)) return;
   __shared__ double s_nrm[kNormal];
   // a pair-capacity overflow leaves tiles unrendered (all of them in the
   // general layout; in the bucket layout those whose list exceeded its
@@ -457,36 +532,35 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
   if (ws.bucket_cap)
     any_ovf = __ldcg(reinterpret_cast<const unsigned long long *>(ws.counters + CNT_REQ_LO)) >
               (unsigned long long)ws.bucket_cap * (unsigned long long)r.T;
-  if (tid < kNormal) {
-    double t = 0.0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) t += s_d[tid * 8 + k];
+  if (lane < kNormal) {
+    double a4[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+    for (int k = 0; k < ngroups; ++k) a4[k & 3] += __ldcg(buf.group_partial + (size_t)k * kNormal + lane);
+    double t = (a4[0] + a4[1]) + (a4[2] + a4[3]);
     // then the loss is NaN, so the LM step rejects this point
-    if (any_ovf && tid == 0) t = __longlong_as_double(0x7ff8000000000000ll);
-    normal[tid] = t;
-    s_nrm[tid] = t;
+    if (any_ovf && lane == 0) t = __longlong_as_double(0x7ff8000000000000ll);
+    normal[lane] = t;
+    s_nrm[lane] = t;
   }
-  if (tid == 0) ws.counters[CNT_DONE_RENDER] = 0u;
-  __syncthreads();
-  // inside the LM loop the step runs here, in the last CTA
+  __syncwarp();
+  // inside the LM loop the step runs here, in the last warp
   if (fuse.state) {
-    lm_step_cta(s_nrm, fuse.state, fuse.pose_try, fuse.pose_best, fuse.cfg);
+    lm_step_warp(s_nrm, fuse.state, fuse.pose_try, fuse.pose_best, fuse.cfg);
     // the bucket layout: if the next linearisation point (as the preprocess
     // stages it in FP32) has left the bounds the candidates were culled for,
     // move the culling pose to it and empty the list; the next preprocess
     // then takes every Gaussian once and re-culls
     if (ws.bucket_cap && ws.cand_n && ws.cull_pose) {
       __shared__ float s_np[12];
-      __shared__ int s_out;
-      __syncthreads();
-      if (tid < 12) s_np[tid] = __double2float_rn(fuse.pose_try[tid]);
-      __syncthreads();
-      if (tid == 0) s_out = within_cull_bounds(s_np, ws.cull_pose) ? 0 : 1;
-      __syncthreads();
-      if (s_out && tid < 12) ws.cull_pose[tid] = s_np[tid];
-      if (tid == 0) {
-        if (s_out) *ws.cand_n = 0u;
-        ws.counters[CNT_RECULL] = s_out ? 1u : 0u;
+      __syncwarp();
+      if (lane < 12) s_np[lane] = __double2float_rn(fuse.pose_try[lane]);
+      __syncwarp();
+      const bool out = !within_cull_bounds(s_np, ws.cull_pose);
+      __syncwarp();
+      if (out && lane < 12) ws.cull_pose[lane] = s_np[lane];
+      if (lane == 0) {
+        if (out) *ws.cand_n = 0u;
+        ws.counters[CNT_RECULL] = out ? 1u : 0u;
       }
     }
   }
@@ -511,7 +585,7 @@ __global__ void lm_init_kernel(const double *__restrict__ pose, double *__restri
 __global__ void lm_step_kernel(const double *__restrict__ normal, double *__restrict__ state,
                                double *__restrict__ pose_try, double *__restrict__ pose_best, dags_lm_cfg c) {
   pdl_wait();
-  lm_step_cta(normal, state, pose_try, pose_best, c);
+  lm_step_warp(normal, state, pose_try, pose_best, c);
 }
 
 }  // namespace
@@ -519,25 +593,19 @@ __global__ void lm_step_kernel(const double *__restrict__ normal, double *__rest
 cudaError_t launch_pose_tangents(const Workspace &ws, const float4 *gauss, int64_t n, const Raster &r, float4 *tan,
                                  int num_sms, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  const int64_t need = (n + kPrepBlock - 1) / kPrepBlock;
-  const unsigned grid = (unsigned)(need < (int64_t)num_sms * 8 ? need : (int64_t)num_sms * 8);
-  // (plus the ranking CTA of the tracking loop)
-  return launch_pdl(pose_tangent_kernel, dim3(grid + (ws.order_next ? 1u : 0u)), dim3(kPrepBlock), 0, s, ws, gauss,
-                    n, r, tan);
-}
-
-// The Jacobian render's dynamic shared memory (the batch's tangent records)
-// exceeds the default 48 KB: raised once per device, at the ctx's first LM
-// call (before any stream capture).
-cudaError_t lm_kernel_setup() {
-  return cudaFuncSetAttribute(render_jac_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kJacTanBytes);
+  const int64_t need = (n + kTanBlock - 1) / kTanBlock;
+  const unsigned grid = (unsigned)(need < (int64_t)num_sms * 3 ? need : (int64_t)num_sms * 3);
+  // the visible Gaussians' CTAs, the tiles' and, in the tracking loop, the
+  // ranking one
+  return launch_pdl(pose_tangent_kernel, dim3(grid + (unsigned)r.T + (ws.order_next ? 1u : 0u)), dim3(kTanBlock), 0, s,
+                    ws, gauss, n, r, tan);
 }
 
 cudaError_t launch_render_jac(const Workspace &ws, const Raster &r, const Loss &l, float delta,
-                              const float4 *targets, const float4 *tan, float *partial, double *normal, float *jac,
-                              float *image, int32_t *last, const LmFuse &fuse, cudaStream_t s) {
-  return launch_pdl(render_jac_kernel, dim3((unsigned)r.T), dim3(kTilePix), kJacTanBytes, s, ws, r, l, delta, targets, tan,
-                    partial, normal, jac, image, last, fuse);
+                              const float4 *targets, const LmBuffers &buf, double *normal, float *jac, float *image,
+                              int32_t *last, const LmFuse &fuse, cudaStream_t s) {
+  return launch_pdl(render_jac_kernel, dim3((unsigned)r.T * kBlocks), dim3(32), 0, s, ws, r, l, delta, targets,
+                    (const float4 *)buf.tan, buf, normal, jac, image, last, fuse);
 }
 
 cudaError_t launch_lm_init(const double *pose, double *state, double *pose_try, double mu0, cudaStream_t s) {
@@ -546,7 +614,7 @@ cudaError_t launch_lm_init(const double *pose, double *state, double *pose_try, 
 
 cudaError_t launch_lm_step(const double *normal, double *state, double *pose_try, double *pose_best,
                            const dags_lm_cfg &c, cudaStream_t s) {
-  return launch_pdl(lm_step_kernel, dim3(1), dim3(64), 0, s, normal, state, pose_try, pose_best, c);
+  return launch_pdl(lm_step_kernel, dim3(1), dim3(32), 0, s, normal, state, pose_try, pose_best, c);
 }
 
 }  // namespace dags
