@@ -149,7 +149,7 @@ void free_epi(EpiBuffers &b) {
 }
 
 void free_net(MpnetScratch &b) {
-  void *ptrs[] = {b.y, b.acts, b.dz2, b.grad, b.inv_n};
+  void *ptrs[] = {b.y, b.acts, b.a1, b.dz2, b.zero, b.grad, b.inv_n};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   b = MpnetScratch();
@@ -1269,7 +1269,7 @@ int mpnet_infer(dags_ctx *ctx, const void *weights, const uint16_t *feats, int32
   cudaStream_t s = (cudaStream_t)stream;
   ctx->last_stream = s;
   const int ev = ctx->timer.begin(DAGS_K_MPNET, s);
-  const cudaError_t e = launch_mpnet_forward(weights, feats, batch, width, height, mp_out, acts,
+  const cudaError_t e = launch_mpnet_forward(weights, feats, batch, width, height, mp_out, acts, nullptr,
                                              ctx->ws.counters + CNT_STATUS, ctx->num_sms, s);
   ctx->timer.end(ev, s);
   return cuda_status(e);
@@ -1286,13 +1286,19 @@ int mpnet_train_step(dags_ctx *ctx, void *weights, float *master, float *adam_m,
   cudaStream_t s = (cudaStream_t)stream;
   ctx->last_stream = s;
   MpnetScratch &sc = ctx->net;
-  if (sc.cap < npix) {
+  const long long planes = mpnet_plane_size(batch, width, height);
+  if (sc.cap < npix || sc.plane_cap < planes) {
     cudaError_t e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_status(e);
+    const long long cap = std::max(sc.cap, npix), plane_cap = std::max(sc.plane_cap, planes);
     free_net(sc);
-    e = alloc(&sc.y, (size_t)npix);
-    if (e == cudaSuccess) e = alloc(&sc.acts, (size_t)npix * DAGS_MPNET_ACT_WORDS);
-    if (e == cudaSuccess) e = alloc(&sc.dz2, (size_t)npix * 32);
+    e = alloc(&sc.y, (size_t)cap);
+    if (e == cudaSuccess) e = alloc(&sc.acts, (size_t)cap * DAGS_MPNET_ACT_WORDS);
+    if (e == cudaSuccess) e = alloc(&sc.a1, (size_t)plane_cap);
+    if (e == cudaSuccess) e = alloc(&sc.dz2, (size_t)plane_cap);
+    if (e == cudaSuccess) e = alloc(&sc.zero, kMpnetStrip + 2);
+    if (e == cudaSuccess) e = cudaMemsetAsync(sc.zero, 0, (kMpnetStrip + 2) * sizeof(uint4), s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // whatever stream the next step runs on
     if (e == cudaSuccess) e = alloc(&sc.grad, DAGS_MPNET_PARAMS);
     if (e == cudaSuccess) e = alloc(&sc.inv_n, 2);
     if (e != cudaSuccess) {
@@ -1300,7 +1306,8 @@ int mpnet_train_step(dags_ctx *ctx, void *weights, float *master, float *adam_m,
       cudaGetLastError();
       return DAGS_E_NOMEM;
     }
-    sc.cap = npix;
+    sc.cap = cap;
+    sc.plane_cap = plane_cap;
   }
   const int ev = ctx->timer.begin(DAGS_K_MPNET_TRAIN, s);
   cudaError_t e = launch_mpnet_train(weights, master, adam_m, adam_v, step, feats, target, batch, width, height, lr,

@@ -15,7 +15,7 @@
 // mpnet_bwd1_kernel  training: BCE gradient, dz3, da2 = dz3 W3 and dz2; the
 //                    weight gradients dW3, dw4 accumulated in TMEM.
 // mpnet_bwd2_kernel  training: da1 by the transposed 3x3 convolution, dz1;
-//                    dW2 per tap and dW1 accumulated in TMEM.
+//                    dW2 per column tap and dW1 accumulated in TMEM.
 // mpnet_adam_kernel  Adam on the FP32 master weights, BF16 blob refresh.
 //
 // Weights are staged once per CTA in the canonical no-swizzle K-major
@@ -35,7 +35,6 @@ namespace {
 constexpr int kNetThreads = 128;          // 4 warps = one warpgroup over the 128 TMEM lanes
 constexpr int kTileW = 128;               // pixels per tile (MMA M)
 constexpr int kHaloW = kTileW + 2;        // 130
-constexpr int kHaloRows = 3 * kHaloW;     // 390
 constexpr int kCh = 32;
 constexpr int kK2 = 9 * kCh;              // 288
 constexpr long long kSpinLimit = 1ll << 22;
@@ -239,7 +238,7 @@ struct FwdUnits {
 __global__ void __launch_bounds__(kFwdThreads, 1)
 mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__restrict__ weights, int batch, int W,
                  int H, FwdUnits units, float *__restrict__ out, uint16_t *__restrict__ acts,
-                 uint32_t *__restrict__ status) {
+                 uint4 *__restrict__ a1p, uint32_t *__restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint8_t *sW1 = smem + kFW1, *sW2 = smem + kFW2, *sW3 = smem + kFW3, *sB2 = smem + kFB2;
@@ -445,6 +444,7 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
     // ---------------------------------------------------------- epilogues
     const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
     const int p = 32 * warp + lane;
+    const size_t plane_w = (size_t)units.tiles_x * kTileW + 2;
     bool ok = true;
     for (long long u = (long long)kGroups * blockIdx.x + g; u < units.count && ok; u += stride) {
       int b, x0, y0, y1;
@@ -476,7 +476,13 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
             for (int c = 0; c < 4; ++c)
               *reinterpret_cast<uint4 *>(a1 + c * kSlotChunk + i * 16) =
                   make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
-            if (acts && own_row && i >= 1 && xx < W) {
+            if (a1p && own_row && (i >= 1 || x0 == 0)) {
+              // planar copy: plane pixel x + 1, zero outside the image
+              uint4 *ga = a1p + ((size_t)b * H + r) * 4 * plane_w + x0 + i;
+#pragma unroll
+              for (int c = 0; c < 4; ++c)
+                ga[c * plane_w] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+            } else if (acts && !a1p && own_row && i >= 1 && xx < W) {
               uint4 *ga = reinterpret_cast<uint4 *>(acts + (((size_t)b * H + r) * W + xx) * 96);
 #pragma unroll
               for (int c = 0; c < 4; ++c) ga[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
@@ -500,7 +506,10 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
             zc = (zc + sb1h[c]) + sb1l[c];
             const uint16_t a = in ? bf16_bits(fmaxf(zc, 0.f)) : (uint16_t)0;
             *reinterpret_cast<uint16_t *>(a1 + (c >> 3) * kSlotChunk + i * 16 + (c & 7) * 2) = a;
-            if (acts && own_row && i <= kTileW && xx < W) acts[(((size_t)b * H + r) * W + xx) * 96 + c] = a;
+            if (a1p && own_row && (i <= kTileW || x0 + kHaloW == (int)plane_w))
+              reinterpret_cast<uint16_t *>(a1p + (((size_t)b * H + r) * 4 + (c >> 3)) * plane_w + x0 + i)[c & 7] = a;
+            else if (acts && !a1p && own_row && i <= kTileW && xx < W)
+              acts[(((size_t)b * H + r) * W + xx) * 96 + c] = a;
           }
           fence_async_smem();
         }
@@ -661,7 +670,7 @@ __device__ __forceinline__ void st_chunks(uint8_t *base, int stride, int row, co
 __global__ void __launch_bounds__(kNetThreads)
 mpnet_bwd1_kernel(const uint8_t *__restrict__ weights, const float *__restrict__ y, const float *__restrict__ target,
                   const uint16_t *__restrict__ acts, int batch, int W, int H, const float *__restrict__ inv_n,
-                  uint16_t *__restrict__ dz2_out, float *__restrict__ grad, double *__restrict__ loss,
+                  uint4 *__restrict__ dz2p, float *__restrict__ grad, double *__restrict__ loss,
                   uint32_t *__restrict__ status) {
   extern __shared__ __align__(128) uint8_t smem[];
   uint8_t *sA2 = smem + kB1A2, *sA3 = smem + kB1A3, *sDz3 = smem + kB1Dz3, *sDz4 = smem + kB1Dz4;
@@ -698,6 +707,7 @@ mpnet_bwd1_kernel(const uint8_t *__restrict__ weights, const float *__restrict__
   float lsum = 0.f;
   const float invn = inv_n[0];
   const int tiles_x = (W + kTileW - 1) / kTileW;
+  const size_t plane_w = (size_t)tiles_x * kTileW + 2;
   const long long ntiles = (long long)batch * H * tiles_x;
   for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
     const int tx = (int)(t % tiles_x), yy = (int)((t / tiles_x) % H), b = (int)(t / ((long long)tiles_x * H));
@@ -762,16 +772,20 @@ mpnet_bwd1_kernel(const uint8_t *__restrict__ weights, const float *__restrict__
     {
       float da[32];
       tmem_ld32(tmem + lane_base + 0, da);
-      if (in) {
-        uint32_t w[16];
+      uint32_t w[16];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-          const float a2lo = __uint_as_float(a2w[k] << 16), a2hi = __uint_as_float(a2w[k] & 0xFFFF0000u);
-          w[k] = pack_bf16x2(a2lo > 0.f ? da[2 * k] : 0.f, a2hi > 0.f ? da[2 * k + 1] : 0.f);
-        }
-        uint4 *dst = reinterpret_cast<uint4 *>(dz2_out + pix * 32);
+      for (int k = 0; k < 16; ++k) {   // a2 = 0 outside the image
+        const float a2lo = __uint_as_float(a2w[k] << 16), a2hi = __uint_as_float(a2w[k] & 0xFFFF0000u);
+        w[k] = pack_bf16x2(a2lo > 0.f ? da[2 * k] : 0.f, a2hi > 0.f ? da[2 * k + 1] : 0.f);
+      }
+      uint4 *dst = dz2p + ((size_t)b * H + yy) * 4 * plane_w + x + 1;
+      const bool right = x + 3 == (int)plane_w;
 #pragma unroll
-        for (int g = 0; g < 4; ++g) dst[g] = make_uint4(w[4 * g], w[4 * g + 1], w[4 * g + 2], w[4 * g + 3]);
+      for (int g = 0; g < 4; ++g) {
+        uint4 *d = dst + g * plane_w;
+        *d = make_uint4(w[4 * g], w[4 * g + 1], w[4 * g + 2], w[4 * g + 3]);
+        if (x == 0) d[-1] = make_uint4(0u, 0u, 0u, 0u);
+        if (right) d[1] = make_uint4(0u, 0u, 0u, 0u);
       }
     }
     tc_before_sync();
@@ -805,49 +819,95 @@ mpnet_bwd1_kernel(const uint8_t *__restrict__ weights, const float *__restrict__
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128));
 }
 
-// bwd2 shared memory: two sets (double buffering) of the dz2 and a1 halos
-// (3 rows x 130 pixels; a1 with its ones chunk 4) and of x (chunk 0, ones
-// chunk 1), then dz1 and W2 rearranged as B[i][(tap, o)]. The M = 128
-// MN-major reads of a1 and x run past their real chunks into what follows
-// (in bounds, finite).
-constexpr int kHaloChunk = 392 * 16;                     // 6272
-constexpr int kB2SetA1 = 0, kB2SetDz2 = 5 * kHaloChunk, kB2SetBytes = 9 * kHaloChunk;   // 56448
-constexpr int kB2X = 2 * kB2SetBytes;                    // 2 x (x chunk, ones chunk)
-constexpr int kB2Dz1 = kB2X + 4 * kChunkPx;              // dz1: 4 chunks
-constexpr int kB2W2t = kB2Dz1 + 4 * kChunkPx;            // [32 i][288 (tap, o)]
-constexpr int kB2Bar = kB2W2t + 32 * kK2 * 2;
-constexpr int kB2End = kB2Bar + 64;
-constexpr int kB2Span = kB2SetBytes + 16 * kHaloChunk;   // the farthest MN-major read of a1 (set 1)
-constexpr int kB2Smem = (kB2Span > kB2End ? kB2Span : kB2End);
-static_assert(kB2X + 2 * kChunkPx + 16 * kChunkPx <= kB2Smem, "MN-major reads of x stay in shared memory");
+// bwd2: da1 by the transposed 3 x 3 convolution, dz1, and the weight gradients
+// dW2, dW1, db2, db1. A CTA walks its share of the 128-pixel column strips
+// downwards, two output rows (a pair) per step; the rows of a1, dz2 and x come
+// once from the planar copies by bulk copies, each row 2,080 contiguous bytes
+// per 8-channel chunk.
+//
+// Warps 0..3 form dz1 from da1, warp 4 issues the copies, warp 5 the MMAs of
+// da1 and dW1, warps 6..8 those of dW2 (a column tap each) and db2: one
+// thread's MMAs go through at most one per 68 cycles. An MMA costs its operands'
+// shared-memory reads (about 128 B per cycle), so the products are stacked:
+//   dW2, db2: per dz2 row y, column tap kx and 16 pixels one M = 128, N = 32
+//     product of the a1 rows y - 1 .. y + 1 (slots of four chunks and one of
+//     (1, 0, ...) at one stride: 120 rows, the kernel rows and the bias; the
+//     last 8 are whatever follows, their D rows unused): 24 MMAs of about 40
+//     cycles a row instead of 72 of 25 (M = 64, one tap each). N = 64 over two dz2 rows would take
+//     24 of 48 for both, but halves the additions of an accumulator, and with
+//     them the tensor core's truncation (-7.6e-5 relative on dW2 at 16 x 640
+//     x 480): results would differ by that.
+//   da1: N = 64 over both output rows for the dz2 rows y, y + 1, N = 32 for
+//     y - 1 and y + 2; the kernel rows of W2 are stacked along N, so that a
+//     window of them meets the output rows.
+//   dW1, db1: per row dz1 (M = 64, 32 rows used) against x and the ones
+//     (N = 16).
+// About 1,650 tensor cycles per 128-pixel row. 16 x 640 x 480, the launch
+// alone: 976 us with one CTA of 128 threads that fetched three halo rows per
+// output row and waited for each tile's chain, 315 us now (418,000 tensor
+// cycles a CTA, 0.21 ms at 2 GHz, are what bounds it).
+//
+// Rings. Groups g (pairs, and the half pair above and below a segment): dz2
+// of two rows and x, four slots. a1 rows: eight slots; step c (pairs only)
+// reads the window of four slots at 2 (c mod 3), so a row that two windows
+// share is copied again only where the ring wraps (8 copies per 6 rows).
+// Barriers: full_d[4] dz2 and x of a group, full_a[3] the a1 rows of a step,
+// done_d[4] / done_w[4] the group's last use by warp 5 / warps 6..8, done_c[3] step c's
+// dW2, prod[2] da1 of a step, ep[2] its dz1 (and its reads of a1), drain[4].
+constexpr int kB2Threads = 9 * 32;
+constexpr int kB2Slot = 4 * kRowBytes;                   // one row: four chunks of 130 pixels
+constexpr int kB2A1Slot = 5 * kRowBytes;                 // an a1 row and a chunk of ones
+constexpr int kB2A1 = 0;                                 // eight a1 rows
+constexpr int kB2Dz2 = 8 * kB2A1Slot;                    // four groups of two dz2 rows
+constexpr int kB2Dz1 = kB2Dz2 + 8 * kB2Slot;             // two steps of two dz1 rows (128-pixel chunks)
+constexpr int kB2X = kB2Dz1 + 2 * 8 * kChunkPx;          // four groups of x, x, ones
+constexpr int kB2W2 = kB2X + 4 * 3 * kChunkPx;           // [(ky, i)][(kx, o)]
+constexpr int kB2Bar = kB2W2 + 96 * 96 * 2;
+constexpr int kB2NBars = 4 + 3 + 4 + 4 + 3 + 2 + 2 + 4;
+constexpr int kB2Smem = kB2Bar + 8 * kB2NBars + 16;
+constexpr uint32_t kB2ColW2 = 0, kB2ColDa = 128, kB2ColW1 = 256;
+static_assert(kB2Smem <= 227 * 1024, "shared memory");
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool valid) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_t bytes, uint64_t *bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
 }
 
-__global__ void __launch_bounds__(kNetThreads, 1)
-mpnet_bwd2_kernel(const uint8_t *__restrict__ weights, const uint4 *__restrict__ feats, const uint16_t *__restrict__ acts,
-                  const uint16_t *__restrict__ dz2, int batch, int W, int H, float *__restrict__ grad,
-                  uint32_t *__restrict__ status) {
+__global__ void __launch_bounds__(kB2Threads, 1)
+mpnet_bwd2_kernel(const uint8_t *__restrict__ weights, const uint4 *__restrict__ feats, const uint4 *__restrict__ a1p,
+                  const uint4 *__restrict__ dz2p, const uint4 *__restrict__ zero, int W, int H, int tiles_x,
+                  long long npairs, float *__restrict__ grad, uint32_t *__restrict__ status) {
   extern __shared__ __align__(128) uint8_t smem[];
-  uint8_t *sDz1 = smem + kB2Dz1, *sW2t = smem + kB2W2t;
-  uint64_t *bar = reinterpret_cast<uint64_t *>(smem + kB2Bar);
-  uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + kB2Bar + 8);
-  const int tid = threadIdx.x, warp = tid >> 5;
-  for (int e = tid; e < kB2Smem / 16; e += kNetThreads) reinterpret_cast<uint4 *>(smem)[e] = make_uint4(0u, 0u, 0u, 0u);
+  uint64_t *full_d = reinterpret_cast<uint64_t *>(smem + kB2Bar), *full_a = full_d + 4, *done_d = full_a + 3,
+           *done_w = done_d + 4, *done_c = done_w + 4, *prod = done_c + 3, *ep = prod + 2, *drain = ep + 2;
+  uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + kB2Bar + 8 * kB2NBars);
+  volatile uint32_t *s_fail = reinterpret_cast<volatile uint32_t *>(s_tmem + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t base = smem_u32(smem);
+  for (int e = tid; e < kB2W2 / 16; e += kB2Threads) reinterpret_cast<uint4 *>(smem)[e] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
   const uint16_t *gw2 = reinterpret_cast<const uint16_t *>(weights + kOffW2);
-  for (int e = tid; e < 32 * kK2; e += kNetThreads) {
-    const int o = e / kK2, col = e % kK2, tap = col / 32, i = col % 32;
-    *reinterpret_cast<uint16_t *>(sW2t + core_off(i, tap * 32 + o, kK2)) = gw2[e];
+  for (int e = tid; e < 32 * kK2; e += kB2Threads) {
+    const int o = e / kK2, col = e % kK2, tap = col / 32, i = col % 32, ky = tap / 3, kx = tap % 3;
+    *reinterpret_cast<uint16_t *>(smem + kB2W2 + core_off(ky * 32 + i, kx * 32 + o, 96)) = gw2[e];
   }
-  for (int set = 0; set < 2; ++set) {
-    for (int h = tid; h < 392; h += kNetThreads)
-      *reinterpret_cast<uint4 *>(smem + set * kB2SetBytes + kB2SetA1 + 4 * kHaloChunk + h * 16) =
-          make_uint4(0x3F80u, 0u, 0u, 0u);
-    *reinterpret_cast<uint4 *>(smem + kB2X + set * 2 * kChunkPx + kChunkPx + tid * 16) = make_uint4(0x3F80u, 0u, 0u, 0u);
+  for (int e = tid; e < 4 * kTileW; e += kB2Threads)
+    *reinterpret_cast<uint4 *>(smem + kB2X + (e / kTileW) * 3 * kChunkPx + 2 * kChunkPx + (e % kTileW) * 16) =
+        make_uint4(0x3F80u, 0u, 0u, 0u);
+  for (int e = tid; e < 8 * kHaloW; e += kB2Threads)
+    *reinterpret_cast<uint4 *>(smem + kB2A1 + (e / kHaloW) * kB2A1Slot + kB2Slot + (e % kHaloW) * 16) =
+        make_uint4(0x3F80u, 0u, 0u, 0u);
+  if (tid == 0) {
+    for (int k = 0; k < kB2NBars; ++k) {
+      uint64_t *bar = full_d + k;   // ep: the four warps; done_w, done_c: the three warps of dW2
+      const int count = bar >= ep && bar < drain ? 4 : bar >= done_w && bar < prod ? 3 : 1;
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    *s_fail = 0u;
   }
-  if (tid == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)));
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -856,140 +916,249 @@ mpnet_bwd2_kernel(const uint8_t *__restrict__ weights, const uint4 *__restrict__
   tc_before_sync();
   __syncthreads();
   tc_after_sync();
-  // D: da1 cols 0-31; dW2^T of tap t cols 32 + 32 t (t = 0..8, to 319); dW1^T cols 320-351
   const uint32_t tmem = *s_tmem;
-  const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
-  uint32_t phase = 0;
-  bool ok = true, first = true;
-  const int tiles_x = (W + kTileW - 1) / kTileW;
-  const long long ntiles = (long long)batch * H * tiles_x;
-  // asynchronous copies of tile T's halos and x into buffer set `set`
-  // (zero-filled outside the image)
-  auto fetch = [&](long long T, int set) {
-    const int tx = (int)(T % tiles_x), y = (int)((T / tiles_x) % H), b = (int)(T / ((long long)tiles_x * H));
-    const int x0 = tx * kTileW;
-    const uint32_t base = smem_u32(smem) + set * kB2SetBytes;
-    for (int h = tid; h < kHaloRows; h += kNetThreads) {
-      const int r = h / kHaloW, c = h % kHaloW, yy = y - 1 + r, xx = x0 - 1 + c;
-      const bool v = yy >= 0 && yy < H && xx >= 0 && xx < W;
-      const size_t q = v ? ((size_t)b * H + yy) * W + xx : 0;
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        cp_async16(base + kB2SetDz2 + g * kHaloChunk + h * 16, dz2 + q * 32 + 8 * g, v);
-        cp_async16(base + kB2SetA1 + g * kHaloChunk + h * 16, acts + q * 96 + 8 * g, v);
+  const int HP = (H + 1) / 2;
+  const size_t plane_w = (size_t)tiles_x * kTileW + 2;
+  const long long first = npairs * blockIdx.x / gridDim.x, last = npairs * (blockIdx.x + 1) / gridDim.x;
+  // the next segment of the CTA's pairs: n pairs of one strip, the first one
+  // at row y0 of image b
+  auto segment = [&](long long q, int *b, int *x0, int *y0) {
+    const long long strip = q / HP;
+    const int pr = (int)(q - strip * HP);
+    *b = (int)(strip / tiles_x);
+    *x0 = (int)(strip - (long long)*b * tiles_x) * kTileW;
+    *y0 = 2 * pr;
+    const long long left = last - q;
+    return left < HP - pr ? (int)left : HP - pr;
+  };
+  bool ok = true;
+  int g = 0, c = 0;      // groups and steps so far (the same sequence in every role)
+  auto fail = [&] { *s_fail = 1u; };
+  if (warp == 4) {
+    // ------------------------------------------------------------- copies
+    int last_d[4] = {-1, -1, -1, -1}, last_a[3] = {-1, -1, -1};
+    for (long long q = first; q < last && ok;) {
+      int b, x0, y0;
+      const int n = segment(q, &b, &x0, &y0);
+      q += n;
+      const size_t img = (size_t)b * H;
+      const uint32_t xbytes = 16u * (uint32_t)min(kTileW, W - x0);
+      auto row_src = [&](const uint4 *plane, int y, int ch) {
+        return y >= 0 && y < H ? plane + ((img + y) * 4 + ch) * plane_w + x0 : zero;
+      };
+      for (int P = -1; P <= n; ++P, ++g) {
+        const int slot = g & 3, row0 = y0 + 2 * P;
+        if (g >= 4) ok = bar_wait(done_d + slot, (uint32_t)((g >> 2) - 1) & 1u) &&
+                         bar_wait(done_w + slot, (uint32_t)((g >> 2) - 1) & 1u);
+        ok = __all_sync(0xffffffffu, ok && !*s_fail);
+        if (!ok) break;
+        const bool r0 = P >= 0, r1 = P < n, mid = r0 && r1;
+        const int xrows = mid ? min(2, H - row0) : 0;
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(full_d + slot)),
+                       "r"((uint32_t)(r0 + r1) * kB2Slot + (uint32_t)xrows * xbytes)
+                       : "memory");
+        __syncwarp();
+        const uint32_t dz = base + kB2Dz2 + 2 * slot * kB2Slot;
+        if (lane < 8) {
+          const int rr = lane >> 2, ch = lane & 3;
+          if (rr ? r1 : r0)
+            bulk_copy(dz + rr * kB2Slot + ch * kRowBytes, row_src(dz2p, row0 + rr, ch), kRowBytes, full_d + slot);
+        } else if (lane < 8 + xrows) {
+          const int rr = lane - 8;
+          bulk_copy(base + kB2X + (3 * slot + rr) * kChunkPx, feats + (img + row0 + rr) * W + x0, xbytes,
+                    full_d + slot);
+        }
+        last_d[slot] = g;
+        if (P < 1) continue;
+        // the a1 rows of step c, the pair at row0 - 2
+        const int dep = P == 1 ? c - 1 : c - 2, w = c % 3;
+        if (dep >= 0) ok = bar_wait(done_c + dep % 3, (uint32_t)(dep / 3) & 1u) &&
+                           bar_wait(ep + (dep & 1), (uint32_t)(dep >> 1) & 1u);
+        ok = __all_sync(0xffffffffu, ok && !*s_fail);
+        if (!ok) break;
+        const int from = P == 1 || w == 0 ? 0 : 2;      // the first of the window's rows that is copied
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(full_a + w)),
+                       "r"((uint32_t)(4 - from) * kB2Slot)
+                       : "memory");
+        __syncwarp();
+        if (lane < 16 && (lane >> 2) >= from) {
+          const int k = lane >> 2, ch = lane & 3;
+          bulk_copy(base + kB2A1 + (2 * w + k) * kB2A1Slot + ch * kRowBytes, row_src(a1p, row0 - 3 + k, ch), kRowBytes,
+                    full_a + w);
+        }
+        last_a[w] = c;
+        ++c;
       }
     }
-    const int x = x0 + tid;
-    cp_async16(smem_u32(smem) + kB2X + set * 2 * kChunkPx + tid * 16, feats + (x < W ? ((size_t)b * H + y) * W + x : 0),
-               x < W);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  // Per tile: da1 (18 MMAs) is committed on its own and the dW2 MMAs (72)
-  // queue behind it, so the dz1 epilogue runs while the tensor core
-  // accumulates dW2; dW1 (8 MMAs) follows the epilogue. The next tile's da1
-  // commit covers all of them (one thread's MMAs complete in order), so its
-  // wait also frees this tile's buffers for the prefetch two tiles ahead.
-  long long t = blockIdx.x;
-  if (t < ntiles) fetch(t, 0);
-  bool pending = false;   // MMAs issued and not yet covered by a completed wait
-  for (int it = 0; t < ntiles && ok; t += gridDim.x, ++it) {
-    const int set = it & 1, p = tid;
-    uint8_t *sA1 = smem + set * kB2SetBytes + kB2SetA1, *sDz2 = smem + set * kB2SetBytes + kB2SetDz2;
-    uint8_t *sX = smem + kB2X + set * 2 * kChunkPx;
-    // 1. this tile's halos and x have landed
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    fence_async_smem();
-    tc_before_sync();
-    __syncthreads();
-    tc_after_sync();
-    // 2. da1: the transposed 3 x 3 convolution as an implicit GEMM - tap
-    //    (ky, kx) reads dz2 at halo row (2 - ky) * 130 + (2 - kx) + q; then
-    //    dW2^T per tap: a1 at halo row ky * 130 + kx + q against dz2 of the
-    //    centre row (halo row 131 + q), MN-major over the tile's pixels
-    if (tid == 0) {
-      for (int tap = 0; tap < 9; ++tap) {
-        const int ky = tap / 3, kx = tap % 3;
-        for (int j = 0; j < 2; ++j)
-          mma_bf16(tmem + 0, sdesc(smem_u32(sDz2) + 2 * j * kHaloChunk + ((2 - ky) * kHaloW + (2 - kx)) * 16, kHaloChunk, 128),
-                   sdesc(smem_u32(sW2t) + (2 * tap + j) * 256, 128, (kK2 / 8) * 128), idesc_bf16(128, 32),
-                   (tap | j) ? 1u : 0u);
-      }
-      mma_commit(bar);
-      for (int s2 = 0; s2 < kTileW / 16; ++s2) {
-        const uint32_t acc = (!first || s2 > 0) ? 1u : 0u;
-        const uint32_t bdz2 = smem_u32(sDz2) + (kHaloW + 1) * 16 + s2 * 256;
-        for (int tap = 0; tap < 9; ++tap) {
-          const int ky = tap / 3, kx = tap % 3;
-          mma_bf16(tmem + 32 + 32 * tap, sdesc(smem_u32(sA1) + (ky * kHaloW + kx) * 16 + s2 * 256, 128, kHaloChunk),
-                   sdesc(bdz2, 128, kHaloChunk), idesc_bf16_mn(64, 32), acc);
+    if (!ok) fail();
+    // no copy outlives the CTA
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (last_d[k] >= 0) bar_wait(full_d + k, (uint32_t)(last_d[k] >> 2) & 1u);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (last_a[k] >= 0) bar_wait(full_a + k, (uint32_t)(last_a[k] / 3) & 1u);
+  } else if (warp == 5) {
+    // ---------------------------------------------------------- da1 and dW1
+    if (lane == 0) {
+      int have = 0;           // groups whose copies have been waited for
+      bool before = false;    // the previous group was a pair
+      for (long long q = first; q < last && ok;) {
+        int b, x0, y0;
+        const int n = segment(q, &b, &x0, &y0);
+        q += n;
+        for (int P = -1; P <= n && ok; ++P, ++g) {
+          const bool mid = P >= 0 && P < n;
+          for (const int need = mid ? g + 2 : g + 1; have < need && ok; ++have)
+            ok = bar_wait(full_d + (have & 3), (uint32_t)(have >> 2) & 1u);
+          if (*s_fail) ok = false;
+          if (!ok) break;
+          if (mid) {
+            const uint32_t d = tmem + kB2ColDa + 64u * (uint32_t)(c & 1);
+            // dz2 row y0' + k (k = -1..2); pixel q of the output reads halo
+            // pixel q + 2 - kx; blocks blk, blk + 1 of the kernel rows
+            auto conv = [&](int grp, int rr, int blk, uint32_t dcol, int N, int j, uint32_t acc) {
+              const int kx = j >> 1, hh = j & 1;
+              mma_bf16(d + dcol,
+                       sdesc(base + kB2Dz2 + (2 * (grp & 3) + rr) * kB2Slot + 2 * hh * kRowBytes + (2 - kx) * 16,
+                             kRowBytes, 128),
+                       sdesc(base + kB2W2 + blk * 6144 + j * 256, 128, 1536), idesc_bf16(128, N), acc);
+            };
+#pragma unroll
+            for (int j = 0; j < 6; ++j) conv(g, 0, 1, 0, 64, j, j ? 1u : 0u);
+#pragma unroll
+            for (int j = 0; j < 6; ++j) conv(g, 1, 0, 0, 64, j, 1u);
+#pragma unroll
+            for (int j = 0; j < 6; ++j) {
+              conv(g - 1, 1, 2, 0, 32, j, 1u);
+              conv(g + 1, 0, 0, 32, 32, j, 1u);
+            }
+            mma_commit(prod + (c & 1));
+          }
+          if (before) {        // dW1 and db1 of the previous pair, step e
+            const int e = c - 1;
+            ok = bar_wait(ep + (e & 1), (uint32_t)(e >> 1) & 1u);
+            if (!ok) break;
+            tc_after_sync();
+            const uint32_t a = base + kB2Dz1 + (e & 1) * 8 * kChunkPx, x = base + kB2X + 3 * ((g - 1) & 3) * kChunkPx;
+#pragma unroll
+            for (int s = 0; s < kTileW / 16; ++s)
+#pragma unroll
+              for (int rr = 0; rr < 2; ++rr)
+                mma_bf16(tmem + kB2ColW1, sdesc(a + 4 * rr * kChunkPx + s * 256, 128, kChunkPx),
+                         sdesc(x + rr * kChunkPx + s * 256, 128, (2 - rr) * kChunkPx), idesc_bf16_mn(64, 16),
+                         e > 0 || s > 0 || rr ? 1u : 0u);
+          }
+          if (g > 0) mma_commit(done_d + ((g - 1) & 3));
+          before = mid;
+          if (mid) ++c;
         }
       }
+      if (!ok) fail();
+      mma_commit(drain);
+      if (!bar_wait(drain, 0u)) fail();
     }
-    pending = true;
-    ok = bar_wait(bar, phase);   // da1 done, and every MMA of the previous tile
-    phase ^= 1u;
-    tc_after_sync();
-    // 3. the previous tile's buffer set is free: prefetch the next tile
-    if (t + gridDim.x < ntiles) fetch(t + gridDim.x, set ^ 1);
-    // 4. dz1 = da1 [a1 > 0] (a1 of the centre row: halo row 131 + q)
-    {
-      float da[32];
-      tmem_ld32(tmem + lane_base + 0, da);
-      uint32_t a1w[16], w[16];
+  } else if (warp >= 6) {
+    // ---------------------------------------------------------- dW2 and db2
+    if (lane == 0) {
+      const int kx = warp - 6;
+      for (long long q = first; q < last && ok;) {
+        int b, x0, y0;
+        const int n = segment(q, &b, &x0, &y0);
+        q += n;
+        for (int P = -1; P <= n; ++P, ++g) {
+          const bool mid = P >= 0 && P < n;
+          ok = bar_wait(full_d + (g & 3), (uint32_t)(g >> 2) & 1u);
+          if (ok && mid) ok = bar_wait(full_a + c % 3, (uint32_t)(c / 3) & 1u);
+          if (*s_fail) ok = false;
+          if (!ok) break;
+          if (mid) {
+            const uint32_t a = base + kB2A1 + 2 * (c % 3) * kB2A1Slot + kx * 16;
+            const uint32_t z = base + kB2Dz2 + 2 * (g & 3) * kB2Slot + 16;
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        const uint4 u = *reinterpret_cast<const uint4 *>(sA1 + g * kHaloChunk + (kHaloW + 1 + p) * 16);
-        a1w[4 * g] = u.x; a1w[4 * g + 1] = u.y; a1w[4 * g + 2] = u.z; a1w[4 * g + 3] = u.w;
-      }
+            for (int s = 0; s < kTileW / 16; ++s)
 #pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const float lo = __uint_as_float(a1w[k] << 16), hi = __uint_as_float(a1w[k] & 0xFFFF0000u);
-        w[k] = pack_bf16x2(lo > 0.f ? da[2 * k] : 0.f, hi > 0.f ? da[2 * k + 1] : 0.f);
+              for (int rr = 0; rr < 2; ++rr)
+                mma_bf16(tmem + kB2ColW2 + 32 * kx, sdesc(a + rr * kB2A1Slot + s * 256, 128, kRowBytes),
+                         sdesc(z + rr * kB2Slot + s * 256, 128, kRowBytes), idesc_bf16_mn(128, 32),
+                         c > 0 || s > 0 || rr ? 1u : 0u);
+            mma_commit(done_c + c % 3);
+            ++c;
+          }
+          mma_commit(done_w + (g & 3));
+        }
       }
-      st_chunks(sDz1, kChunkPx, p, w);
+      if (!ok) fail();
+      mma_commit(drain + 1 + kx);
+      if (!bar_wait(drain + 1 + kx, 0u)) fail();
     }
-    fence_async_smem();
-    tc_before_sync();
-    __syncthreads();
-    tc_after_sync();
-    // 5. dW1^T: x against dz1
-    if (tid == 0) {
-      for (int s2 = 0; s2 < kTileW / 16; ++s2)
-        mma_bf16(tmem + 320, sdesc(smem_u32(sX) + s2 * 256, 128, kChunkPx),
-                 sdesc(smem_u32(sDz1) + s2 * 256, 128, kChunkPx), idesc_bf16_mn(64, 32),
-                 (!first || s2 > 0) ? 1u : 0u);
+  } else {
+    // ------------------------------------------------------------ epilogues
+    const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
+    for (long long q = first; q < last && ok;) {
+      int b, x0, y0;
+      const int n = segment(q, &b, &x0, &y0);
+      q += n;
+      for (int P = 0; P < n; ++P, ++c) {
+        ok = bar_wait(full_a + c % 3, (uint32_t)(c / 3) & 1u) && bar_wait(prod + (c & 1), (uint32_t)(c >> 1) & 1u);
+        ok = __all_sync(0xffffffffu, ok && !*s_fail);
+        if (!ok) break;
+        tc_after_sync();
+        // dz1 = da1 [a1 > 0]; a1 is zero outside the image
+#pragma unroll
+        for (int rr = 0; rr < 2; ++rr) {
+          float da[32];
+          tmem_ld32(tmem + lane_base + kB2ColDa + 64u * (uint32_t)(c & 1) + 32u * rr, da);
+          const uint8_t *a1 = smem + kB2A1 + (2 * (c % 3) + 1 + rr) * kB2A1Slot + (tid + 1) * 16;
+          uint8_t *dst = smem + kB2Dz1 + ((c & 1) * 8 + rr * 4) * kChunkPx;
+          uint32_t w[16];
+#pragma unroll
+          for (int ch = 0; ch < 4; ++ch) {
+            const uint4 u = *reinterpret_cast<const uint4 *>(a1 + ch * kRowBytes);
+            const uint32_t aw[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const float lo = __uint_as_float(aw[k] << 16), hi = __uint_as_float(aw[k] & 0xFFFF0000u);
+              w[4 * ch + k] = pack_bf16x2(lo > 0.f ? da[8 * ch + 2 * k] : 0.f, hi > 0.f ? da[8 * ch + 2 * k + 1] : 0.f);
+            }
+          }
+          st_chunks(dst, kChunkPx, tid, w);
+        }
+        fence_async_smem();
+        tc_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(ep + (c & 1));
+      }
     }
-    first = false;
-    tc_before_sync();
-    ok = __syncthreads_and(ok) != 0;   // uniform loop exit
+    if (!ok) fail();
   }
-  // the last tile's dW MMAs (after a wait that gave up: everything still in
-  // flight) under one more commit and one more bounded wait
-  if (pending) {
-    if (tid == 0) mma_commit(bar);
-    const bool done = bar_wait(bar, phase);
-    phase ^= 1u;
-    ok = __syncthreads_and(ok && done) != 0;
-  }
-  asm volatile("cp.async.wait_group 0;" ::: "memory");   // no copy outlives the CTA
-  if (!ok && tid == 0) atomicOr(status, kStatusTimeout);
-  if (!first) {
-    tc_after_sync();
+  tc_before_sync();
+  __syncthreads();
+  tc_after_sync();
+  if (*s_fail && tid == 0) atomicOr(status, kStatusTimeout);
+  // the CTA's sums into the global gradient: every MMA has completed
+  if (warp < 4) {
+    const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
     float d[32];
-    const int r = m64_row(tid);
-    for (int tap = 0; tap < 9; ++tap) {
-      tmem_ld32(tmem + lane_base + 32 + 32 * tap, d);
-      if (r >= 0 && r < 32) {
-        for (int o = 0; o < 32; ++o) atomicAdd(grad + kGW2 + o * 288 + tap * 32 + r, d[o]);
-      } else if (r == 32 && tap == 0) {
+    const int ky = tid / 40, i = tid % 40;   // D row 40 ky + i; i = 32: the ones
+    for (int kx = 0; kx < 3; ++kx) {
+      tmem_ld32(tmem + lane_base + kB2ColW2 + 32 * kx, d);
+      if (ky < 3 && i < 32) {
+#pragma unroll
+        for (int o = 0; o < 32; ++o) atomicAdd(grad + kGW2 + o * 288 + (3 * ky + kx) * 32 + i, d[o]);
+      } else if (kx == 0 && ky == 0 && i == 32) {
+#pragma unroll
         for (int o = 0; o < 32; ++o) atomicAdd(grad + kGb2 + o, d[o]);
       }
     }
-    tmem_ld32(tmem + lane_base + 320, d);
-    if (r >= 0 && r < 8) {
-      for (int o = 0; o < 32; ++o) atomicAdd(grad + kGW1 + o * 16 + r, d[o]);
-    } else if (r == 8) {
-      for (int o = 0; o < 32; ++o) atomicAdd(grad + kGb1 + o, d[o]);
+    const int r = m64_row(tid);
+    tmem_ld32(tmem + lane_base + kB2ColW1, d);
+    if (r >= 0 && r < 32) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) atomicAdd(grad + kGW1 + r * 16 + k, d[k]);
+      atomicAdd(grad + kGb1 + r, d[8]);
     }
   }
   tc_before_sync();
@@ -1028,7 +1197,7 @@ cudaError_t launch_selftest_wait(uint32_t *status, long long limit, cudaStream_t
 }
 
 cudaError_t launch_mpnet_forward(const void *weights, const uint16_t *feats, int batch, int W, int H, float *out,
-                                 uint16_t *acts, uint32_t *status, int num_sms, cudaStream_t s) {
+                                 uint16_t *acts, uint4 *a1p, uint32_t *status, int num_sms, cudaStream_t s) {
   if (batch <= 0 || W <= 0 || H <= 0) return cudaSuccess;
   // units: strips x row segments; the segment length balances the units over
   // the warpgroups (a unit of S output rows takes S + 4 pipeline steps)
@@ -1072,7 +1241,7 @@ cudaError_t launch_mpnet_forward(const void *weights, const uint16_t *feats, int
   cudaError_t e = cudaFuncSetAttribute(mpnet_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem);
   if (e != cudaSuccess) return e;
   mpnet_fwd_kernel<<<grid, kFwdThreads, kFwdSmem, s>>>(map, static_cast<const uint8_t *>(weights), batch, W, H, un,
-                                                       out, acts, status);
+                                                       out, acts, a1p, status);
   return cudaGetLastError();
 }
 
@@ -1090,21 +1259,24 @@ cudaError_t launch_mpnet_train(void *weights, float *master, float *adam_m, floa
   if (e != cudaSuccess) return e;
   mpnet_count_kernel<<<num_sms, 256, 0, s>>>(target, npix, sc.inv_n, nullptr);
   mpnet_count_finish_kernel<<<1, 1, 0, s>>>(sc.inv_n);
-  e = launch_mpnet_forward(weights, feats, batch, W, H, sc.y, sc.acts, status, num_sms, s);
+  e = launch_mpnet_forward(weights, feats, batch, W, H, sc.y, sc.acts, sc.a1, status, num_sms, s);
   if (e != cudaSuccess) return e;
-  const long long ntiles = (long long)batch * H * ((W + kTileW - 1) / kTileW);
-  const int grid = (int)(ntiles < num_sms ? ntiles : num_sms);
+  const int tiles_x = (W + kTileW - 1) / kTileW;
+  const long long ntiles = (long long)batch * H * tiles_x;
   // bwd1 holds 128 TMEM columns and 43 KB of shared memory: four CTAs per SM
   // give four independent tile streams
   const int grid1 = (int)(ntiles < 4ll * num_sms ? ntiles : 4ll * num_sms);
+  // bwd2: the row pairs of all strips, one contiguous range per CTA
+  const long long npairs = (long long)batch * tiles_x * ((H + 1) / 2);
+  const int grid2 = (int)(npairs < num_sms ? npairs : num_sms);
   e = cudaFuncSetAttribute(mpnet_bwd1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kB1Smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(mpnet_bwd2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kB2Smem);
   if (e != cudaSuccess) return e;
   mpnet_bwd1_kernel<<<grid1, kNetThreads, kB1Smem, s>>>(static_cast<const uint8_t *>(weights), sc.y, target, sc.acts,
                                                        batch, W, H, sc.inv_n, sc.dz2, sc.grad, loss, status);
-  mpnet_bwd2_kernel<<<grid, kNetThreads, kB2Smem, s>>>(static_cast<const uint8_t *>(weights),
-                                                       reinterpret_cast<const uint4 *>(feats), sc.acts, sc.dz2, batch,
-                                                       W, H, sc.grad, status);
+  mpnet_bwd2_kernel<<<grid2, kB2Threads, kB2Smem, s>>>(static_cast<const uint8_t *>(weights),
+                                                       reinterpret_cast<const uint4 *>(feats), sc.a1, sc.dz2, sc.zero,
+                                                       W, H, tiles_x, npairs, sc.grad, status);
   const float beta1 = 0.9f, beta2 = 0.999f;
   const float bc1 = 1.f - powf(beta1, (float)step), bc2 = 1.f - powf(beta2, (float)step);
   mpnet_adam_kernel<<<(kGTotal + 255) / 256, 256, 0, s>>>(static_cast<uint8_t *>(weights), master, adam_m, adam_v,
