@@ -26,6 +26,8 @@
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace dags {
@@ -154,17 +156,20 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // 1.4 products of N = 32 instead of three.
 //
 // Pipeline, step s of a unit with nO output rows (nA = nO + 2 a1 rows):
-//   control: wait for the previous step's epilogues; fetch the input of a1
-//     row s + 2; z1 of a1 row s (s < nA), commit; the bias of slot
+//   control: wait for the previous step's epilogues; the bias of slot
 //     (s - 1) mod 3 and the product of a1 row s - 1 (1 <= s <= nA) with
 //     z3 of output row s - 4 (4 <= s <= nA + 1) issued between its first
-//     MMAs, commit after z3, commit after the product.
+//     MMAs, commit after z3, commit after the product. Once epilogue 1 of
+//     this step is done: fetch the input three rows ahead, z1 of a1 row
+//     s + 1 (at the last step, of the next unit's first row), commit.
 //   epilogues: epilogue 1 once z1 is done (a1 row s into buffer s mod 2; the
 //     halo pixels 128 and 129 on the CUDA cores); epilogue 3 once z3 is done
 //     (a3, the dot product with w4 and the sigmoid of output row s - 4);
 //     epilogue 2 once the product is done (output row s - 3 complete in slot
 //     s mod 3: a2 into its buffer).
-// The product runs on the tensor core while epilogues 1 and 3 run. Every
+// The product runs on the tensor core while epilogues 1 and 3 run, the next
+// step's z1 while epilogues 3 and 2 do, so a step begins with its z1 done.
+// Every
 // buffer is rewritten only after the barrier that follows its last reader:
 // the a1 buffer s mod 2 was last read by the product of step s - 1, which
 // the commits of step s cover; the a2 buffer by the z3 of step s; a slot
@@ -183,7 +188,7 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // The third layer's bias is added in FP32 in its epilogue.
 constexpr int kGroups = 3;
 constexpr int kFwdThreads = 160 * kGroups;              // 4 epilogue warps + 1 control warp per warpgroup
-constexpr int kBars = 8;                                // mbarriers per warpgroup
+constexpr int kBars = 9;                                // mbarriers per warpgroup
 constexpr int kRowBytes = kHaloW * 16;                  // 2080 = the TMA box (8 x 130 x 1 x 1 bf16)
 constexpr int kInBuf = 2176;                            // one input row (+ pad)
 constexpr int kInBufs = 3;
@@ -230,9 +235,11 @@ __device__ __forceinline__ void tma_row(const CUtensorMap *map, uint32_t dst, ui
 
 __device__ __forceinline__ uint16_t bf16_bits(float x) { return __bfloat16_as_ushort(__float2bfloat16_rn(x)); }
 
+// The output rows of all 128-pixel column strips (strip after strip, image
+// after image), split evenly over the warpgroups.
 struct FwdUnits {
-  int tiles_x, segs, seg_rows;
-  long long count;
+  int tiles_x;
+  long long rows, slots;
 };
 
 __global__ void __launch_bounds__(kFwdThreads, 1)
@@ -258,9 +265,9 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
   uint8_t *wg = smem + g * kWgBytes;
   uint8_t *sA1 = wg + kWgA1, *sA2 = wg + kWgA2;
   // per warpgroup: in0..in2 (TMA), z1, z3, prod (MMA commits), ep (all
-  // epilogues done), drain (the final wait)
+  // epilogues done), drain (the final wait), ep1 (epilogue 1 done)
   uint64_t *bar_in = bars + kBars * g, *bar_z1 = bar_in + 3, *bar_z3 = bar_in + 4, *bar_prod = bar_in + 5,
-           *bar_ep = bar_in + 6, *bar_drain = bar_in + 7;
+           *bar_ep = bar_in + 6, *bar_drain = bar_in + 7, *bar_ep1 = bar_in + 8;
 
   // weights into the K-major core-matrix layouts; bias columns (hi, lo)
   const uint16_t *gw1 = reinterpret_cast<const uint16_t *>(weights + kOffW1);
@@ -307,7 +314,7 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
     sb4[0] = reinterpret_cast<const float *>(weights + kOffB4)[0];
     for (int k = 0; k < kBars * kGroups; ++k) {
       const int kind = k % kBars;   // ep: one arrival per epilogue warp
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bars + k)), "r"(kind == 6 ? 4 : 1));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bars + k)), "r"(kind == 6 || kind == 8 ? 4 : 1));
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     for (int k = 0; k < kGroups; ++k) s_fail[k] = 0u;
@@ -324,15 +331,15 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
   const uint32_t tmem = *s_tmem + kWgCols * (uint32_t)g;
   const uint32_t wg_u32 = smem_u32(wg);
   const uint32_t ones = wg_u32 + kWgOnes;
-  const long long stride = (long long)kGroups * gridDim.x;
-  // unit u -> image b, strip x0, rows [y0, y1)
-  auto unit = [&](long long u, int *b, int *x0, int *y0, int *y1) {
-    const int seg = (int)(u % units.segs);
-    const long long rest = u / units.segs;
-    *x0 = (int)(rest % units.tiles_x) * kTileW;
-    *b = (int)(rest / units.tiles_x);
-    *y0 = seg * units.seg_rows;
-    *y1 = min(*y0 + units.seg_rows, H);
+  // the warpgroup's rows [pos, end) of all strips' output rows in order; the
+  // unit at pos: image b, strip x0, rows [y0, y1)
+  const long long slot = (long long)kGroups * blockIdx.x + g;
+  auto unit = [&](long long pos, long long end, int *b, int *x0, int *y0, int *y1) {
+    const long long strip = pos / H;
+    *y0 = (int)(pos - strip * H);
+    *x0 = (int)(strip % units.tiles_x) * kTileW;
+    *b = (int)(strip / units.tiles_x);
+    *y1 = (int)min((long long)H, *y0 + (end - pos));
   };
   uint32_t qbase = 0;          // a1 rows of the earlier units (input buffer and phase)
   uint32_t sc = 0;             // steps of the earlier units (epilogue barrier phase)
@@ -349,38 +356,47 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
         tma_row(&in_map, wg_u32 + buf * kInBuf, bar_in + buf, x0 - 1, r, b);
         in_flight = (in_flight & ~(0x101u << buf)) | (1u << buf) | (((q / kInBufs) & 1u) << (8 + buf));
       };
-      long long u = (long long)kGroups * blockIdx.x + g;
-      if (u < units.count) {
-        int b, x0, y0, y1;
-        unit(u, &b, &x0, &y0, &y1);
-        fetch(0, x0, y0 - 1, b);
-        fetch(1, x0, y0, b);
+      const long long end = slot < units.slots ? units.rows * (slot + 1) / units.slots : 0;
+      long long pos = units.rows * slot / units.slots;
+      int b, x0, y0, y1;
+      // z1 of the next a1 row (halo pixels 0..127; the last two on the CUDA cores)
+      uint32_t qz = 0;
+      auto z1 = [&] {
+        const uint32_t buf = qz % kInBufs;
+        if (!bar_wait(bar_in + buf, (qz / kInBufs) & 1u)) return false;
+        in_flight = (in_flight & ~(1u << buf)) | 8u;
+        const uint32_t in = wg_u32 + buf * kInBuf, lbo = ones - in;
+        mma_bf16(tmem + kColD1, sdesc(in, lbo, 128), sdesc(smem_u32(sW1), 128, 256), idesc_bf16(128, 32), 0u);
+        mma_commit(bar_z1);
+        ++qz;
+        return true;
+      };
+      if (pos < end) {
+        unit(pos, end, &b, &x0, &y0, &y1);
+        for (int k = 0; k < kInBufs; ++k) fetch(k, x0, y0 - 1 + k, b);
+        ok = z1();
       }
-      for (; u < units.count && ok; u += stride) {
-        int b, x0, y0, y1;
-        unit(u, &b, &x0, &y0, &y1);
+      while (pos < end && ok) {
+        unit(pos, end, &b, &x0, &y0, &y1);
+        pos += y1 - y0;
         const int nO = y1 - y0, nA = nO + 2;
         int nb = 0, nx0 = 0, ny0 = 0, ny1 = 0;
-        const bool has_next = u + stride < units.count;
-        if (has_next) unit(u + stride, &nb, &nx0, &ny0, &ny1);
+        const bool has_next = pos < end;
+        if (has_next) unit(pos, end, &nb, &nx0, &ny0, &ny1);
         for (int s = 0; s < nA + 2; ++s, ++sc) {
-          const bool d1 = s < nA, dp = s >= 1 && s <= nA, d3 = s >= 4;
-          const uint32_t q = qbase + (uint32_t)s;
+          const bool dp = s >= 1 && s <= nA, d3 = s >= 4;
           if (s_fail[g]) { ok = false; break; }
-          // the previous step's epilogues have read D1, D3 and their slot and
-          // written a1 and a2; the input buffer of a1 row s - 1 is free
+          // the previous step's epilogues have read D3 and their slot and
+          // written a1 and a2
           if (sc > 0) ok = bar_wait(bar_ep, (sc - 1) & 1u);
           if (!ok) break;
           tc_after_sync();
-          if (s + 2 < nA) fetch(q + 2, x0, y0 + s + 1, b);
-          else if (has_next && s + 2 - nA < 2) fetch(q + 2, nx0, ny0 - 1 + (s + 2 - nA), nb);
           // The MMAs of one accumulator run one after another (about 68
-          // cycles apart); the three independent groups are interleaved so
-          // that the tensor core overlaps them: the bias of slot (s - 1) mod 3
-          // and the product of a1 row s - 1 (1 <= s <= nA), with z1 of a1 row
-          // s (s < nA; halo pixels 0..127, the last two on the CUDA cores)
-          // and z3 of output row s - 4 (4 <= s <= nA + 1) between its steps.
-          // A commit covers everything issued before it.
+          // cycles apart); the two independent groups are interleaved so that
+          // the tensor core overlaps them: the bias of slot (s - 1) mod 3 and
+          // the product of a1 row s - 1 (1 <= s <= nA), with z3 of output row
+          // s - 4 (4 <= s <= nA + 1) between its steps. A commit covers
+          // everything issued before it.
           const int k = s - 1, pk = (k + 3) % 3;
           const uint32_t a1 = smem_u32(sA1) + (uint32_t)(k & 1) * kSlotBytes;
           auto prod = [&](int j) {   // j = 2 * kx + hh
@@ -393,16 +409,6 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
             mma_bf16(tmem + kColD3, sdesc(a2 + 2 * h * (kTileW * 16), kTileW * 16, 128),
                      sdesc(smem_u32(sW3) + h * 256, 128, 512), idesc_bf16(128, 32), h ? 1u : 0u);
           };
-          if (d1) {
-            const uint32_t buf = q % kInBufs;
-            ok = bar_wait(bar_in + buf, (q / kInBufs) & 1u);
-            if (!ok) break;
-            in_flight = (in_flight & ~(1u << buf)) | 8u;
-            const uint32_t in = wg_u32 + buf * kInBuf, lbo = ones - in;
-            mma_bf16(tmem + kColD1, sdesc(in, lbo, 128), sdesc(smem_u32(sW1), 128, 256), idesc_bf16(128, 32), 0u);
-            mma_commit(bar_z1);
-            ++n_z1;
-          }
           in_flight |= 8u;
           if (dp) {
             mma_bf16(tmem + kColRing + 32 * (uint32_t)pk, sdesc(ones, 2048, 128), sdesc(smem_u32(sB2), 128, 256),
@@ -414,14 +420,25 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
           if (d3) {
             z3(1);
             mma_commit(bar_z3);
-            ++n_z3;
           }
           if (dp) {
 #pragma unroll
             for (int j = 2; j < 6; ++j) prod(j);
             mma_commit(bar_prod);
-            ++n_prod;
           }
+          // epilogue 1 of this step has read D1 and the input row: fetch three
+          // rows ahead into its buffer and issue the next z1, which runs under
+          // epilogues 3 and 2
+          ok = bar_wait(bar_ep1, sc & 1u);
+          if (!ok) break;
+          tc_after_sync();
+          if (s < nA) {
+            const uint32_t q = qbase + (uint32_t)s + kInBufs;
+            if (s + kInBufs < nA) fetch(q, x0, y0 - 1 + s + kInBufs, b);
+            else if (has_next) fetch(q, nx0, ny0 - 1 + (s + kInBufs - nA), nb);
+          }
+          if (s + 1 < nA || (s == nA + 1 && has_next)) ok = z1();
+          if (!ok) break;
         }
         qbase += (uint32_t)nA;
       }
@@ -446,9 +463,11 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
     const int p = 32 * warp + lane;
     const size_t plane_w = (size_t)units.tiles_x * kTileW + 2;
     bool ok = true;
-    for (long long u = (long long)kGroups * blockIdx.x + g; u < units.count && ok; u += stride) {
+    const long long end = slot < units.slots ? units.rows * (slot + 1) / units.slots : 0;
+    for (long long pos = units.rows * slot / units.slots; pos < end && ok;) {
       int b, x0, y0, y1;
-      unit(u, &b, &x0, &y0, &y1);
+      unit(pos, end, &b, &x0, &y0, &y1);
+      pos += y1 - y0;
       const int nO = y1 - y0, nA = nO + 2;
       for (int s = 0; s < nA + 2; ++s, ++sc) {
         const bool d1 = s < nA, d2 = s >= 3 && s <= nA, d3 = s >= 4;
@@ -513,6 +532,11 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
           }
           fence_async_smem();
         }
+        if (!ok) break;
+        // D1 and the input row are read: the next z1 may start
+        tc_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_ep1);
         // epilogue 3: a3, the dot product with w4 and the sigmoid of output
         // row y0 + s - 4
         if (ok && d3) {
@@ -1199,25 +1223,14 @@ cudaError_t launch_selftest_wait(uint32_t *status, long long limit, cudaStream_t
 cudaError_t launch_mpnet_forward(const void *weights, const uint16_t *feats, int batch, int W, int H, float *out,
                                  uint16_t *acts, uint4 *a1p, uint32_t *status, int num_sms, cudaStream_t s) {
   if (batch <= 0 || W <= 0 || H <= 0) return cudaSuccess;
-  // units: strips x row segments; the segment length balances the units over
-  // the warpgroups (a unit of S output rows takes S + 4 pipeline steps)
+  // One contiguous range of rows per warpgroup: a range costs its rows and,
+  // for each strip that it touches, four steps to fill and drain the pipeline.
+  // Ranges below four rows would spend more on filling than on rows.
   FwdUnits un;
   un.tiles_x = (W + kTileW - 1) / kTileW;
-  const long long strips = (long long)batch * un.tiles_x;
-  const long long slots = (long long)num_sms * kGroups;
-  double best = 1e300;
-  un.seg_rows = H;
-  for (int S = 4; S <= 96; ++S) {
-    const long long segs = (H + S - 1) / S;
-    const long long rounds = (strips * segs + slots - 1) / slots;
-    const double cost = (double)rounds * (S + 4);   // pipeline fill and drain: 4 steps
-    if (cost < best - 1e-9) { best = cost; un.seg_rows = S; }
-    if (S >= H) break;
-  }
-  un.segs = (H + un.seg_rows - 1) / un.seg_rows;
-  un.count = strips * un.segs;
-  const long long ctas = (un.count + kGroups - 1) / kGroups;
-  const int grid = (int)(ctas < num_sms ? ctas : num_sms);
+  un.rows = (long long)batch * un.tiles_x * H;
+  un.slots = std::max(1ll, std::min((long long)num_sms * kGroups, un.rows / 4));
+  const int grid = (int)((un.slots + kGroups - 1) / kGroups);
   static PFN_cuTensorMapEncodeTiled_v12000 encode = [] {
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult q;
