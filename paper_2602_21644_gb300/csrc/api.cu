@@ -149,7 +149,7 @@ void free_epi(EpiBuffers &b) {
 }
 
 void free_net(MpnetScratch &b) {
-  void *ptrs[] = {b.y, b.acts, b.a1, b.dz2, b.zero, b.grad, b.inv_n};
+  void *ptrs[] = {b.y, b.planes, b.dz2, b.zero, b.grad, b.inv_n};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   b = MpnetScratch();
@@ -1293,8 +1293,7 @@ int mpnet_train_step(dags_ctx *ctx, void *weights, float *master, float *adam_m,
     const long long cap = std::max(sc.cap, npix), plane_cap = std::max(sc.plane_cap, planes);
     free_net(sc);
     e = alloc(&sc.y, (size_t)cap);
-    if (e == cudaSuccess) e = alloc(&sc.acts, (size_t)cap * DAGS_MPNET_ACT_WORDS);
-    if (e == cudaSuccess) e = alloc(&sc.a1, (size_t)plane_cap);
+    if (e == cudaSuccess) e = alloc(&sc.planes, 3 * (size_t)plane_cap);
     if (e == cudaSuccess) e = alloc(&sc.dz2, (size_t)plane_cap);
     if (e == cudaSuccess) e = alloc(&sc.zero, kMpnetStrip + 2);
     if (e == cudaSuccess) e = cudaMemsetAsync(sc.zero, 0, (kMpnetStrip + 2) * sizeof(uint4), s);

@@ -267,20 +267,20 @@ cudaError_t launch_epipolar(const Raster &r, const double *pose_1, const double 
                             uint32_t *status, cudaStream_t s);
 
 cudaError_t launch_mpnet_forward(const void *weights, const uint16_t *feats, int batch, int W, int H, float *out,
-                                 uint16_t *acts, uint4 *a1p, uint32_t *status, int num_sms, cudaStream_t s);
+                                 uint16_t *acts, uint4 *planes, uint32_t *status, int num_sms, cudaStream_t s);
 
 // Scratch of a training step of the MP network (owned by the ctx).
 struct MpnetScratch {
   float *y = nullptr;        // [pixels]
-  uint16_t *acts = nullptr;  // [pixels][96] bf16
   // bf16 [image][row][4 chunks of 8 channels][1 + 128 strips + 1 pixels][8]:
-  // pixel x at plane position x + 1, zero outside the image
-  uint4 *a1 = nullptr, *dz2 = nullptr;
+  // pixel x at plane position x + 1; a1 and dz2 are zero outside the image
+  uint4 *planes = nullptr;   // a1, a2, a3
+  uint4 *dz2 = nullptr;
   uint4 *zero = nullptr;     // one zero row of 130 pixels x 8 channels
   float *grad = nullptr;     // [10881]
   float *inv_n = nullptr;    // [2]: 1 / valid pixels, valid count
   long long cap = 0;         // pixels
-  long long plane_cap = 0;   // uint4 of a1 and of dz2
+  long long plane_cap = 0;   // uint4 of one plane
 };
 constexpr int kMpnetStrip = 128;   // pixels of a column strip
 inline long long mpnet_plane_size(int batch, int W, int H) {

@@ -242,10 +242,13 @@ struct FwdUnits {
   long long rows, slots;
 };
 
+// kSave: the activations are kept, pixel-major for a caller (acts) or in
+// planes for the training step.
+template <bool kSave>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__restrict__ weights, int batch, int W,
                  int H, FwdUnits units, float *__restrict__ out, uint16_t *__restrict__ acts,
-                 uint4 *__restrict__ a1p, uint32_t *__restrict__ status) {
+                 uint4 *__restrict__ planes, size_t plane_n, uint32_t *__restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint8_t *sW1 = smem + kFW1, *sW2 = smem + kFW2, *sW3 = smem + kFW3, *sB2 = smem + kFB2;
@@ -495,13 +498,13 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
             for (int c = 0; c < 4; ++c)
               *reinterpret_cast<uint4 *>(a1 + c * kSlotChunk + i * 16) =
                   make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
-            if (a1p && own_row && (i >= 1 || x0 == 0)) {
+            if (kSave && planes && own_row && (i >= 1 || x0 == 0)) {
               // planar copy: plane pixel x + 1, zero outside the image
-              uint4 *ga = a1p + ((size_t)b * H + r) * 4 * plane_w + x0 + i;
+              uint4 *ga = planes + ((size_t)b * H + r) * 4 * plane_w + x0 + i;
 #pragma unroll
               for (int c = 0; c < 4; ++c)
                 ga[c * plane_w] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
-            } else if (acts && !a1p && own_row && i >= 1 && xx < W) {
+            } else if (kSave && acts && own_row && i >= 1 && xx < W) {
               uint4 *ga = reinterpret_cast<uint4 *>(acts + (((size_t)b * H + r) * W + xx) * 96);
 #pragma unroll
               for (int c = 0; c < 4; ++c) ga[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
@@ -525,9 +528,9 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
             zc = (zc + sb1h[c]) + sb1l[c];
             const uint16_t a = in ? bf16_bits(fmaxf(zc, 0.f)) : (uint16_t)0;
             *reinterpret_cast<uint16_t *>(a1 + (c >> 3) * kSlotChunk + i * 16 + (c & 7) * 2) = a;
-            if (a1p && own_row && (i <= kTileW || x0 + kHaloW == (int)plane_w))
-              reinterpret_cast<uint16_t *>(a1p + (((size_t)b * H + r) * 4 + (c >> 3)) * plane_w + x0 + i)[c & 7] = a;
-            else if (acts && !a1p && own_row && i <= kTileW && xx < W)
+            if (kSave && planes && own_row && (i <= kTileW || x0 + kHaloW == (int)plane_w))
+              reinterpret_cast<uint16_t *>(planes + (((size_t)b * H + r) * 4 + (c >> 3)) * plane_w + x0 + i)[c & 7] = a;
+            else if (kSave && acts && own_row && i <= kTileW && xx < W)
               acts[(((size_t)b * H + r) * W + xx) * 96 + c] = a;
           }
           fence_async_smem();
@@ -557,11 +560,17 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
           if (x0 + p < W) {
             const size_t pix = ((size_t)b * H + y) * W + x0 + p;
             out[pix] = __fdividef(1.f, 1.f + __expf(-acc));
-            if (acts) {
+            if (kSave && acts) {
               uint4 *ga = reinterpret_cast<uint4 *>(acts + pix * 96 + 64);
 #pragma unroll
               for (int c = 0; c < 4; ++c) ga[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
             }
+          }
+          if (kSave && planes) {
+            uint4 *ga = planes + 2 * plane_n + ((size_t)b * H + y) * 4 * plane_w + x0 + p + 1;
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              ga[c * plane_w] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
           }
         }
         // epilogue 2: output row y0 + s - 3 is complete in slot s mod 3 (its
@@ -581,7 +590,12 @@ mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__re
           for (int c = 0; c < 4; ++c)
             *reinterpret_cast<uint4 *>(sA2 + c * (kTileW * 16) + p * 16) =
                 make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
-          if (acts && x0 + p < W) {
+          if (kSave && planes) {
+            uint4 *ga = planes + plane_n + ((size_t)b * H + y) * 4 * plane_w + x0 + p + 1;
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              ga[c * plane_w] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+          } else if (kSave && acts && x0 + p < W) {
             uint4 *ga = reinterpret_cast<uint4 *>(acts + (((size_t)b * H + y) * W + x0 + p) * 96 + 32);
 #pragma unroll
             for (int c = 0; c < 4; ++c) ga[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
@@ -673,17 +687,22 @@ __host__ __device__ constexpr uint32_t idesc_bf16_mn(int M, int N) {
 
 constexpr int kChunkPx = kTileW * 16;                    // 2048: one chunk of a 128-pixel tile
 
-// bwd1 shared memory: a2 and a3 (5 chunks each: 4 real + ones, then 11 more
-// readable chunks for the M = 128 MMA), dz3 (4 chunks), dz4 (2 chunks), W3^T
-constexpr int kB1A2 = 0;
-constexpr int kB1A3 = kB1A2 + 5 * kChunkPx;
-constexpr int kB1Dz3 = kB1A3 + 5 * kChunkPx;
+// bwd1: BCE gradient, dz3, da2 = dz3 W3 and dz2; dW3, dw4, db3, db4. It is
+// bound by memory (200 B per pixel: a2 and a3 in, dz2 out), so its operands
+// come by bulk copies from the planar a2 and a3 two tiles ahead, straight into
+// the layout that the MMAs read, and four CTAs per SM overlap the tiles'
+// chains. Warps 0..3 compute (thread = pixel), warp 4 issues copies and MMAs.
+// Shared memory: two stages of a2 and a3 (five chunks each: four real and the
+// ones; an M = 64 MMA reads three more chunks past them, in bounds, their D
+// rows unused), dz3 (four chunks), dz4 (two chunks), W3^T.
+constexpr int kB1Threads = kNetThreads + 32;
+constexpr int kB1Stage = 10 * kChunkPx;
+constexpr int kB1Dz3 = 2 * kB1Stage;
 constexpr int kB1Dz4 = kB1Dz3 + 4 * kChunkPx;
 constexpr int kB1W3T = kB1Dz4 + 2 * kChunkPx;
 constexpr int kB1Par = kB1W3T + 2048;
 constexpr int kB1Bar = kB1Par + 128;
-constexpr int kB1Span = 16 * kChunkPx;                    // the farthest MN-major read from kB1A3
-constexpr int kB1Smem = (kB1A3 + kB1Span > kB1Bar + 64 ? kB1A3 + kB1Span : kB1Bar + 64);
+constexpr int kB1Smem = kB1Bar + 64;
 
 __device__ __forceinline__ void st_chunks(uint8_t *base, int stride, int row, const uint32_t *w) {
 #pragma unroll
@@ -691,31 +710,44 @@ __device__ __forceinline__ void st_chunks(uint8_t *base, int stride, int row, co
     *reinterpret_cast<uint4 *>(base + c * stride + row * 16) = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
 }
 
-__global__ void __launch_bounds__(kNetThreads)
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_t bytes, uint64_t *bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
+}
+
+__global__ void __launch_bounds__(kB1Threads, 4)
 mpnet_bwd1_kernel(const uint8_t *__restrict__ weights, const float *__restrict__ y, const float *__restrict__ target,
-                  const uint16_t *__restrict__ acts, int batch, int W, int H, const float *__restrict__ inv_n,
-                  uint4 *__restrict__ dz2p, float *__restrict__ grad, double *__restrict__ loss,
-                  uint32_t *__restrict__ status) {
+                  const uint4 *__restrict__ a2p, const uint4 *__restrict__ a3p, int batch, int W, int H,
+                  const float *__restrict__ inv_n, uint4 *__restrict__ dz2p, float *__restrict__ grad,
+                  double *__restrict__ loss, uint32_t *__restrict__ status) {
   extern __shared__ __align__(128) uint8_t smem[];
-  uint8_t *sA2 = smem + kB1A2, *sA3 = smem + kB1A3, *sDz3 = smem + kB1Dz3, *sDz4 = smem + kB1Dz4;
-  uint8_t *sW3T = smem + kB1W3T;
+  uint8_t *sDz3 = smem + kB1Dz3, *sDz4 = smem + kB1Dz4, *sW3T = smem + kB1W3T;
   float *sw4 = reinterpret_cast<float *>(smem + kB1Par);
-  uint64_t *bar = reinterpret_cast<uint64_t *>(smem + kB1Bar);
-  uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + kB1Bar + 8);
+  // full[2] the copies of a stage, ready dz3 and dz4 written, done the tile's MMAs
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + kB1Bar), *ready = full + 2, *done = full + 3, *drain = full + 4;
+  uint32_t *s_tmem = reinterpret_cast<uint32_t *>(full + 5);
+  volatile uint32_t *s_fail = reinterpret_cast<volatile uint32_t *>(s_tmem + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint16_t *gw3 = reinterpret_cast<const uint16_t *>(weights + kOffW3);
-  // everything starts at zero (the M = 128 reads past the real rows see finite
-  // values); the ones chunks; W3^T in the K-major core-matrix layout
-  for (int e = tid; e < kB1Smem / 16; e += kNetThreads) reinterpret_cast<uint4 *>(smem)[e] = make_uint4(0u, 0u, 0u, 0u);
-  __syncthreads();
-  for (int e = tid; e < 32 * 32; e += kNetThreads) {
+  // everything starts at zero; the ones chunks; W3^T in the K-major
+  // core-matrix layout
+  for (int e = tid; e < kB1W3T / 16; e += kB1Threads) {
+    const int chunk = e / kTileW;
+    reinterpret_cast<uint4 *>(smem)[e] = make_uint4(chunk < 20 && chunk % 5 == 4 ? 0x3F80u : 0u, 0u, 0u, 0u);
+  }
+  for (int e = tid; e < 32 * 32; e += kB1Threads) {
     const int o = e / 32, i = e % 32;
     *reinterpret_cast<uint16_t *>(sW3T + core_off(i, o, 32)) = gw3[e];
   }
-  *reinterpret_cast<uint4 *>(sA2 + 4 * kChunkPx + tid * 16) = make_uint4(0x3F80u, 0u, 0u, 0u);
-  *reinterpret_cast<uint4 *>(sA3 + 4 * kChunkPx + tid * 16) = make_uint4(0x3F80u, 0u, 0u, 0u);
   if (tid < kCh) sw4[tid] = __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(weights + kOffW4)[tid]);
-  if (tid == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)));
+  if (tid == 0) {
+    for (int k = 0; k < 5; ++k)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(full + k)), "r"(k == 2 ? 4 : 1));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    *s_fail = 0u;
+  }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(128));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -725,105 +757,155 @@ mpnet_bwd1_kernel(const uint8_t *__restrict__ weights, const float *__restrict__
   __syncthreads();
   tc_after_sync();
   const uint32_t tmem = *s_tmem;   // D: da2 cols 0-31, dW3^T cols 32-63, dw4 cols 64-79
-  const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
-  uint32_t phase = 0;
-  bool ok = true, first = true;
-  float lsum = 0.f;
-  const float invn = inv_n[0];
   const int tiles_x = (W + kTileW - 1) / kTileW;
   const size_t plane_w = (size_t)tiles_x * kTileW + 2;
   const long long ntiles = (long long)batch * H * tiles_x;
-  for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-    const int tx = (int)(t % tiles_x), yy = (int)((t / tiles_x) % H), b = (int)(t / ((long long)tiles_x * H));
-    const int p = tid, x = tx * kTileW + p;
-    const bool in = x < W;
-    const size_t pix = ((size_t)b * H + yy) * W + x;
-    float dz4 = 0.f;
-    uint32_t a2w[16], a3w[16];
-    if (in) {
-      const float tg = target[pix], yv = y[pix];
+  bool ok = true;
+  float lsum = 0.f;
+  if (warp == 4) {
+    if (lane == 0) {
+      int last[2] = {-1, -1};
+      auto load = [&](long long t, int i) {   // the CTA's i-th tile into stage i mod 2
+        const long long row = t / tiles_x;
+        const size_t src = (size_t)row * 4 * plane_w + (size_t)(t - row * tiles_x) * kTileW + 1;
+        uint64_t *bar = full + (i & 1);
+        const uint32_t dst = smem_u32(smem) + (i & 1) * kB1Stage;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(8 * kChunkPx)
+                     : "memory");
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          bulk_copy(dst + c * kChunkPx, a2p + src + c * plane_w, kChunkPx, bar);
+          bulk_copy(dst + (5 + c) * kChunkPx, a3p + src + c * plane_w, kChunkPx, bar);
+        }
+        last[i & 1] = i;
+      };
+      const long long grid = gridDim.x;
+      load(blockIdx.x, 0);
+      if (blockIdx.x + grid < ntiles) load(blockIdx.x + grid, 1);
+      int i = 0;
+      for (long long t = blockIdx.x; t < ntiles; t += grid, ++i) {
+        ok = bar_wait(full + (i & 1), (uint32_t)(i >> 1) & 1u) && bar_wait(ready, (uint32_t)i & 1u);
+        if (*s_fail) ok = false;
+        if (!ok) break;
+        tc_after_sync();
+        const uint32_t a2 = smem_u32(smem) + (i & 1) * kB1Stage, a3 = a2 + 5 * kChunkPx;
+        // da2 = dz3 W3 (M = pixels, K = o)
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+          mma_bf16(tmem + 0, sdesc(smem_u32(sDz3) + 2 * c * kChunkPx, kChunkPx, 128),
+                   sdesc(smem_u32(sW3T) + c * 256, 128, 512), idesc_bf16(128, 32), c > 0 ? 1u : 0u);
+        // dW3^T (M = i, N = o) and dw4 (M = i, N = 16) over the tile's pixels
+#pragma unroll
+        for (int s = 0; s < kTileW / 16; ++s) {
+          const uint32_t acc = i > 0 || s > 0 ? 1u : 0u;
+          mma_bf16(tmem + 32, sdesc(a2 + s * 256, 128, kChunkPx), sdesc(smem_u32(sDz3) + s * 256, 128, kChunkPx),
+                   idesc_bf16_mn(64, 32), acc);
+          mma_bf16(tmem + 64, sdesc(a3 + s * 256, 128, kChunkPx), sdesc(smem_u32(sDz4) + s * 256, 128, kChunkPx),
+                   idesc_bf16_mn(64, 16), acc);
+        }
+        mma_commit(done);
+        if (t + 2 * grid < ntiles) {   // the stage is free once the MMAs are done
+          ok = bar_wait(done, (uint32_t)i & 1u);
+          if (!ok) break;
+          load(t + 2 * grid, i + 2);
+        }
+      }
+      if (!ok) *s_fail = 1u;
+      // no copy and no MMA outlives the CTA
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        if (last[k] >= 0) bar_wait(full + k, (uint32_t)(last[k] >> 1) & 1u);
+      mma_commit(drain);
+      if (!bar_wait(drain, 0u)) *s_fail = 1u;
+    }
+  } else {
+    const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
+    const float invn = inv_n[0];
+    const int p = tid;
+    auto fetch = [&](long long t, float *tg, float *yv) {   // target and output of this thread's pixel
+      const long long row = t / tiles_x;
+      const int x = (int)(t - row * tiles_x) * kTileW + p;
+      *tg = -1.f;
+      *yv = 0.f;
+      if (t < ntiles && x < W) {
+        *tg = target[(size_t)row * W + x];
+        *yv = y[(size_t)row * W + x];
+      }
+    };
+    float tg, yv;
+    fetch(blockIdx.x, &tg, &yv);
+    int i = 0;
+    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
+      float dz4 = 0.f;
       if (tg >= 0.f) {
         dz4 = (yv - tg) * invn;
         const float yc = fminf(fmaxf(yv, 1e-12f), 0.99999994f);   // largest float below 1
         lsum -= (tg * logf(yc) + (1.f - tg) * logf(1.f - yc)) * invn;
       }
-      const uint4 *ga = reinterpret_cast<const uint4 *>(acts + pix * 96);
+      ok = bar_wait(full + (i & 1), (uint32_t)(i >> 1) & 1u);
+      ok = __all_sync(0xffffffffu, ok && !*s_fail);
+      if (!ok) break;
+      const uint8_t *a2 = smem + (i & 1) * kB1Stage + p * 16, *a3 = a2 + 5 * kChunkPx;
+      // dz3 = dz4 w4 [a3 > 0], and the bits [a2 > 0]
+      uint32_t dzw[16], pos = 0u;
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        const uint4 u2 = ga[4 + g], u3 = ga[8 + g];
-        a2w[4 * g] = u2.x; a2w[4 * g + 1] = u2.y; a2w[4 * g + 2] = u2.z; a2w[4 * g + 3] = u2.w;
-        a3w[4 * g] = u3.x; a3w[4 * g + 1] = u3.y; a3w[4 * g + 2] = u3.z; a3w[4 * g + 3] = u3.w;
+      for (int c = 0; c < 4; ++c) {
+        const uint4 u3 = *reinterpret_cast<const uint4 *>(a3 + c * kChunkPx);
+        const uint4 u2 = *reinterpret_cast<const uint4 *>(a2 + c * kChunkPx);
+        const uint32_t w3[4] = {u3.x, u3.y, u3.z, u3.w}, w2[4] = {u2.x, u2.y, u2.z, u2.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int k = 4 * c + e;
+          const float lo = __uint_as_float(w3[e] << 16), hi = __uint_as_float(w3[e] & 0xFFFF0000u);
+          dzw[k] = pack_bf16x2(lo > 0.f ? dz4 * sw4[2 * k] : 0.f, hi > 0.f ? dz4 * sw4[2 * k + 1] : 0.f);
+          pos |= (__uint_as_float(w2[e] << 16) > 0.f ? 1u << (2 * k) : 0u) |
+                 (__uint_as_float(w2[e] & 0xFFFF0000u) > 0.f ? 2u << (2 * k) : 0u);
+        }
       }
-    } else {
-#pragma unroll
-      for (int k = 0; k < 16; ++k) { a2w[k] = 0u; a3w[k] = 0u; }
-    }
-    // dz3 = dz4 w4 [a3 > 0]
-    uint32_t dzw[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const float a3lo = __uint_as_float(a3w[k] << 16), a3hi = __uint_as_float(a3w[k] & 0xFFFF0000u);
-      dzw[k] = pack_bf16x2(a3lo > 0.f ? dz4 * sw4[2 * k] : 0.f, a3hi > 0.f ? dz4 * sw4[2 * k + 1] : 0.f);
-    }
-    st_chunks(sA2, kChunkPx, p, a2w);
-    st_chunks(sA3, kChunkPx, p, a3w);
-    st_chunks(sDz3, kChunkPx, p, dzw);
-    *reinterpret_cast<uint4 *>(sDz4 + p * 16) = make_uint4(__bfloat16_as_ushort(__float2bfloat16_rn(dz4)), 0u, 0u, 0u);
-    fence_async_smem();
-    tc_before_sync();
-    __syncthreads();
-    tc_after_sync();
-    if (tid == 0) {
-      // da2 = dz3 W3 (M = pixels, K = o)
-      for (int c = 0; c < 2; ++c)
-        mma_bf16(tmem + 0, sdesc(smem_u32(sDz3) + 2 * c * kChunkPx, kChunkPx, 128),
-                 sdesc(smem_u32(sW3T) + c * 256, 128, 512), idesc_bf16(128, 32), c > 0 ? 1u : 0u);
-      // dW3^T (M = i, N = o) and dw4 (M = i, N = 16) over the tile's pixels
-      for (int s = 0; s < kTileW / 16; ++s) {
-        const uint32_t acc = (!first || s > 0) ? 1u : 0u;
-        mma_bf16(tmem + 32, sdesc(smem_u32(sA2) + s * 256, 128, kChunkPx),
-                 sdesc(smem_u32(sDz3) + s * 256, 128, kChunkPx), idesc_bf16_mn(64, 32), acc);
-        mma_bf16(tmem + 64, sdesc(smem_u32(sA3) + s * 256, 128, kChunkPx),
-                 sdesc(smem_u32(sDz4) + s * 256, 128, kChunkPx), idesc_bf16_mn(64, 16), acc);
-      }
-      mma_commit(bar);
-    }
-    ok = bar_wait(bar, phase);
-    phase ^= 1u;
-    tc_after_sync();
-    first = false;
-    // dz2 = (dz3 W3) [a2 > 0] -> global (bf16) for the second backward kernel
-    {
+      st_chunks(sDz3, kChunkPx, p, dzw);
+      *reinterpret_cast<uint4 *>(sDz4 + p * 16) = make_uint4(__bfloat16_as_ushort(__float2bfloat16_rn(dz4)), 0u, 0u, 0u);
+      fence_async_smem();
+      tc_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(ready);
+      fetch(t + gridDim.x, &tg, &yv);
+      ok = bar_wait(done, (uint32_t)i & 1u);
+      ok = __all_sync(0xffffffffu, ok && !*s_fail);
+      if (!ok) break;
+      tc_after_sync();
+      // dz2 = (dz3 W3) [a2 > 0] -> global (bf16) for the second backward
+      // kernel; dz3 is zero outside the image
       float da[32];
       tmem_ld32(tmem + lane_base + 0, da);
-      uint32_t w[16];
+      const long long row = t / tiles_x;
+      const int x = (int)(t - row * tiles_x) * kTileW + p;
+      uint4 *dst = dz2p + (size_t)row * 4 * plane_w + x + 1;
+      const bool left = x == 0, right = x + 3 == (int)plane_w;
 #pragma unroll
-      for (int k = 0; k < 16; ++k) {   // a2 = 0 outside the image
-        const float a2lo = __uint_as_float(a2w[k] << 16), a2hi = __uint_as_float(a2w[k] & 0xFFFF0000u);
-        w[k] = pack_bf16x2(a2lo > 0.f ? da[2 * k] : 0.f, a2hi > 0.f ? da[2 * k + 1] : 0.f);
-      }
-      uint4 *dst = dz2p + ((size_t)b * H + yy) * 4 * plane_w + x + 1;
-      const bool right = x + 3 == (int)plane_w;
+      for (int c = 0; c < 4; ++c) {
+        uint32_t w[4];
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        uint4 *d = dst + g * plane_w;
-        *d = make_uint4(w[4 * g], w[4 * g + 1], w[4 * g + 2], w[4 * g + 3]);
-        if (x == 0) d[-1] = make_uint4(0u, 0u, 0u, 0u);
+        for (int e = 0; e < 4; ++e) {
+          const int k = 4 * c + e;
+          w[e] = pack_bf16x2(pos >> (2 * k) & 1u ? da[2 * k] : 0.f, pos >> (2 * k + 1) & 1u ? da[2 * k + 1] : 0.f);
+        }
+        uint4 *d = dst + c * plane_w;
+        *d = make_uint4(w[0], w[1], w[2], w[3]);
+        if (left) d[-1] = make_uint4(0u, 0u, 0u, 0u);
         if (right) d[1] = make_uint4(0u, 0u, 0u, 0u);
       }
     }
-    tc_before_sync();
-    ok = __syncthreads_and(ok) != 0;   // uniform loop exit
+    if (!ok) *s_fail = 1u;
   }
-  if (!ok) {
-    if (tid == 0) atomicOr(status, kStatusTimeout);
-    bar_wait(bar, phase ^ 1u);
-  }
-  // the CTA's accumulated weight gradients: row r of D = input channel (or the
-  // ones row), column = output channel; an M = 64 accumulator's row r is in
-  // TMEM lane 32 (r / 16) + r % 16
-  if (!first) {
-    tc_after_sync();
+  tc_before_sync();
+  __syncthreads();
+  tc_after_sync();
+  if (*s_fail && tid == 0) atomicOr(status, kStatusTimeout);
+  if (warp < 4) {
+    // the CTA's accumulated weight gradients: row r of D = input channel (or
+    // the ones row), column = output channel; an M = 64 accumulator's row r is
+    // in TMEM lane 32 (r / 16) + r % 16
+    const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
     float d[32];
     tmem_ld32(tmem + lane_base + 32, d);
     const int r = m64_row(tid);
@@ -891,13 +973,6 @@ constexpr int kB2NBars = 4 + 3 + 4 + 4 + 3 + 2 + 2 + 4;
 constexpr int kB2Smem = kB2Bar + 8 * kB2NBars + 16;
 constexpr uint32_t kB2ColW2 = 0, kB2ColDa = 128, kB2ColW1 = 256;
 static_assert(kB2Smem <= 227 * 1024, "shared memory");
-
-__device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_t bytes, uint64_t *bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
 
 __global__ void __launch_bounds__(kB2Threads, 1)
 mpnet_bwd2_kernel(const uint8_t *__restrict__ weights, const uint4 *__restrict__ feats, const uint4 *__restrict__ a1p,
@@ -1221,7 +1296,7 @@ cudaError_t launch_selftest_wait(uint32_t *status, long long limit, cudaStream_t
 }
 
 cudaError_t launch_mpnet_forward(const void *weights, const uint16_t *feats, int batch, int W, int H, float *out,
-                                 uint16_t *acts, uint4 *a1p, uint32_t *status, int num_sms, cudaStream_t s) {
+                                 uint16_t *acts, uint4 *planes, uint32_t *status, int num_sms, cudaStream_t s) {
   if (batch <= 0 || W <= 0 || H <= 0) return cudaSuccess;
   // One contiguous range of rows per warpgroup: a range costs its rows and,
   // for each strip that it touches, four steps to fill and drain the pipeline.
@@ -1251,10 +1326,11 @@ cudaError_t launch_mpnet_forward(const void *weights, const uint16_t *feats, int
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(mpnet_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem);
+  const auto kernel = acts || planes ? mpnet_fwd_kernel<true> : mpnet_fwd_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem);
   if (e != cudaSuccess) return e;
-  mpnet_fwd_kernel<<<grid, kFwdThreads, kFwdSmem, s>>>(map, static_cast<const uint8_t *>(weights), batch, W, H, un,
-                                                       out, acts, a1p, status);
+  kernel<<<grid, kFwdThreads, kFwdSmem, s>>>(map, static_cast<const uint8_t *>(weights), batch, W, H, un, out, acts,
+                                             planes, (size_t)mpnet_plane_size(batch, W, H), status);
   return cudaGetLastError();
 }
 
@@ -1272,11 +1348,11 @@ cudaError_t launch_mpnet_train(void *weights, float *master, float *adam_m, floa
   if (e != cudaSuccess) return e;
   mpnet_count_kernel<<<num_sms, 256, 0, s>>>(target, npix, sc.inv_n, nullptr);
   mpnet_count_finish_kernel<<<1, 1, 0, s>>>(sc.inv_n);
-  e = launch_mpnet_forward(weights, feats, batch, W, H, sc.y, sc.acts, sc.a1, status, num_sms, s);
+  e = launch_mpnet_forward(weights, feats, batch, W, H, sc.y, nullptr, sc.planes, status, num_sms, s);
   if (e != cudaSuccess) return e;
   const int tiles_x = (W + kTileW - 1) / kTileW;
   const long long ntiles = (long long)batch * H * tiles_x;
-  // bwd1 holds 128 TMEM columns and 43 KB of shared memory: four CTAs per SM
+  // bwd1 holds 128 TMEM columns and 55 KB of shared memory: four CTAs per SM
   // give four independent tile streams
   const int grid1 = (int)(ntiles < 4ll * num_sms ? ntiles : 4ll * num_sms);
   // bwd2: the row pairs of all strips, one contiguous range per CTA
@@ -1285,10 +1361,12 @@ cudaError_t launch_mpnet_train(void *weights, float *master, float *adam_m, floa
   e = cudaFuncSetAttribute(mpnet_bwd1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kB1Smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(mpnet_bwd2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kB2Smem);
   if (e != cudaSuccess) return e;
-  mpnet_bwd1_kernel<<<grid1, kNetThreads, kB1Smem, s>>>(static_cast<const uint8_t *>(weights), sc.y, target, sc.acts,
-                                                       batch, W, H, sc.inv_n, sc.dz2, sc.grad, loss, status);
+  const size_t plane_n = (size_t)mpnet_plane_size(batch, W, H);
+  mpnet_bwd1_kernel<<<grid1, kB1Threads, kB1Smem, s>>>(static_cast<const uint8_t *>(weights), sc.y, target,
+                                                      sc.planes + plane_n, sc.planes + 2 * plane_n, batch, W, H,
+                                                      sc.inv_n, sc.dz2, sc.grad, loss, status);
   mpnet_bwd2_kernel<<<grid2, kB2Threads, kB2Smem, s>>>(static_cast<const uint8_t *>(weights),
-                                                       reinterpret_cast<const uint4 *>(feats), sc.a1, sc.dz2, sc.zero,
+                                                       reinterpret_cast<const uint4 *>(feats), sc.planes, sc.dz2, sc.zero,
                                                        W, H, tiles_x, npairs, sc.grad, status);
   const float beta1 = 0.9f, beta2 = 0.999f;
   const float bc1 = 1.f - powf(beta1, (float)step), bc2 = 1.f - powf(beta2, (float)step);
