@@ -128,7 +128,7 @@ void free_ws(Workspace &w) {
 }
 
 void free_mp(MpBuffers &b) {
-  void *ptrs[] = {b.e, b.mpf, b.acc, b.mhat, b.sige, b.U, b.Mt, b.Ut, b.obs, b.hist, b.sel};
+  void *ptrs[] = {b.e, b.mpf, b.acc, b.mhat, b.sige, b.U, b.Mt, b.Ut, b.idx, b.hist, b.sel};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   b = MpBuffers();
@@ -340,8 +340,8 @@ int dags_create(dags_ctx **out, int64_t max_gaussians, int32_t max_width, int32_
   A(alloc(&mb.U, (size_t)w.max_n));
   A(alloc(&mb.Mt, (size_t)w.max_n));
   A(alloc(&mb.Ut, (size_t)w.max_n));
-  A(alloc(&mb.obs, (size_t)w.max_n));
-  A(alloc(&mb.hist, (size_t)2 * 2048));
+  A(alloc(&mb.idx, (size_t)w.max_n));
+  A(alloc(&mb.hist, (size_t)3 * 2 * 2048));
   A(alloc(&mb.sel, (size_t)8));
   if (e == cudaSuccess) e = cudaMemset(w.counters, 0, CNT_N * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(w.evals, 0, 4 * sizeof(unsigned long long));

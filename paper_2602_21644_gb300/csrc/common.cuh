@@ -307,8 +307,8 @@ struct MpBuffers {
   float *pyr = nullptr;               // [mp_pyramid_floats] levels 1.. of the association pyramid
   double *acc = nullptr;              // [DAGS_MP_MAX_REGIONS * 4]
   float *mhat = nullptr, *sige = nullptr, *U = nullptr, *Mt = nullptr, *Ut = nullptr;  // [max_n]
-  uint8_t *obs = nullptr;             // [max_n]
-  uint32_t *hist = nullptr;           // [2 * 2048]
+  uint32_t *idx = nullptr;            // [max_n]
+  uint32_t *hist = nullptr;           // [3 * 2 * 2048]
   uint32_t *sel = nullptr;            // [8]
 };
 cudaError_t launch_semantic_trigger(const double *stats, const dags_sched_cfg &cfg, int seg_refreshed,

@@ -20,17 +20,14 @@
 //                         radius r_s around pi(G) / 2^s, over the stored M_p
 //                         (or the caller's map); M_hat, Eq. (8), with weights
 //                         2^-s exp(-d^2 / (2 sigma_w^2)); Var{M_p}; sigma_e,G;
-//                         U, Eq. (10); CTA min/max of U -> global
-//   mp_apply_kernel       per observed Gaussian: normalised U, C, alpha,
-//                         Eqs. (11), (17); M^t, Eq. (9), written into the
-//                         record; first radix-select level of the two medians
-//   mp_select_kernel      further radix-select levels (exact lower medians of
-//                         M^t and U_tilde over the observed Gaussians, bits
-//                         31-21, 20-10, 9-0 of the non-negative floats);
-//                         the last CTA of the last level writes tau, U_bar
-//   mp_labels_kernel      labels, Eq. (12)
-// The last CTA of each histogram kernel finds the bin holding the median's
-// rank (one warp scans the bins).
+//                         U, Eq. (10); min/max of U; the observed Gaussians
+//                         as a compact list (in no particular order)
+//   mp_apply_kernel       one cooperative launch over that list: normalised U,
+//                         C, alpha, Eqs. (11), (17); M^t, Eq. (9), written
+//                         into the records; exact lower medians of M^t and
+//                         U_tilde by radix select (bits 31-21, 20-10, 9-0 of
+//                         the non-negative floats, a grid barrier per level);
+//                         tau, U_bar; labels, Eq. (12); region statistics
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -42,6 +39,7 @@ namespace {
 
 constexpr int kMpBlock = 256;
 constexpr int kSelBins = 2048;
+constexpr int kSelLevels = 3;
 
 struct MpCfg {
   float kappa_c, lam, sigma_min, e_floor, sigma_g, sigma_c, lam_u, eps, alpha_min, alpha_max, rho, r_s, sigma_w,
@@ -55,11 +53,12 @@ constexpr int kMaxScales = DAGS_MP_MAX_SCALES;
 struct MpWs {
   float *e;              // [P] residual per pixel
   double *acc;           // [256][4] region count, sum, centred sum of squares, -
+  // the observed Gaussians, compact: index, M_hat, sigma_e, U; Mt: their MP,
+  // then M^t; Ut: U_tilde
+  uint32_t *idx;         // [N]
   float *mhat, *sige, *U, *Mt, *Ut;  // [N]
-  uint8_t *obs;          // [N]
-  uint32_t *hist;        // [2][kSelBins]
-  uint32_t *sel;         // select state: [0] n_obs, [1] Umin bits, [2] Umax bits, [3] done counter,
-                         // [4..5] prefix (M, U), [6..7] remaining rank (M, U)
+  uint32_t *hist;        // [kSelLevels][2][kSelBins]
+  uint32_t *sel;         // [0] n_obs, [1] Umin bits, [2] Umax bits, [3] arrivals at the grid barriers
   double *stats;         // caller's output
   const float *mp_map;   // [P] external per-pixel MP replacing M_p, or null
   float *mp_pixel;       // [P] out: the fused M_p, or null
@@ -105,12 +104,12 @@ mp_pixel_sum_kernel(MpWs m, const float4 *__restrict__ targets, const float *__r
   for (int k = threadIdx.x; k < c.n_regions; k += blockDim.x) { s_cnt[k] = 0.f; s_sum[k] = 0.f; }
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   // select state and histograms start cleared (used from mp_gauss_kernel on)
-  for (int k = p; k < 2 * kSelBins; k += gridDim.x * blockDim.x) m.hist[k] = 0u;
+  for (int k = p; k < kSelLevels * 2 * kSelBins; k += gridDim.x * blockDim.x) m.hist[k] = 0u;
   if (p == 0) {
     m.sel[0] = 0u;            // observed count
     m.sel[1] = 0xFFFFFFFFu;   // min of U (ordered key)
     m.sel[2] = 0u;            // max of U (ordered key)
-    m.sel[3] = 0u;            // CTA counter
+    m.sel[3] = 0u;            // barrier arrivals
   }
   __syncthreads();
   float e = 0.f;
@@ -312,263 +311,280 @@ __device__ __forceinline__ bool disk_rect(float us, float vs, int Ws, int Hs, fl
   return *i0 <= *i1 && *j0 <= *j1;
 }
 
+// Sums over the members of N(G): f(level weight, dx^2 + dy^2, pixel, level).
+// kSmall: r_s <= 2, so a row of the disk has at most five pixels: the row is
+// unrolled with its loads side by side (a member outside the disk adds zero,
+// which leaves the sums' bits as they are).
+template <bool kSmall, typename F>
+__device__ __forceinline__ void for_disk(const MpWs &m, const MpCfg &c, float u, float v, F &&f) {
+  const float rs2 = c.r_s * c.r_s;
+#pragma unroll
+  for (int s = 0; s < kMaxScales; ++s) {
+    if (s >= c.scales) break;
+    const float sc = 1.f / (float)(1 << s);              // 2^-s: exact
+    const float us = u * sc, vs = v * sc;
+    const int Ws = m.lw[s];
+    int i0, i1, j0, j1;
+    if (!disk_rect(us, vs, Ws, m.lh[s], c.r_s, &i0, &i1, &j0, &j1)) continue;
+    for (int jj = j0; jj <= j1; ++jj) {
+      const size_t row = (size_t)jj * Ws;
+      const float dy = (float)jj - vs;
+      if (kSmall) {
+#pragma unroll
+        for (int t = 0; t < 5; ++t) {
+          const int ii = i0 + t;
+          const float dx = (float)ii - us, d2 = dx * dx + dy * dy;
+          f(sc, d2, row + (size_t)min(ii, i1), s, ii <= i1 && !(d2 > rs2));
+        }
+      } else {
+        for (int ii = i0; ii <= i1; ++ii) {
+          const float dx = (float)ii - us, d2 = dx * dx + dy * dy;
+          if (!(d2 > rs2)) f(sc, d2, row + (size_t)ii, s, true);
+        }
+      }
+    }
+  }
+}
+
+// A thread per Gaussian, bound by the latency of the gathers (up to 13 pixels x
+// 3 levels x 5 loads). Maps are appended frame by frame, so Gaussians in view
+// come in runs and fill their warps: compacting them per CTA first made the
+// CTAs uneven (300k Gaussians: 42 us against 17).
+template <bool kSmall>
 __global__ void __launch_bounds__(kMpBlock)
-mp_gauss_kernel(MpWs m, const float4 *__restrict__ gauss, int64_t n, const double *__restrict__ pose,
-                const float *__restrict__ image, Raster r, MpCfg c) {
+mp_gauss_kernel(MpWs m, const float4 *__restrict__ gauss, int64_t n, const double *__restrict__ pose, Raster r,
+                MpCfg c) {
   pdl_wait();
   __shared__ float sp[12];
-  __shared__ uint32_t s_min, s_max, s_cnt;
+  __shared__ uint32_t s_min, s_max, s_obs, s_base;
   const float *__restrict__ mpsrc = m.mp_map ? m.mp_map : m.mpf;
+  const int lane = threadIdx.x & 31;
   if (threadIdx.x < 12) sp[threadIdx.x] = (float)pose[threadIdx.x];
-  if (threadIdx.x == 0) { s_min = 0xFFFFFFFFu; s_max = 0u; s_cnt = 0u; }
+  if (threadIdx.x == 0) { s_min = 0xFFFFFFFFu; s_max = 0u; s_obs = 0u; }
   __syncthreads();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  bool observed = false;
+  float mhat = 0.f, sige = 0.f, U = 0.f, M0 = 0.f;
   if (i < n) {
-    const float4 g0 = __ldg(gauss + 4 * i), g2 = __ldg(gauss + 4 * i + 2);
+    const float4 g0 = __ldg(gauss + 4 * i);
     const float x = sp[0] * g0.x + sp[1] * g0.y + sp[2] * g0.z + sp[3];
     const float y = sp[4] * g0.x + sp[5] * g0.y + sp[6] * g0.z + sp[7];
     const float z = depth_key(g0, sp);
-    bool observed = false;
-    float mhat = 0.f, var = 0.f, sige = 0.f;
     const float u = r.fx * x / z + r.cx, v = r.fy * y / z + r.cy;
     if (z > c.z_near) {
-      const float rs2 = c.r_s * c.r_s, inv2s2 = 1.f / (2.f * c.sigma_w * c.sigma_w);
+      const float inv2s2 = 1.f / (2.f * c.sigma_w * c.sigma_w);
       float sw = 0.f, swm = 0.f, sm = 0.f, se = 0.f, dmax = -INFINITY;
       int cnt = 0;
-#pragma unroll
-      for (int s = 0; s < kMaxScales; ++s) {
-        if (s >= c.scales) break;
-        const float sc = 1.f / (float)(1 << s);              // 2^-s: exact
-        const float us = u * sc, vs = v * sc;
-        const int Ws = m.lw[s];
-        int i0, i1, j0, j1;
-        if (!disk_rect(us, vs, Ws, m.lh[s], c.r_s, &i0, &i1, &j0, &j1)) continue;
-        const float *__restrict__ lm = s == 0 ? mpsrc : m.lm[s];
-        const float *__restrict__ le = m.le[s], *__restrict__ ld = m.ld[s];
-        for (int jj = j0; jj <= j1; ++jj)
-          for (int ii = i0; ii <= i1; ++ii) {
-            const float dx = (float)ii - us, dy = (float)jj - vs, d2 = dx * dx + dy * dy;
-            if (d2 > rs2) continue;
-            const size_t p = (size_t)jj * Ws + ii;
-            const float e = le[p];
-            const float mp = lm[p];
-            const float w = sc * expf(-d2 * inv2s2);
-            sw += w; swm += w * mp; sm += mp; se += e; ++cnt;
-            dmax = fmaxf(dmax, ld[p]);
-          }
-      }
+      for_disk<kSmall>(m, c, u, v, [&](float sc, float d2, size_t p, int s, bool ok) {
+        const float e = ok ? m.le[s][p] : 0.f;
+        const float mp = ok ? (s == 0 ? mpsrc : m.lm[s])[p] : 0.f;
+        const float d = ok ? m.ld[s][p] : -INFINITY;
+        const float w = ok ? sc * expf(-d2 * inv2s2) : 0.f;
+        sw += w; swm += w * mp; sm += mp; se += e; cnt += ok;
+        dmax = fmaxf(dmax, d);
+      });
       observed = cnt > 0 && !(c.vis_tol > 0.f && dmax > 0.f && z > dmax + c.vis_tol);
       if (observed) {
         mhat = swm / sw;
         const float mm = sm / cnt, me = se / cnt;
         float vm = 0.f, ve = 0.f;
-#pragma unroll
-        for (int s = 0; s < kMaxScales; ++s) {
-          if (s >= c.scales) break;
-          const float sc = 1.f / (float)(1 << s);
-          const float us = u * sc, vs = v * sc;
-          const int Ws = m.lw[s];
-          int i0, i1, j0, j1;
-          if (!disk_rect(us, vs, Ws, m.lh[s], c.r_s, &i0, &i1, &j0, &j1)) continue;
-          const float *__restrict__ lm = s == 0 ? mpsrc : m.lm[s];
-          const float *__restrict__ le = m.le[s];
-          for (int jj = j0; jj <= j1; ++jj)
-            for (int ii = i0; ii <= i1; ++ii) {
-              const float dx = (float)ii - us, dy = (float)jj - vs;
-              if (dx * dx + dy * dy > rs2) continue;
-              const size_t p = (size_t)jj * Ws + ii;
-              const float e = le[p];
-              const float mp = lm[p];
-              vm += (mp - mm) * (mp - mm);
-              ve += (e - me) * (e - me);
-            }
-        }
-        var = vm / cnt;
+        for_disk<kSmall>(m, c, u, v, [&](float, float, size_t p, int s, bool ok) {
+          const float de = ok ? m.le[s][p] - me : 0.f;
+          const float dm = ok ? (s == 0 ? mpsrc : m.lm[s])[p] - mm : 0.f;
+          vm += dm * dm;
+          ve += de * de;
+        });
         sige = sqrtf(ve / cnt);
+        M0 = __ldg(reinterpret_cast<const float *>(gauss + 4 * i) + 11);
+        U = -M0 * logf(M0 + c.eps) - (1.f - M0) * logf(1.f - M0 + c.eps) + c.lam_u * (vm / cnt);
+        atomicMin(&s_min, f2o(U));
+        atomicMax(&s_max, f2o(U));
       }
     }
-    float U = 0.f;
-    if (observed) {
-      const float M0 = g2.w;
-      U = -M0 * logf(M0 + c.eps) - (1.f - M0) * logf(1.f - M0 + c.eps) + c.lam_u * var;
-      atomicMin(&s_min, f2o(U));
-      atomicMax(&s_max, f2o(U));
-      atomicAdd(&s_cnt, 1u);
-    }
-    m.obs[i] = observed ? 1 : 0;
-    m.mhat[i] = mhat;
-    m.sige[i] = sige;
-    m.U[i] = U;
   }
+  const unsigned b = __ballot_sync(0xffffffffu, observed);
+  uint32_t at = 0u;
+  if (lane == 0 && b) at = atomicAdd(&s_obs, (uint32_t)__popc(b));
+  at = __shfl_sync(0xffffffffu, at, 0) + __popc(b & ((1u << lane) - 1u));
   __syncthreads();
-  if (threadIdx.x == 0 && s_cnt) {
+  if (threadIdx.x == 0 && s_obs) {
     atomicMin(&m.sel[1], s_min);
     atomicMax(&m.sel[2], s_max);
-    atomicAdd(&m.sel[0], s_cnt);
+    s_base = atomicAdd(&m.sel[0], s_obs);
+  }
+  __syncthreads();
+  if (observed) {
+    const size_t q = (size_t)s_base + at;
+    m.idx[q] = (uint32_t)i;
+    m.U[q] = U;
+    m.sige[q] = sige;
+    m.mhat[q] = mhat;
+    m.Mt[q] = M0;
   }
 }
 
-// One warp finds, for rank r, the bin b with cum(b - 1) <= r < cum(b) of a
-// kSelBins histogram; returns b and writes the rank within the bin.
-__device__ __forceinline__ int find_bin(const uint32_t *hist, uint32_t r, uint32_t *r_in_bin) {
-  const int lane = threadIdx.x & 31;
-  constexpr int per = kSelBins / 32;
-  uint32_t mine = 0;
-  for (int b = 0; b < per; ++b) mine += __ldcg(hist + lane * per + b);
+constexpr int kApplyBlock = 1024;
+constexpr int kApplyHeld = 8;      // list entries that a thread keeps in registers
+constexpr int kBarrierSpins = 1 << 22;
+
+// All CTAs of the grid (a cooperative launch) have arrived `round` times;
+// false if one did not within the spin limit.
+__device__ bool grid_barrier(uint32_t *arrivals, uint32_t round, uint32_t *status) {
+  __shared__ int s_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(arrivals, 1u);
+    bool ok = false;
+    for (int it = 0; it < kBarrierSpins && !ok; ++it) {
+      uint32_t v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(arrivals) : "memory");
+      ok = v >= round * gridDim.x;
+    }
+    if (!ok) atomicOr(status, kStatusTimeout);
+    __threadfence();
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
+// Radix-select level l of the floats' bits: 31-21, 20-10, 9-0.
+__device__ __forceinline__ int select_shift(int level) { return level == 0 ? 21 : level == 1 ? 10 : 0; }
+
+// For the ranks rank[0], rank[1]: the bins of the two histograms (kSelBins
+// each, contiguous) that hold them, and the ranks within those bins. The
+// CTA's halves take a histogram each, a thread four bins.
+__device__ void find_bins(const uint32_t *hist, uint32_t *rank, uint32_t *bin) {
+  __shared__ uint32_t s_sum[32], s_bin[2], s_rank[2];
+  const int h = threadIdx.x / (kApplyBlock / 2), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  static_assert(kSelBins == 4 * (kApplyBlock / 2), "four bins per thread");
+  const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(hist) + threadIdx.x);
+  const uint32_t mine = v.x + v.y + v.z + v.w;
   uint32_t inc = mine;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
     if (lane >= o) inc += y;
   }
-  const uint32_t before = inc - mine;
-  const unsigned hit = __ballot_sync(0xffffffffu, before <= r && r < inc);
-  const int owner = __ffs(hit) - 1;
-  int bin = -1;
-  uint32_t rr = 0;
-  if (lane == owner) {
-    uint32_t run = before;
-    for (int b = 0; b < per; ++b) {
-      const uint32_t hcount = __ldcg(hist + lane * per + b);
-      if (r < run + hcount) { bin = lane * per + b; rr = r - run; break; }
-      run += hcount;
-    }
-  }
-  bin = __shfl_sync(0xffffffffu, bin, owner < 0 ? 0 : owner);
-  rr = __shfl_sync(0xffffffffu, rr, owner < 0 ? 0 : owner);
-  *r_in_bin = rr;
-  return bin;
-}
-
-// Level-l radix select step over the observed Gaussians' (M^t, U_tilde):
-// level 0 uses bits 31-21, level 1 bits 20-10, level 2 bits 9-0.
-__device__ __forceinline__ void select_shift(int level, int *shift, uint32_t *mask) {
-  *shift = level == 0 ? 21 : (level == 1 ? 10 : 0);
-  *mask = level == 2 ? 0x3FFu : 0x7FFu;
-}
-
-__device__ bool last_cta(uint32_t *counter) {
-  __shared__ int s_last;
+  if (lane == 31) s_sum[warp] = inc;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned t = atomicAdd(counter, 1u);
-    s_last = (t == gridDim.x - 1);
-    if (s_last) __threadfence();
+  uint32_t before = inc - mine;
+  for (int w = 16 * h; w < warp; ++w) before += s_sum[w];
+  const uint32_t r = rank[h];
+  if (before <= r && r < before + mine) {
+    uint32_t b = 4u * (threadIdx.x % (kApplyBlock / 2)), run = before;
+    const uint32_t cnt[3] = {v.x, v.y, v.z};
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (b % 4u == (uint32_t)k && r >= run + cnt[k]) { run += cnt[k]; ++b; }
+    s_bin[h] = b;
+    s_rank[h] = r - run;
   }
   __syncthreads();
-  return s_last != 0;
-}
-
-// After a histogram level: the last CTA finds both medians' bins, advances
-// their prefixes and remaining ranks, clears the histograms; after the last
-// level it writes the statistics.
-__device__ void select_finish(const MpWs &m, int level, const MpCfg &c) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp < 2) {
-    const uint32_t nobs = __ldcg(m.sel + 0);
-    if (nobs > 0) {
-      const uint32_t rank = level == 0 ? (nobs - 1) / 2 : __ldcg(m.sel + 6 + warp);
-      uint32_t rin = 0;
-      const int bin = find_bin(m.hist + warp * kSelBins, rank, &rin);
-      int shift;
-      uint32_t mask;
-      select_shift(level, &shift, &mask);
-      if (lane == 0) {
-        const uint32_t prefix = (level == 0 ? 0u : __ldcg(m.sel + 4 + warp)) | ((uint32_t)bin << shift);
-        m.sel[4 + warp] = prefix;
-        m.sel[6 + warp] = rin;
-      }
-    }
-  }
+  for (int k = 0; k < 2; ++k) { bin[k] = s_bin[k]; rank[k] = s_rank[k]; }
   __syncthreads();
-  for (int k = threadIdx.x; k < 2 * kSelBins; k += blockDim.x) m.hist[k] = 0u;
-  if (level == 2 && threadIdx.x == 0) {
-    const uint32_t nobs = __ldcg(m.sel + 0);
-    const float medM = nobs ? __uint_as_float(__ldcg(m.sel + 4)) : nanf("");
-    const float medU = nobs ? __uint_as_float(__ldcg(m.sel + 5)) : 0.f;
-    m.stats[0] = nobs ? fmax((double)medM, (double)c.tau_floor) : (double)c.tau_floor;
-    m.stats[1] = medU;
-    m.stats[2] = medM;
-    m.stats[3] = nobs ? (double)o2f(__ldcg(m.sel + 1)) : 0.0;
-    m.stats[4] = nobs ? (double)o2f(__ldcg(m.sel + 2)) : 0.0;
-    m.stats[5] = (double)nobs;
-  }
-  if (threadIdx.x == 0) m.sel[3] = 0u;
 }
 
-__global__ void __launch_bounds__(kMpBlock)
-mp_apply_kernel(MpWs m, float4 *__restrict__ gauss, int64_t n, MpCfg c) {
-  pdl_wait();
+// The list is read once; each thread keeps its entries' M^t and U_tilde in
+// registers over the three select levels and the labels (entries past
+// kApplyHeld per thread, above 1.2M observed, are read again). Every CTA finds
+// the bins for itself after a barrier, so that no level waits for one CTA.
+// In place of five launches that each walked all N Gaussians and ended on one
+// CTA's serial search: 51 -> 23 us at 300k Gaussians, each launch alone.
+__global__ void __launch_bounds__(kApplyBlock, 1)
+mp_apply_kernel(MpWs m, float *__restrict__ gauss, uint8_t *__restrict__ labels, MpCfg c) {
   __shared__ uint32_t s_h[2 * kSelBins];
-  for (int k = threadIdx.x; k < 2 * kSelBins; k += blockDim.x) s_h[k] = 0u;
-  __syncthreads();
+  const uint32_t nobs = m.sel[0];
   const float umin = o2f(m.sel[1]), umax = o2f(m.sel[2]);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    if (!m.obs[i]) continue;
-    const float ut = umax > umin ? (m.U[i] - umin) / (umax - umin) : 0.f;
-    const float C = expf(-m.sige[i] / c.sigma_c);
+  const size_t T = (size_t)gridDim.x * kApplyBlock, first = (size_t)blockIdx.x * kApplyBlock + threadIdx.x;
+  if (blockIdx.x == gridDim.x - 1)
+    for (int k = threadIdx.x; k < c.n_regions; k += kApplyBlock) {
+      float4 reg;
+      region_params(m, c, k, &reg);
+      const double cnt = m.acc[4 * k + 0];
+      double *o = m.stats + DAGS_MP_STATS_HEAD + 4 * k;
+      o[0] = cnt;
+      o[1] = cnt > 0.0 ? m.acc[4 * k + 1] / cnt : 0.0;
+      o[2] = cnt > 0.0 ? sqrt(m.acc[4 * k + 2] / cnt) : 0.0;
+      o[3] = reg.y;
+    }
+  if (nobs == 0u) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      m.stats[0] = (double)c.tau_floor;
+      m.stats[1] = 0.0;
+      m.stats[2] = nanf("");
+      m.stats[3] = m.stats[4] = m.stats[5] = 0.0;
+    }
+    return;
+  }
+  uint32_t id[kApplyHeld];
+  float Mt[kApplyHeld], Ut[kApplyHeld];
+  auto apply = [&](size_t q, uint32_t *i, float *M, float *Un) {
+    const float ut = umax > umin ? (m.U[q] - umin) / (umax - umin) : 0.f;
+    const float C = expf(-m.sige[q] / c.sigma_c);
     float a = c.alpha_min + (c.alpha_max - c.alpha_min) * (1.f - ut) * C;
     a = fminf(fmaxf(a, c.alpha_min), c.alpha_max);
     if (!c.seg_refreshed) a *= c.rho;
-    float *rec = reinterpret_cast<float *>(gauss + 4 * i);
-    const float M0 = rec[11];
-    const float Mt = (1.f - a) * M0 + a * m.mhat[i];
-    rec[11] = Mt;
-    m.Mt[i] = Mt;
-    m.Ut[i] = ut;
-    atomicAdd(&s_h[__float_as_uint(Mt) >> 21], 1u);
-    atomicAdd(&s_h[kSelBins + (__float_as_uint(ut) >> 21)], 1u);
+    *i = m.idx[q];
+    *Un = ut;
+    *M = (1.f - a) * m.Mt[q] + a * m.mhat[q];
+    gauss[16 * (size_t)*i + 11] = *M;
+  };
+#pragma unroll
+  for (int j = 0; j < kApplyHeld; ++j) {
+    const size_t q = first + j * T;
+    id[j] = 0u;
+    Mt[j] = Ut[j] = 0.f;
+    if (q < nobs) apply(q, &id[j], &Mt[j], &Ut[j]);
   }
-  __syncthreads();
-  for (int k = threadIdx.x; k < 2 * kSelBins; k += blockDim.x)
-    if (s_h[k]) atomicAdd(&m.hist[k], s_h[k]);
-  if (last_cta(m.sel + 3)) select_finish(m, 0, c);
-}
-
-__global__ void __launch_bounds__(kMpBlock)
-mp_select_kernel(MpWs m, int64_t n, int level, MpCfg c) {
-  pdl_wait();
-  __shared__ uint32_t s_h[2 * kSelBins];
-  for (int k = threadIdx.x; k < 2 * kSelBins; k += blockDim.x) s_h[k] = 0u;
-  __syncthreads();
-  int shift;
-  uint32_t mask;
-  select_shift(level, &shift, &mask);
-  const int top = shift + (level == 2 ? 10 : 11);   // bits above this level are the prefix
-  const uint32_t pm = m.sel[4], pu = m.sel[5];
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    if (!m.obs[i]) continue;
-    const uint32_t bm = __float_as_uint(m.Mt[i]), bu = __float_as_uint(m.Ut[i]);
-    if ((bm >> top) == (pm >> top)) atomicAdd(&s_h[(bm >> shift) & mask], 1u);
-    if ((bu >> top) == (pu >> top)) atomicAdd(&s_h[kSelBins + ((bu >> shift) & mask)], 1u);
+  for (size_t q = first + kApplyHeld * T; q < nobs; q += T) {
+    uint32_t i;
+    float M, Un;
+    apply(q, &i, &M, &Un);
+    m.Mt[q] = M;
+    m.Ut[q] = Un;
   }
-  __syncthreads();
-  for (int k = threadIdx.x; k < 2 * kSelBins; k += blockDim.x)
-    if (s_h[k]) atomicAdd(&m.hist[k], s_h[k]);
-  if (last_cta(m.sel + 3)) select_finish(m, level, c);
-}
-
-__global__ void __launch_bounds__(kMpBlock)
-mp_labels_kernel(MpWs m, int64_t n, uint8_t *__restrict__ labels) {
-  pdl_wait();
-  const double tau = m.stats[0];
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    if (m.obs[i]) labels[i] = (double)m.Mt[i] > tau ? 1 : 0;
-}
-
-__global__ void mp_region_stats_kernel(MpWs m, MpCfg c) {
-  pdl_wait();
-  for (int k = threadIdx.x; k < c.n_regions; k += blockDim.x) {
-    float4 reg;
-    region_params(m, c, k, &reg);
-    const double cnt = m.acc[4 * k + 0];
-    double *o = m.stats + DAGS_MP_STATS_HEAD + 4 * k;
-    o[0] = cnt;
-    o[1] = cnt > 0.0 ? m.acc[4 * k + 1] / cnt : 0.0;
-    o[2] = cnt > 0.0 ? sqrt(m.acc[4 * k + 2] / cnt) : 0.0;
-    o[3] = reg.y;
+  uint32_t rank[2] = {(nobs - 1u) / 2u, (nobs - 1u) / 2u}, prefix[2] = {0u, 0u};
+  for (int level = 0; level < kSelLevels; ++level) {
+    for (int k = threadIdx.x; k < 2 * kSelBins; k += kApplyBlock) s_h[k] = 0u;
+    __syncthreads();
+    const int shift = select_shift(level);
+    const uint32_t mask = level == 2 ? 0x3FFu : 0x7FFu;
+    auto count = [&](float M, float Un) {
+      // the bits above this level equal the prefix
+      const uint32_t bm = __float_as_uint(M), bu = __float_as_uint(Un);
+      if (level == 0 || ((bm ^ prefix[0]) >> shift) <= mask) atomicAdd(&s_h[(bm >> shift) & mask], 1u);
+      if (level == 0 || ((bu ^ prefix[1]) >> shift) <= mask) atomicAdd(&s_h[kSelBins + ((bu >> shift) & mask)], 1u);
+    };
+#pragma unroll
+    for (int j = 0; j < kApplyHeld; ++j)
+      if (first + j * T < nobs) count(Mt[j], Ut[j]);
+    for (size_t q = first + kApplyHeld * T; q < nobs; q += T) count(m.Mt[q], m.Ut[q]);
+    __syncthreads();
+    uint32_t *hist = m.hist + level * 2 * kSelBins;
+    for (int k = threadIdx.x; k < 2 * kSelBins; k += kApplyBlock)
+      if (s_h[k]) atomicAdd(&hist[k], s_h[k]);
+    if (!grid_barrier(m.sel + 3, (uint32_t)level + 1u, m.status)) return;
+    uint32_t bin[2];
+    find_bins(hist, rank, bin);
+    prefix[0] |= bin[0] << shift;
+    prefix[1] |= bin[1] << shift;
   }
+  const float medM = __uint_as_float(prefix[0]);
+  const double tau = fmax((double)medM, (double)c.tau_floor);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    m.stats[0] = tau;
+    m.stats[1] = __uint_as_float(prefix[1]);
+    m.stats[2] = medM;
+    m.stats[3] = (double)umin;
+    m.stats[4] = (double)umax;
+    m.stats[5] = (double)nobs;
+  }
+#pragma unroll
+  for (int j = 0; j < kApplyHeld; ++j)
+    if (first + j * T < nobs) labels[id[j]] = (double)Mt[j] > tau ? 1 : 0;
+  for (size_t q = first + kApplyHeld * T; q < nobs; q += T) labels[m.idx[q]] = (double)m.Mt[q] > tau ? 1 : 0;
 }
 
 // Semantic-on-demand trigger, Eqs. (13)-(16): one thread reads the frame's
@@ -605,7 +621,7 @@ cudaError_t launch_mp_update(const MpBuffers &b, float *gauss, int64_t n, const 
   m.mp_pixel = mp_pixel;
   m.mpf = b.mpf;
   m.e = b.e; m.acc = b.acc; m.mhat = b.mhat; m.sige = b.sige; m.U = b.U; m.Mt = b.Mt; m.Ut = b.Ut;
-  m.obs = b.obs; m.hist = b.hist; m.sel = b.sel; m.stats = stats;
+  m.idx = b.idx; m.hist = b.hist; m.sel = b.sel; m.stats = stats;
   MpCfg c;
   c.kappa_c = cfg.kappa_c; c.lam = cfg.lam; c.sigma_min = cfg.sigma_min; c.e_floor = cfg.e_floor;
   c.sigma_g = cfg.sigma_g; c.sigma_c = cfg.sigma_c; c.lam_u = cfg.lam_u; c.eps = cfg.eps;
@@ -642,10 +658,8 @@ cudaError_t launch_mp_update(const MpBuffers &b, float *gauss, int64_t n, const 
   if (e != cudaSuccess) return e;
   const unsigned gp = (unsigned)((P + kMpBlock - 1) / kMpBlock);
   const unsigned gg = (unsigned)((n + kMpBlock - 1) / kMpBlock > 0 ? (n + kMpBlock - 1) / kMpBlock : 1);
-  // the histogram passes (median selection) and the labels: two CTAs per SM
-  // striding over the Gaussians, so that each CTA's clearing and flushing of
-  // its 2 x 2048 shared bins is spread over several Gaussians per thread
-  const unsigned gs = gg < 2u * (unsigned)num_sms ? gg : 2u * (unsigned)num_sms;
+  const int64_t blocks = (n + kApplyBlock - 1) / kApplyBlock;
+  const unsigned ga = (unsigned)(blocks < 1 ? 1 : blocks < num_sms ? blocks : num_sms);
   mp_pixel_sum_kernel<<<gp, kMpBlock, 0, s>>>(m, targets, image, inst, P, c);
   if (e == cudaSuccess) e = launch_pdl(mp_pixel_var_kernel, dim3(gp), dim3(kMpBlock), 0, s, m, inst, P, c);
   if (!mp_map || mp_pixel)
@@ -659,14 +673,21 @@ cudaError_t launch_mp_update(const MpBuffers &b, float *gauss, int64_t n, const 
                      pyr_out[l][0], pyr_out[l][1], pyr_out[l][2]);
   }
   if (e == cudaSuccess)
-    e = launch_pdl(mp_gauss_kernel, dim3(gg), dim3(kMpBlock), 0, s, m, reinterpret_cast<const float4 *>(gauss), n,
-                   pose, image, r, c);
-  if (e == cudaSuccess)
-    e = launch_pdl(mp_apply_kernel, dim3(gs), dim3(kMpBlock), 0, s, m, reinterpret_cast<float4 *>(gauss), n, c);
-  if (e == cudaSuccess) e = launch_pdl(mp_select_kernel, dim3(gs), dim3(kMpBlock), 0, s, m, n, 1, c);
-  if (e == cudaSuccess) e = launch_pdl(mp_select_kernel, dim3(gs), dim3(kMpBlock), 0, s, m, n, 2, c);
-  if (e == cudaSuccess) e = launch_pdl(mp_labels_kernel, dim3(gs), dim3(kMpBlock), 0, s, m, n, labels);
-  if (e == cudaSuccess) e = launch_pdl(mp_region_stats_kernel, dim3(1), dim3(256), 0, s, m, c);
+    e = launch_pdl(c.r_s <= 2.f ? mp_gauss_kernel<true> : mp_gauss_kernel<false>, dim3(gg), dim3(kMpBlock), 0, s, m,
+                   reinterpret_cast<const float4 *>(gauss), n, pose, r, c);
+  if (e == cudaSuccess) {
+    // cooperative: its CTAs (one per SM at most) wait for one another
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ga);
+    cfg.blockDim = dim3(kApplyBlock);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, mp_apply_kernel, m, gauss, labels, c);
+  }
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
