@@ -149,7 +149,7 @@ void free_epi(EpiBuffers &b) {
 }
 
 void free_net(MpnetScratch &b) {
-  void *ptrs[] = {b.y, b.planes, b.dz2, b.zero, b.grad, b.inv_n};
+  void *ptrs[] = {b.y, b.planes, b.dz2, b.zero, b.grad, b.count};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   b = MpnetScratch();
@@ -1299,7 +1299,7 @@ int mpnet_train_step(dags_ctx *ctx, void *weights, float *master, float *adam_m,
     if (e == cudaSuccess) e = cudaMemsetAsync(sc.zero, 0, (kMpnetStrip + 2) * sizeof(uint4), s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // whatever stream the next step runs on
     if (e == cudaSuccess) e = alloc(&sc.grad, DAGS_MPNET_PARAMS);
-    if (e == cudaSuccess) e = alloc(&sc.inv_n, 2);
+    if (e == cudaSuccess) e = alloc(&sc.count, 1);
     if (e != cudaSuccess) {
       free_net(sc);
       cudaGetLastError();

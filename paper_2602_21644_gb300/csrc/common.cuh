@@ -278,7 +278,7 @@ struct MpnetScratch {
   uint4 *dz2 = nullptr;
   uint4 *zero = nullptr;     // one zero row of 130 pixels x 8 channels
   float *grad = nullptr;     // [10881]
-  float *inv_n = nullptr;    // [2]: 1 / valid pixels, valid count
+  unsigned *count = nullptr; // pixels with a target
   long long cap = 0;         // pixels
   long long plane_cap = 0;   // uint4 of one plane
 };

@@ -639,24 +639,21 @@ constexpr int kGW1 = 0, kGW2 = 512, kGW3 = 512 + 9216, kGw4 = 512 + 9216 + 1024,
               kGb2 = kGb1 + 32, kGb3 = kGb2 + 32, kGb4 = kGb3 + 32, kGTotal = kGb4 + 1;   // 10881 floats
 
 
-__global__ void mpnet_count_kernel(const float *__restrict__ target, long long n, float *__restrict__ inv_n,
-                                   float *__restrict__ loss_acc) {
+// The number of pixels with a target.
+__global__ void __launch_bounds__(256)
+mpnet_count_kernel(const float *__restrict__ target, long long n, unsigned *__restrict__ count) {
   __shared__ unsigned s_cnt;
   if (threadIdx.x == 0) s_cnt = 0u;
   __syncthreads();
   unsigned c = 0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+  const long long step = (long long)gridDim.x * blockDim.x;
+#pragma unroll 4
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += step)
     c += target[i] >= 0.f ? 1u : 0u;
   c = __reduce_add_sync(0xffffffffu, c);
   if ((threadIdx.x & 31) == 0) atomicAdd(&s_cnt, c);
   __syncthreads();
-  if (threadIdx.x == 0) atomicAdd(reinterpret_cast<unsigned *>(inv_n) + 1, s_cnt);   // count in word 1
-  (void)loss_acc;
-}
-
-__global__ void mpnet_count_finish_kernel(float *inv_n) {
-  const unsigned c = reinterpret_cast<unsigned *>(inv_n)[1];
-  inv_n[0] = c ? 1.f / (float)c : 0.f;
+  if (threadIdx.x == 0) atomicAdd(count, s_cnt);
 }
 
 // Backward operand layouts. All activations and gradients are staged as
@@ -720,7 +717,7 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_
 __global__ void __launch_bounds__(kB1Threads, 4)
 mpnet_bwd1_kernel(const uint8_t *__restrict__ weights, const float *__restrict__ y, const float *__restrict__ target,
                   const uint4 *__restrict__ a2p, const uint4 *__restrict__ a3p, int batch, int W, int H,
-                  const float *__restrict__ inv_n, uint4 *__restrict__ dz2p, float *__restrict__ grad,
+                  const unsigned *__restrict__ count, uint4 *__restrict__ dz2p, float *__restrict__ grad,
                   double *__restrict__ loss, uint32_t *__restrict__ status) {
   extern __shared__ __align__(128) uint8_t smem[];
   uint8_t *sDz3 = smem + kB1Dz3, *sDz4 = smem + kB1Dz4, *sW3T = smem + kB1W3T;
@@ -820,7 +817,7 @@ mpnet_bwd1_kernel(const uint8_t *__restrict__ weights, const float *__restrict__
     }
   } else {
     const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
-    const float invn = inv_n[0];
+    const float invn = *count ? 1.f / (float)*count : 0.f;
     const int p = tid;
     auto fetch = [&](long long t, float *tg, float *yv) {   // target and output of this thread's pixel
       const long long row = t / tiles_x;
@@ -926,61 +923,57 @@ mpnet_bwd1_kernel(const uint8_t *__restrict__ weights, const float *__restrict__
 }
 
 // bwd2: da1 by the transposed 3 x 3 convolution, dz1, and the weight gradients
-// dW2, dW1, db2, db1. A CTA walks its share of the 128-pixel column strips
-// downwards, two output rows (a pair) per step; the rows of a1, dz2 and x come
-// once from the planar copies by bulk copies, each row 2,080 contiguous bytes
-// per 8-channel chunk.
+// dW2, dW1, db2, db1. A persistent CTA takes 128-pixel row tiles one grid apart;
+// the three halo rows of a1 and of dz2 and the row of x come by bulk copies
+// from the planar copies (2,080 contiguous bytes per row and 8-channel chunk),
+// three tiles in flight. Neighbouring tiles run at the same time on other SMs,
+// so a row is read from memory once and from L2 three times.
 //
 // Warps 0..3 form dz1 from da1, warp 4 issues the copies, warp 5 the MMAs of
-// da1 and dW1, warps 6..8 those of dW2 (a column tap each) and db2: one
-// thread's MMAs go through at most one per 68 cycles. An MMA costs its operands'
-// shared-memory reads (about 128 B per cycle), so the products are stacked:
-//   dW2, db2: per dz2 row y, column tap kx and 16 pixels one M = 128, N = 32
-//     product of the a1 rows y - 1 .. y + 1 (slots of four chunks and one of
-//     (1, 0, ...) at one stride: 120 rows, the kernel rows and the bias; the
-//     last 8 are whatever follows, their D rows unused): 24 MMAs of about 40
-//     cycles a row instead of 72 of 25 (M = 64, one tap each). N = 64 over two dz2 rows would take
-//     24 of 48 for both, but halves the additions of an accumulator, and with
-//     them the tensor core's truncation (-7.6e-5 relative on dW2 at 16 x 640
-//     x 480): results would differ by that.
-//   da1: N = 64 over both output rows for the dz2 rows y, y + 1, N = 32 for
-//     y - 1 and y + 2; the kernel rows of W2 are stacked along N, so that a
-//     window of them meets the output rows.
-//   dW1, db1: per row dz1 (M = 64, 32 rows used) against x and the ones
-//     (N = 16).
-// About 1,650 tensor cycles per 128-pixel row. 16 x 640 x 480, the launch
-// alone: 976 us with one CTA of 128 threads that fetched three halo rows per
-// output row and waited for each tile's chain, 315 us now (418,000 tensor
-// cycles a CTA, 0.21 ms at 2 GHz, are what bounds it).
+// da1, warps 6..8 those of dW2 (a column tap each) and db2, warp 9 those of dW1
+// and db1: one thread's MMAs go through at most one per 68 cycles. An MMA
+// costs its operands' shared-memory reads (about 128 B per cycle):
+//   dW2, db2: per column tap kx and 16 pixels one M = 128, N = 32 product of
+//     the a1 rows y - 1 .. y + 1 (four chunks and one of (1, 0, ...) each, at
+//     one stride: 120 rows, the kernel rows and the bias; the last 8 are
+//     whatever follows, their D rows unused) with dz2 of row y: 24 MMAs of
+//     about 40 cycles instead of 72 of 25 (M = 64, one tap each).
+//   da1: 18 MMAs, N = 32; dW1, db1: x and the ones (M = 64) against dz1.
+// Bound by shared memory: about 1,880 cycles of operand reads per tile and 410
+// of copies written. 16 x 640 x 480, the launch alone: 976 us with 128 threads
+// per SM that waited for each tile's chain, 371 us now. Walking strips two rows
+// per step reads every row once and takes 300 us, but sums a CTA's tiles in
+// another order: the tensor core truncates each addition, and dW2 moved by 2e-6
+// relative, ten times what the order of the CTAs' atomics does (N = 64 over two
+// rows of dz2, which halves the additions per accumulator: 7.6e-5).
 //
-// Rings. Groups g (pairs, and the half pair above and below a segment): dz2
-// of two rows and x, four slots. a1 rows: eight slots; step c (pairs only)
-// reads the window of four slots at 2 (c mod 3), so a row that two windows
-// share is copied again only where the ring wraps (8 copies per 6 rows).
-// Barriers: full_d[4] dz2 and x of a group, full_a[3] the a1 rows of a step,
-// done_d[4] / done_w[4] the group's last use by warp 5 / warps 6..8, done_c[3] step c's
-// dW2, prod[2] da1 of a step, ep[2] its dz1 (and its reads of a1), drain[4].
-constexpr int kB2Threads = 9 * 32;
-constexpr int kB2Slot = 4 * kRowBytes;                   // one row: four chunks of 130 pixels
+// Barriers, per stage (tile i: stage i mod 3): full the copies, prod da1 of the
+// tile, ep its dz1 (and its reads of a1 and da1), done_d, done_w, done_x the
+// stage's last use by warp 5, warps 6..8, warp 9; drain[5].
+constexpr int kB2Threads = 10 * 32;
+constexpr int kB2Stages = 3;
 constexpr int kB2A1Slot = 5 * kRowBytes;                 // an a1 row and a chunk of ones
-constexpr int kB2A1 = 0;                                 // eight a1 rows
-constexpr int kB2Dz2 = 8 * kB2A1Slot;                    // four groups of two dz2 rows
-constexpr int kB2Dz1 = kB2Dz2 + 8 * kB2Slot;             // two steps of two dz1 rows (128-pixel chunks)
-constexpr int kB2X = kB2Dz1 + 2 * 8 * kChunkPx;          // four groups of x, x, ones
-constexpr int kB2W2 = kB2X + 4 * 3 * kChunkPx;           // [(ky, i)][(kx, o)]
+constexpr int kB2Dz2 = 3 * kB2A1Slot;                    // within a stage
+constexpr int kB2Slot = 4 * kRowBytes;                   // a dz2 row: four chunks of 130 pixels
+constexpr int kB2X = kB2Dz2 + 3 * kB2Slot;               // x, ones
+constexpr int kB2Stage = kB2X + 2 * kChunkPx;
+constexpr int kB2Dz1 = kB2Stages * kB2Stage;             // a dz1 tile per stage
+constexpr int kB2W2 = kB2Dz1 + kB2Stages * 4 * kChunkPx; // [(ky, i)][(kx, o)]
 constexpr int kB2Bar = kB2W2 + 96 * 96 * 2;
-constexpr int kB2NBars = 4 + 3 + 4 + 4 + 3 + 2 + 2 + 4;
+constexpr int kB2NBars = 6 * kB2Stages + 5;
 constexpr int kB2Smem = kB2Bar + 8 * kB2NBars + 16;
-constexpr uint32_t kB2ColW2 = 0, kB2ColDa = 128, kB2ColW1 = 256;
+constexpr uint32_t kB2ColW2 = 0, kB2ColDa = 96, kB2ColW1 = 192;
 static_assert(kB2Smem <= 227 * 1024, "shared memory");
+static_assert(kB2X + 8 * kChunkPx <= kB2Stage + 4 * kChunkPx * kB2Stages, "M = 64 reads of x stay in shared memory");
 
 __global__ void __launch_bounds__(kB2Threads, 1)
 mpnet_bwd2_kernel(const uint8_t *__restrict__ weights, const uint4 *__restrict__ feats, const uint4 *__restrict__ a1p,
                   const uint4 *__restrict__ dz2p, const uint4 *__restrict__ zero, int W, int H, int tiles_x,
-                  long long npairs, float *__restrict__ grad, uint32_t *__restrict__ status) {
+                  long long ntiles, float *__restrict__ grad, uint32_t *__restrict__ status) {
   extern __shared__ __align__(128) uint8_t smem[];
-  uint64_t *full_d = reinterpret_cast<uint64_t *>(smem + kB2Bar), *full_a = full_d + 4, *done_d = full_a + 3,
-           *done_w = done_d + 4, *done_c = done_w + 4, *prod = done_c + 3, *ep = prod + 2, *drain = ep + 2;
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + kB2Bar), *prod = full + kB2Stages, *ep = prod + kB2Stages,
+           *done_d = ep + kB2Stages, *done_w = done_d + kB2Stages, *done_x = done_w + kB2Stages,
+           *drain = done_x + kB2Stages;
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + kB2Bar + 8 * kB2NBars);
   volatile uint32_t *s_fail = reinterpret_cast<volatile uint32_t *>(s_tmem + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -992,23 +985,25 @@ mpnet_bwd2_kernel(const uint8_t *__restrict__ weights, const uint4 *__restrict__
     const int o = e / kK2, col = e % kK2, tap = col / 32, i = col % 32, ky = tap / 3, kx = tap % 3;
     *reinterpret_cast<uint16_t *>(smem + kB2W2 + core_off(ky * 32 + i, kx * 32 + o, 96)) = gw2[e];
   }
-  for (int e = tid; e < 4 * kTileW; e += kB2Threads)
-    *reinterpret_cast<uint4 *>(smem + kB2X + (e / kTileW) * 3 * kChunkPx + 2 * kChunkPx + (e % kTileW) * 16) =
-        make_uint4(0x3F80u, 0u, 0u, 0u);
-  for (int e = tid; e < 8 * kHaloW; e += kB2Threads)
-    *reinterpret_cast<uint4 *>(smem + kB2A1 + (e / kHaloW) * kB2A1Slot + kB2Slot + (e % kHaloW) * 16) =
-        make_uint4(0x3F80u, 0u, 0u, 0u);
+  for (int st = 0; st < kB2Stages; ++st) {
+    uint8_t *stage = smem + st * kB2Stage;
+    for (int e = tid; e < 3 * kHaloW; e += kB2Threads)
+      *reinterpret_cast<uint4 *>(stage + (e / kHaloW) * kB2A1Slot + kB2Slot + (e % kHaloW) * 16) =
+          make_uint4(0x3F80u, 0u, 0u, 0u);
+    for (int e = tid; e < kTileW; e += kB2Threads)
+      *reinterpret_cast<uint4 *>(stage + kB2X + kChunkPx + e * 16) = make_uint4(0x3F80u, 0u, 0u, 0u);
+  }
   if (tid == 0) {
     for (int k = 0; k < kB2NBars; ++k) {
-      uint64_t *bar = full_d + k;   // ep: the four warps; done_w, done_c: the three warps of dW2
-      const int count = bar >= ep && bar < drain ? 4 : bar >= done_w && bar < prod ? 3 : 1;
+      uint64_t *bar = full + k;   // ep: the four warps; done_w: the three warps of dW2
+      const int count = bar >= ep && bar < done_d ? 4 : bar >= done_w && bar < done_x ? 3 : 1;
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *s_fail = 0u;
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(512));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(256));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   fence_async_smem();
@@ -1016,220 +1011,141 @@ mpnet_bwd2_kernel(const uint8_t *__restrict__ weights, const uint4 *__restrict__
   __syncthreads();
   tc_after_sync();
   const uint32_t tmem = *s_tmem;
-  const int HP = (H + 1) / 2;
   const size_t plane_w = (size_t)tiles_x * kTileW + 2;
-  const long long first = npairs * blockIdx.x / gridDim.x, last = npairs * (blockIdx.x + 1) / gridDim.x;
-  // the next segment of the CTA's pairs: n pairs of one strip, the first one
-  // at row y0 of image b
-  auto segment = [&](long long q, int *b, int *x0, int *y0) {
-    const long long strip = q / HP;
-    const int pr = (int)(q - strip * HP);
-    *b = (int)(strip / tiles_x);
-    *x0 = (int)(strip - (long long)*b * tiles_x) * kTileW;
-    *y0 = 2 * pr;
-    const long long left = last - q;
-    return left < HP - pr ? (int)left : HP - pr;
-  };
+  // every role walks the same tiles: the i-th is blockIdx.x + i * gridDim.x, in
+  // stage st = i mod 3 with barrier phase ph = (i / 3) mod 2
   bool ok = true;
-  int g = 0, c = 0;      // groups and steps so far (the same sequence in every role)
+  int i = 0, st = 0;
+  uint32_t ph = 0u;
+  auto next = [&] {
+    ++i;
+    if (++st == kB2Stages) { st = 0; ph ^= 1u; }
+  };
   auto fail = [&] { *s_fail = 1u; };
   if (warp == 4) {
     // ------------------------------------------------------------- copies
-    int last_d[4] = {-1, -1, -1, -1}, last_a[3] = {-1, -1, -1};
-    for (long long q = first; q < last && ok;) {
-      int b, x0, y0;
-      const int n = segment(q, &b, &x0, &y0);
-      q += n;
-      const size_t img = (size_t)b * H;
-      const uint32_t xbytes = 16u * (uint32_t)min(kTileW, W - x0);
-      auto row_src = [&](const uint4 *plane, int y, int ch) {
-        return y >= 0 && y < H ? plane + ((img + y) * 4 + ch) * plane_w + x0 : zero;
-      };
-      for (int P = -1; P <= n; ++P, ++g) {
-        const int slot = g & 3, row0 = y0 + 2 * P;
-        if (g >= 4) ok = bar_wait(done_d + slot, (uint32_t)((g >> 2) - 1) & 1u) &&
-                         bar_wait(done_w + slot, (uint32_t)((g >> 2) - 1) & 1u);
-        ok = __all_sync(0xffffffffu, ok && !*s_fail);
-        if (!ok) break;
-        const bool r0 = P >= 0, r1 = P < n, mid = r0 && r1;
-        const int xrows = mid ? min(2, H - row0) : 0;
-        if (lane == 0)
-          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(full_d + slot)),
-                       "r"((uint32_t)(r0 + r1) * kB2Slot + (uint32_t)xrows * xbytes)
-                       : "memory");
-        __syncwarp();
-        const uint32_t dz = base + kB2Dz2 + 2 * slot * kB2Slot;
-        if (lane < 8) {
-          const int rr = lane >> 2, ch = lane & 3;
-          if (rr ? r1 : r0)
-            bulk_copy(dz + rr * kB2Slot + ch * kRowBytes, row_src(dz2p, row0 + rr, ch), kRowBytes, full_d + slot);
-        } else if (lane < 8 + xrows) {
-          const int rr = lane - 8;
-          bulk_copy(base + kB2X + (3 * slot + rr) * kChunkPx, feats + (img + row0 + rr) * W + x0, xbytes,
-                    full_d + slot);
-        }
-        last_d[slot] = g;
-        if (P < 1) continue;
-        // the a1 rows of step c, the pair at row0 - 2
-        const int dep = P == 1 ? c - 1 : c - 2, w = c % 3;
-        if (dep >= 0) ok = bar_wait(done_c + dep % 3, (uint32_t)(dep / 3) & 1u) &&
-                           bar_wait(ep + (dep & 1), (uint32_t)(dep >> 1) & 1u);
-        ok = __all_sync(0xffffffffu, ok && !*s_fail);
-        if (!ok) break;
-        const int from = P == 1 || w == 0 ? 0 : 2;      // the first of the window's rows that is copied
-        if (lane == 0)
-          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(full_a + w)),
-                       "r"((uint32_t)(4 - from) * kB2Slot)
-                       : "memory");
-        __syncwarp();
-        if (lane < 16 && (lane >> 2) >= from) {
-          const int k = lane >> 2, ch = lane & 3;
-          bulk_copy(base + kB2A1 + (2 * w + k) * kB2A1Slot + ch * kRowBytes, row_src(a1p, row0 - 3 + k, ch), kRowBytes,
-                    full_a + w);
-        }
-        last_a[w] = c;
-        ++c;
+    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, next()) {
+      if (i >= kB2Stages)
+        ok = bar_wait(done_d + st, ph ^ 1u) && bar_wait(done_w + st, ph ^ 1u) && bar_wait(done_x + st, ph ^ 1u);
+      ok = __all_sync(0xffffffffu, ok && !*s_fail);
+      if (!ok) break;
+      const long long row = t / tiles_x, img = row / H * H;   // rows of all images; the image's first
+      const int x0 = (int)(t - row * tiles_x) * kTileW, y = (int)(row - img);
+      const uint32_t stage = base + st * kB2Stage, xbytes = 16u * (uint32_t)min(kTileW, W - x0);
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(full + st)),
+                     "r"(6u * kB2Slot + xbytes)
+                     : "memory");
+      __syncwarp();
+      if (lane < 24) {
+        const int k = lane % 12, r = k >> 2, ch = k & 3, yy = y - 1 + r;
+        const bool a1 = lane < 12;
+        const uint4 *src = yy >= 0 && yy < H
+                               ? (a1 ? a1p : dz2p) + ((size_t)(img + yy) * 4 + ch) * plane_w + x0 : zero;
+        bulk_copy(stage + (a1 ? r * kB2A1Slot : kB2Dz2 + r * kB2Slot) + ch * kRowBytes, src, kRowBytes, full + st);
+      } else if (lane == 24) {
+        bulk_copy(stage + kB2X, feats + (size_t)row * W + x0, xbytes, full + st);
       }
     }
     if (!ok) fail();
-    // no copy outlives the CTA
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (last_d[k] >= 0) bar_wait(full_d + k, (uint32_t)(last_d[k] >> 2) & 1u);
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-      if (last_a[k] >= 0) bar_wait(full_a + k, (uint32_t)(last_a[k] / 3) & 1u);
+    // no copy outlives the CTA: the last tile of each stage
+    for (int k = i < kB2Stages ? 0 : i - kB2Stages; k < i; ++k)
+      bar_wait(full + k % kB2Stages, (uint32_t)(k / kB2Stages) & 1u);
   } else if (warp == 5) {
-    // ---------------------------------------------------------- da1 and dW1
+    // ------------------------------------------------------------------ da1
     if (lane == 0) {
-      int have = 0;           // groups whose copies have been waited for
-      bool before = false;    // the previous group was a pair
-      for (long long q = first; q < last && ok;) {
-        int b, x0, y0;
-        const int n = segment(q, &b, &x0, &y0);
-        q += n;
-        for (int P = -1; P <= n && ok; ++P, ++g) {
-          const bool mid = P >= 0 && P < n;
-          for (const int need = mid ? g + 2 : g + 1; have < need && ok; ++have)
-            ok = bar_wait(full_d + (have & 3), (uint32_t)(have >> 2) & 1u);
-          if (*s_fail) ok = false;
-          if (!ok) break;
-          if (mid) {
-            const uint32_t d = tmem + kB2ColDa + 64u * (uint32_t)(c & 1);
-            // dz2 row y0' + k (k = -1..2); pixel q of the output reads halo
-            // pixel q + 2 - kx; blocks blk, blk + 1 of the kernel rows
-            auto conv = [&](int grp, int rr, int blk, uint32_t dcol, int N, int j, uint32_t acc) {
-              const int kx = j >> 1, hh = j & 1;
-              mma_bf16(d + dcol,
-                       sdesc(base + kB2Dz2 + (2 * (grp & 3) + rr) * kB2Slot + 2 * hh * kRowBytes + (2 - kx) * 16,
-                             kRowBytes, 128),
-                       sdesc(base + kB2W2 + blk * 6144 + j * 256, 128, 1536), idesc_bf16(128, N), acc);
-            };
+      for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, next()) {
+        ok = bar_wait(full + st, ph);
+        if (ok && i >= kB2Stages) ok = bar_wait(ep + st, ph ^ 1u);   // the stage's former da1 is read
+        if (*s_fail) ok = false;
+        if (!ok) break;
+        tc_after_sync();
+        // tap (ky, kx): pixel q of row y reads dz2 row y + 1 - ky at halo pixel q + 2 - kx
+        const uint32_t z = base + st * kB2Stage + kB2Dz2;
 #pragma unroll
-            for (int j = 0; j < 6; ++j) conv(g, 0, 1, 0, 64, j, j ? 1u : 0u);
+        for (int tap = 0; tap < 9; ++tap) {
+          const int ky = tap / 3, kx = tap % 3;
 #pragma unroll
-            for (int j = 0; j < 6; ++j) conv(g, 1, 0, 0, 64, j, 1u);
-#pragma unroll
-            for (int j = 0; j < 6; ++j) {
-              conv(g - 1, 1, 2, 0, 32, j, 1u);
-              conv(g + 1, 0, 0, 32, 32, j, 1u);
-            }
-            mma_commit(prod + (c & 1));
-          }
-          if (before) {        // dW1 and db1 of the previous pair, step e
-            const int e = c - 1;
-            ok = bar_wait(ep + (e & 1), (uint32_t)(e >> 1) & 1u);
-            if (!ok) break;
-            tc_after_sync();
-            const uint32_t a = base + kB2Dz1 + (e & 1) * 8 * kChunkPx, x = base + kB2X + 3 * ((g - 1) & 3) * kChunkPx;
-#pragma unroll
-            for (int s = 0; s < kTileW / 16; ++s)
-#pragma unroll
-              for (int rr = 0; rr < 2; ++rr)
-                mma_bf16(tmem + kB2ColW1, sdesc(a + 4 * rr * kChunkPx + s * 256, 128, kChunkPx),
-                         sdesc(x + rr * kChunkPx + s * 256, 128, (2 - rr) * kChunkPx), idesc_bf16_mn(64, 16),
-                         e > 0 || s > 0 || rr ? 1u : 0u);
-          }
-          if (g > 0) mma_commit(done_d + ((g - 1) & 3));
-          before = mid;
-          if (mid) ++c;
+          for (int j = 0; j < 2; ++j)
+            mma_bf16(tmem + kB2ColDa + 32u * (uint32_t)st,
+                     sdesc(z + (2 - ky) * kB2Slot + 2 * j * kRowBytes + (2 - kx) * 16, kRowBytes, 128),
+                     sdesc(base + kB2W2 + ky * 6144 + (2 * kx + j) * 256, 128, 1536), idesc_bf16(128, 32),
+                     (tap | j) ? 1u : 0u);
         }
+        mma_commit(prod + st);
+        mma_commit(done_d + st);
       }
       if (!ok) fail();
       mma_commit(drain);
       if (!bar_wait(drain, 0u)) fail();
     }
+  } else if (warp == 9) {
+    // ---------------------------------------------------------- dW1 and db1
+    if (lane == 0) {
+      for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, next()) {
+        ok = bar_wait(full + st, ph) && bar_wait(ep + st, ph);
+        if (*s_fail) ok = false;
+        if (!ok) break;
+        tc_after_sync();
+        const uint32_t x = base + st * kB2Stage + kB2X, z = base + kB2Dz1 + st * 4 * kChunkPx;
+#pragma unroll
+        for (int s = 0; s < kTileW / 16; ++s)
+          mma_bf16(tmem + kB2ColW1, sdesc(x + s * 256, 128, kChunkPx), sdesc(z + s * 256, 128, kChunkPx),
+                   idesc_bf16_mn(64, 32), i > 0 || s > 0 ? 1u : 0u);
+        mma_commit(done_x + st);
+      }
+      if (!ok) fail();
+      mma_commit(drain + 1);
+      if (!bar_wait(drain + 1, 0u)) fail();
+    }
   } else if (warp >= 6) {
     // ---------------------------------------------------------- dW2 and db2
     if (lane == 0) {
       const int kx = warp - 6;
-      for (long long q = first; q < last && ok;) {
-        int b, x0, y0;
-        const int n = segment(q, &b, &x0, &y0);
-        q += n;
-        for (int P = -1; P <= n; ++P, ++g) {
-          const bool mid = P >= 0 && P < n;
-          ok = bar_wait(full_d + (g & 3), (uint32_t)(g >> 2) & 1u);
-          if (ok && mid) ok = bar_wait(full_a + c % 3, (uint32_t)(c / 3) & 1u);
-          if (*s_fail) ok = false;
-          if (!ok) break;
-          if (mid) {
-            const uint32_t a = base + kB2A1 + 2 * (c % 3) * kB2A1Slot + kx * 16;
-            const uint32_t z = base + kB2Dz2 + 2 * (g & 3) * kB2Slot + 16;
+      for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, next()) {
+        ok = bar_wait(full + st, ph);
+        if (*s_fail) ok = false;
+        if (!ok) break;
+        const uint32_t a = base + st * kB2Stage + kx * 16, z = base + st * kB2Stage + kB2Dz2 + kB2Slot + 16;
 #pragma unroll
-            for (int s = 0; s < kTileW / 16; ++s)
-#pragma unroll
-              for (int rr = 0; rr < 2; ++rr)
-                mma_bf16(tmem + kB2ColW2 + 32 * kx, sdesc(a + rr * kB2A1Slot + s * 256, 128, kRowBytes),
-                         sdesc(z + rr * kB2Slot + s * 256, 128, kRowBytes), idesc_bf16_mn(128, 32),
-                         c > 0 || s > 0 || rr ? 1u : 0u);
-            mma_commit(done_c + c % 3);
-            ++c;
-          }
-          mma_commit(done_w + (g & 3));
-        }
+        for (int s = 0; s < kTileW / 16; ++s)
+          mma_bf16(tmem + kB2ColW2 + 32 * kx, sdesc(a + s * 256, 128, kRowBytes), sdesc(z + s * 256, 128, kRowBytes),
+                   idesc_bf16_mn(128, 32), i > 0 || s > 0 ? 1u : 0u);
+        mma_commit(done_w + st);
       }
       if (!ok) fail();
-      mma_commit(drain + 1 + kx);
-      if (!bar_wait(drain + 1 + kx, 0u)) fail();
+      mma_commit(drain + 2 + kx);
+      if (!bar_wait(drain + 2 + kx, 0u)) fail();
     }
   } else {
     // ------------------------------------------------------------ epilogues
     const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
-    for (long long q = first; q < last && ok;) {
-      int b, x0, y0;
-      const int n = segment(q, &b, &x0, &y0);
-      q += n;
-      for (int P = 0; P < n; ++P, ++c) {
-        ok = bar_wait(full_a + c % 3, (uint32_t)(c / 3) & 1u) && bar_wait(prod + (c & 1), (uint32_t)(c >> 1) & 1u);
-        ok = __all_sync(0xffffffffu, ok && !*s_fail);
-        if (!ok) break;
-        tc_after_sync();
-        // dz1 = da1 [a1 > 0]; a1 is zero outside the image
+    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, next()) {
+      ok = bar_wait(full + st, ph) && bar_wait(prod + st, ph);
+      ok = __all_sync(0xffffffffu, ok && !*s_fail);
+      if (!ok) break;
+      tc_after_sync();
+      // dz1 = da1 [a1 > 0]; a1 is zero outside the image. The copies of this
+      // stage waited for its former dz1 to be read
+      float da[32];
+      tmem_ld32(tmem + lane_base + kB2ColDa + 32u * (uint32_t)st, da);
+      const uint8_t *a1 = smem + st * kB2Stage + kB2A1Slot + (tid + 1) * 16;
+      uint32_t w[16];
 #pragma unroll
-        for (int rr = 0; rr < 2; ++rr) {
-          float da[32];
-          tmem_ld32(tmem + lane_base + kB2ColDa + 64u * (uint32_t)(c & 1) + 32u * rr, da);
-          const uint8_t *a1 = smem + kB2A1 + (2 * (c % 3) + 1 + rr) * kB2A1Slot + (tid + 1) * 16;
-          uint8_t *dst = smem + kB2Dz1 + ((c & 1) * 8 + rr * 4) * kChunkPx;
-          uint32_t w[16];
+      for (int ch = 0; ch < 4; ++ch) {
+        const uint4 u = *reinterpret_cast<const uint4 *>(a1 + ch * kRowBytes);
+        const uint32_t aw[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-          for (int ch = 0; ch < 4; ++ch) {
-            const uint4 u = *reinterpret_cast<const uint4 *>(a1 + ch * kRowBytes);
-            const uint32_t aw[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float lo = __uint_as_float(aw[k] << 16), hi = __uint_as_float(aw[k] & 0xFFFF0000u);
-              w[4 * ch + k] = pack_bf16x2(lo > 0.f ? da[8 * ch + 2 * k] : 0.f, hi > 0.f ? da[8 * ch + 2 * k + 1] : 0.f);
-            }
-          }
-          st_chunks(dst, kChunkPx, tid, w);
+        for (int k = 0; k < 4; ++k) {
+          const float lo = __uint_as_float(aw[k] << 16), hi = __uint_as_float(aw[k] & 0xFFFF0000u);
+          w[4 * ch + k] = pack_bf16x2(lo > 0.f ? da[8 * ch + 2 * k] : 0.f, hi > 0.f ? da[8 * ch + 2 * k + 1] : 0.f);
         }
-        fence_async_smem();
-        tc_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(ep + (c & 1));
       }
+      st_chunks(smem + kB2Dz1 + st * 4 * kChunkPx, kChunkPx, tid, w);
+      fence_async_smem();
+      tc_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(ep + st);
     }
     if (!ok) fail();
   }
@@ -1241,28 +1157,30 @@ mpnet_bwd2_kernel(const uint8_t *__restrict__ weights, const uint4 *__restrict__
   if (warp < 4) {
     const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
     float d[32];
-    const int ky = tid / 40, i = tid % 40;   // D row 40 ky + i; i = 32: the ones
+    const int ky = tid / 40, ci = tid % 40;   // D row 40 ky + ci; ci = 32: the ones
     for (int kx = 0; kx < 3; ++kx) {
       tmem_ld32(tmem + lane_base + kB2ColW2 + 32 * kx, d);
-      if (ky < 3 && i < 32) {
+      if (ky < 3 && ci < 32) {
 #pragma unroll
-        for (int o = 0; o < 32; ++o) atomicAdd(grad + kGW2 + o * 288 + (3 * ky + kx) * 32 + i, d[o]);
-      } else if (kx == 0 && ky == 0 && i == 32) {
+        for (int o = 0; o < 32; ++o) atomicAdd(grad + kGW2 + o * 288 + (3 * ky + kx) * 32 + ci, d[o]);
+      } else if (kx == 0 && ky == 0 && ci == 32) {
 #pragma unroll
         for (int o = 0; o < 32; ++o) atomicAdd(grad + kGb2 + o, d[o]);
       }
     }
-    const int r = m64_row(tid);
     tmem_ld32(tmem + lane_base + kB2ColW1, d);
-    if (r >= 0 && r < 32) {
+    const int r = m64_row(tid);               // D row r: input channel; 8: the ones
+    if (r >= 0 && r < 8) {
 #pragma unroll
-      for (int k = 0; k < 8; ++k) atomicAdd(grad + kGW1 + r * 16 + k, d[k]);
-      atomicAdd(grad + kGb1 + r, d[8]);
+      for (int o = 0; o < 32; ++o) atomicAdd(grad + kGW1 + o * 16 + r, d[o]);
+    } else if (r == 8) {
+#pragma unroll
+      for (int o = 0; o < 32; ++o) atomicAdd(grad + kGb1 + o, d[o]);
     }
   }
   tc_before_sync();
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256));
 }
 
 // Adam on the FP32 master parameters (gradient layout), refreshing the BF16
@@ -1343,11 +1261,10 @@ cudaError_t launch_mpnet_train(void *weights, float *master, float *adam_m, floa
                                double *loss, const MpnetScratch &sc, uint32_t *status, int num_sms, cudaStream_t s) {
   const long long npix = (long long)batch * H * W;
   cudaError_t e = cudaMemsetAsync(sc.grad, 0, kGTotal * sizeof(float), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(sc.inv_n, 0, 2 * sizeof(float), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(sc.count, 0, sizeof(unsigned), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(loss, 0, sizeof(double), s);
   if (e != cudaSuccess) return e;
-  mpnet_count_kernel<<<num_sms, 256, 0, s>>>(target, npix, sc.inv_n, nullptr);
-  mpnet_count_finish_kernel<<<1, 1, 0, s>>>(sc.inv_n);
+  mpnet_count_kernel<<<(unsigned)std::min(8ll * num_sms, (npix + 255) / 256), 256, 0, s>>>(target, npix, sc.count);
   e = launch_mpnet_forward(weights, feats, batch, W, H, sc.y, nullptr, sc.planes, status, num_sms, s);
   if (e != cudaSuccess) return e;
   const int tiles_x = (W + kTileW - 1) / kTileW;
@@ -1355,19 +1272,17 @@ cudaError_t launch_mpnet_train(void *weights, float *master, float *adam_m, floa
   // bwd1 holds 128 TMEM columns and 55 KB of shared memory: four CTAs per SM
   // give four independent tile streams
   const int grid1 = (int)(ntiles < 4ll * num_sms ? ntiles : 4ll * num_sms);
-  // bwd2: the row pairs of all strips, one contiguous range per CTA
-  const long long npairs = (long long)batch * tiles_x * ((H + 1) / 2);
-  const int grid2 = (int)(npairs < num_sms ? npairs : num_sms);
+  const int grid2 = (int)(ntiles < num_sms ? ntiles : num_sms);
   e = cudaFuncSetAttribute(mpnet_bwd1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kB1Smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(mpnet_bwd2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kB2Smem);
   if (e != cudaSuccess) return e;
   const size_t plane_n = (size_t)mpnet_plane_size(batch, W, H);
   mpnet_bwd1_kernel<<<grid1, kB1Threads, kB1Smem, s>>>(static_cast<const uint8_t *>(weights), sc.y, target,
                                                       sc.planes + plane_n, sc.planes + 2 * plane_n, batch, W, H,
-                                                      sc.inv_n, sc.dz2, sc.grad, loss, status);
+                                                      sc.count, sc.dz2, sc.grad, loss, status);
   mpnet_bwd2_kernel<<<grid2, kB2Threads, kB2Smem, s>>>(static_cast<const uint8_t *>(weights),
                                                        reinterpret_cast<const uint4 *>(feats), sc.planes, sc.dz2, sc.zero,
-                                                       W, H, tiles_x, npairs, sc.grad, status);
+                                                       W, H, tiles_x, ntiles, sc.grad, status);
   const float beta1 = 0.9f, beta2 = 0.999f;
   const float bc1 = 1.f - powf(beta1, (float)step), bc2 = 1.f - powf(beta2, (float)step);
   mpnet_adam_kernel<<<(kGTotal + 255) / 256, 256, 0, s>>>(static_cast<uint8_t *>(weights), master, adam_m, adam_v,

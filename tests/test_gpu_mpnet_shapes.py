@@ -1,5 +1,5 @@
 """Training gradients of the MP network at the edges of its kernels' tiling:
-strips of 128 pixels, row pairs, one contiguous range of rows per CTA or
+strips of 128 pixels, one contiguous range of rows per
 warpgroup (fewer rows than CTAs, ranges that cross strips and images), and one
 context whose scratch serves frames that shrink and grow."""
 import numpy as np
