@@ -142,7 +142,7 @@ void free_lm(LmBuffers &b) {
 }
 
 void free_epi(EpiBuffers &b) {
-  void *ptrs[] = {b.count, b.off, b.block_sum, b.rank, b.vals, b.dist, b.F};
+  void *ptrs[] = {b.count, b.off, b.cursor, b.rank, b.vals, b.dist};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   b = EpiBuffers();
@@ -1101,11 +1101,9 @@ int splat_edge_warp(dags_ctx *ctx, const dags_camera *cam, const float *depth_i,
     return DAGS_E_INVAL;
   Raster r;
   if ((rc = make_raster(cam, nullptr, &r))) return rc;
-  if (!ctx->edge_partial || !ctx->rel32) {
-    cudaError_t a = ctx->edge_partial
-                        ? cudaSuccess
-                        : alloc(&ctx->edge_partial, (size_t)edge_warp_blocks((int64_t)ctx->ws.max_w * ctx->ws.max_h) * 13);
-    if (a == cudaSuccess && !ctx->rel32) a = alloc(&ctx->rel32, (size_t)12);
+  if (!ctx->edge_partial) {
+    const cudaError_t a =
+        alloc(&ctx->edge_partial, (size_t)edge_warp_blocks((int64_t)ctx->ws.max_w * ctx->ws.max_h) * 13);
     if (a != cudaSuccess) {
       cudaGetLastError();
       return a == cudaErrorMemoryAllocation ? DAGS_E_NOMEM : DAGS_E_CUDA;
@@ -1115,7 +1113,7 @@ int splat_edge_warp(dags_ctx *ctx, const dags_camera *cam, const float *depth_i,
   ctx->last_stream = s;
   const int ev = ctx->timer.begin(DAGS_K_REGULARISER, s);
   const cudaError_t e = launch_edge_warp(r, depth_i, depth_j, weight_j, pose_i, pose_j, c, lambda,
-                                         ctx->edge_partial, ctx->ws.counters + CNT_DONE_REG, out, ctx->rel32, s);
+                                         ctx->edge_partial, ctx->ws.counters + CNT_DONE_REG, out, s);
   ctx->timer.end(ev, s);
   return cuda_status(e);
 }
@@ -1142,11 +1140,10 @@ int epipolar_verify(dags_ctx *ctx, const dags_camera *cam, const double *pose_1,
     auto A = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
     A(alloc(&b.count, (size_t)cn));
     A(alloc(&b.off, (size_t)cn));
-    A(alloc(&b.block_sum, (size_t)epi_scan_blocks(cn) + 1));
+    A(alloc(&b.cursor, 1));
     A(alloc(&b.rank, (size_t)cm));
     A(alloc(&b.vals, (size_t)cm));
     A(alloc(&b.dist, (size_t)cm));
-    A(alloc(&b.F, (size_t)9));
     if (e != cudaSuccess) {
       cudaGetLastError();
       free_epi(b);

@@ -1,15 +1,14 @@
 // Epipolar verification and static recovery (Sec. IV-C, Eqs. (18), (19)) on
 // sm_103a:
 //
-//   epi_F_kernel        F = K^-T [t]x R K^-1 from the two poses, FP64, one
-//                       thread
-//   epi_dist_kernel     per match: the point-to-epipolar-line distance d of
+//   epi_dist_kernel     F = K^-T [t]x R K^-1 from the two poses, FP64, per CTA;
+//                       per match: the point-to-epipolar-line distance d of
 //                       Eq. (18) in FP64, and the match's
 //                       rank inside its Gaussian's group (one atomic per
 //                       match on the Gaussian's count)
-//   scan (3 kernels)    exclusive scan of the per-Gaussian counts into group
-//                       offsets: 1024 counts per CTA, the CTA sums by one CTA,
-//                       then the offsets added back
+//   epi_offsets_kernel  group offsets: a scan of 1024 counts per CTA, placed
+//                       behind one another by an atomic cursor (the groups'
+//                       order does not matter)
 //   epi_scatter_kernel  d into its group's slot (offset + rank)
 //   epi_median_kernel   per Gaussian with matches: the lower median of its
 //                       group by rank counting (the groups hold a few values;
@@ -30,50 +29,53 @@ constexpr int kEpiBlock = 256;
 constexpr int kScanItems = 4;                  // counts per thread in the block scan
 constexpr int kScanTile = kEpiBlock * kScanItems;
 
-// F = K^-T [t]x R K^-1 of the relative pose (R, t) = T_2W T_1W^-1, in FP64
-// by one thread (FP64 instructions are scarce on GB300: the per-match kernel
-// only reads it).
-__global__ void epi_F_kernel(Raster r, const double *__restrict__ pose_1, const double *__restrict__ pose_2,
-                             double *__restrict__ F) {
-  pdl_wait();
-  if (threadIdx.x != 0) return;
-  {
-    // R = R2 R1^T, t = t2 - R t1, E = [t]x R, F = K^-T E K^-1
-    double R[9], t[3], E[9];
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b)
-        R[3 * a + b] = pose_2[4 * a] * pose_1[4 * b] + pose_2[4 * a + 1] * pose_1[4 * b + 1] +
-                       pose_2[4 * a + 2] * pose_1[4 * b + 2];
-    for (int a = 0; a < 3; ++a)
-      t[a] = pose_2[4 * a + 3] - (R[3 * a] * pose_1[3] + R[3 * a + 1] * pose_1[7] + R[3 * a + 2] * pose_1[11]);
-    const double tx[9] = {0.0, -t[2], t[1], t[2], 0.0, -t[0], -t[1], t[0], 0.0};
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) E[3 * a + b] = tx[3 * a] * R[b] + tx[3 * a + 1] * R[3 + b] + tx[3 * a + 2] * R[6 + b];
-    // K^-1 = [[1/fx, 0, -cx/fx], [0, 1/fy, -cy/fy], [0, 0, 1]]
-    const double ifx = 1.0 / (double)r.fx, ify = 1.0 / (double)r.fy;
-    const double kx = -(double)r.cx * ifx, ky = -(double)r.cy * ify;
-    double EK[9];   // E K^-1
-    for (int a = 0; a < 3; ++a) {
-      EK[3 * a + 0] = E[3 * a] * ifx;
-      EK[3 * a + 1] = E[3 * a + 1] * ify;
-      EK[3 * a + 2] = E[3 * a] * kx + E[3 * a + 1] * ky + E[3 * a + 2];
+// F = K^-T [t]x R K^-1 of the relative pose (R, t) = T_2W T_1W^-1, in FP64 by
+// the first nine threads of a CTA (FP64 instructions are scarce on GB300, but
+// a launch of its own costs more than every CTA's few dozen).
+__device__ __forceinline__ void epi_F(const Raster &r, const double *__restrict__ pose_1,
+                                      const double *__restrict__ pose_2, double *F) {
+  __shared__ double s_R[9], s_EK[9], s_t[3];
+  const int k = threadIdx.x, a = k / 3, b = k % 3;
+  // R = R2 R1^T, t = t2 - R t1, E = [t]x R, F = K^-T E K^-1
+  if (k < 9)
+    s_R[k] = pose_2[4 * a] * pose_1[4 * b] + pose_2[4 * a + 1] * pose_1[4 * b + 1] +
+             pose_2[4 * a + 2] * pose_1[4 * b + 2];
+  __syncthreads();
+  if (k < 3)
+    s_t[k] = pose_2[4 * k + 3] - (s_R[3 * k] * pose_1[3] + s_R[3 * k + 1] * pose_1[7] + s_R[3 * k + 2] * pose_1[11]);
+  __syncthreads();
+  // K^-1 = [[1/fx, 0, -cx/fx], [0, 1/fy, -cy/fy], [0, 0, 1]]
+  const double ifx = 1.0 / (double)r.fx, ify = 1.0 / (double)r.fy;
+  const double kx = -(double)r.cx * ifx, ky = -(double)r.cy * ify;
+  if (k < 3) {   // row k of E K^-1
+    const double tx[9] = {0.0, -s_t[2], s_t[1], s_t[2], 0.0, -s_t[0], -s_t[1], s_t[0], 0.0};
+    double E[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const double t0 = k == 0 ? tx[0] : k == 1 ? tx[3] : tx[6], t1 = k == 0 ? tx[1] : k == 1 ? tx[4] : tx[7],
+                   t2 = k == 0 ? tx[2] : k == 1 ? tx[5] : tx[8];
+      E[j] = t0 * s_R[j] + t1 * s_R[3 + j] + t2 * s_R[6 + j];
     }
-    // K^-T (E K^-1): rows 0, 1 scale, row 2 combines
-    for (int b = 0; b < 3; ++b) {
-      F[b] = EK[b] * ifx;
-      F[3 + b] = EK[3 + b] * ify;
-      F[6 + b] = EK[b] * kx + EK[3 + b] * ky + EK[6 + b];
-    }
+    s_EK[3 * k + 0] = E[0] * ifx;
+    s_EK[3 * k + 1] = E[1] * ify;
+    s_EK[3 * k + 2] = E[0] * kx + E[1] * ky + E[2];
   }
+  __syncthreads();
+  // K^-T (E K^-1): rows 0, 1 scale, row 2 combines
+  if (k < 3) F[k] = s_EK[k] * ifx;
+  else if (k < 6) F[k] = s_EK[k] * ify;
+  else if (k < 9) F[k] = s_EK[b] * kx + s_EK[3 + b] * ky + s_EK[6 + b];
 }
 
 __global__ void __launch_bounds__(kEpiBlock)
-epi_dist_kernel(const double *__restrict__ F, const float2 *__restrict__ p1, const float2 *__restrict__ p2,
-                const int32_t *__restrict__ gid, int64_t m, int64_t n, float *__restrict__ dist,
-                uint32_t *__restrict__ count, uint32_t *__restrict__ rank, uint32_t *status) {
+epi_dist_kernel(Raster r, const double *__restrict__ pose_1, const double *__restrict__ pose_2,
+                const float2 *__restrict__ p1, const float2 *__restrict__ p2, const int32_t *__restrict__ gid,
+                int64_t m, int64_t n, float *__restrict__ dist, uint32_t *__restrict__ count,
+                uint32_t *__restrict__ rank, uint32_t *__restrict__ cursor, uint32_t *status) {
   pdl_wait();
   __shared__ double s_F[9];
-  if (threadIdx.x < 9) s_F[threadIdx.x] = F[threadIdx.x];
+  if (blockIdx.x == 0 && threadIdx.x == 0) *cursor = 0u;
+  epi_F(r, pose_1, pose_2, s_F);
   __syncthreads();
   const int64_t k = (int64_t)blockIdx.x * kEpiBlock + threadIdx.x;
   if (k >= m) return;
@@ -94,14 +96,16 @@ epi_dist_kernel(const double *__restrict__ F, const float2 *__restrict__ p1, con
   rank[k] = atomicAdd(count + g, 1u);
 }
 
-// Exclusive scan of count[0, n) into off[0, n): per CTA 1024 counts (four
-// per thread, then a shared-memory scan of the thread sums); block sums out.
+// The first slot of every group: per CTA an exclusive scan of 1024 counts (four
+// per thread, a warp scan of the thread sums, the eight warp sums), offset by
+// the CTA's share of a global cursor. Three launches (tile scans, their sums,
+// the addition) gave the groups in order, which nothing needs.
 __global__ void __launch_bounds__(kEpiBlock)
-scan_tiles_kernel(const uint32_t *__restrict__ count, int64_t n, uint32_t *__restrict__ off,
-                  uint32_t *__restrict__ block_sum) {
+epi_offsets_kernel(const uint32_t *__restrict__ count, int64_t n, uint32_t *__restrict__ off,
+                   uint32_t *__restrict__ cursor) {
   pdl_wait();
-  __shared__ uint32_t s[kEpiBlock];
-  const int tid = threadIdx.x;
+  __shared__ uint32_t s_warp[kEpiBlock / 32], s_base;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)tid * kScanItems;
   uint32_t v[kScanItems], acc = 0;
 #pragma unroll
@@ -109,54 +113,25 @@ scan_tiles_kernel(const uint32_t *__restrict__ count, int64_t n, uint32_t *__res
     v[j] = base + j < n ? count[base + j] : 0u;
     acc += v[j];
   }
-  s[tid] = acc;
-  __syncthreads();
-  for (int o = 1; o < kEpiBlock; o <<= 1) {
-    const uint32_t add = tid >= o ? s[tid - o] : 0u;
-    __syncthreads();
-    s[tid] += add;
-    __syncthreads();
+  uint32_t inc = acc;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t add = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += add;
   }
-  uint32_t run = s[tid] - acc;   // exclusive prefix of this thread's items
+  if (lane == 31) s_warp[warp] = inc;
+  __syncthreads();
+  uint32_t run = inc - acc;
+#pragma unroll
+  for (int w = 0; w < kEpiBlock / 32; ++w) run += w < warp ? s_warp[w] : 0u;
+  if (tid == kEpiBlock - 1) s_base = run + acc ? atomicAdd(cursor, run + acc) : 0u;
+  __syncthreads();
+  run += s_base;
 #pragma unroll
   for (int j = 0; j < kScanItems; ++j) {
-    if (base + j < n) off[base + j] = run;
+    if (v[j]) off[base + j] = run;
     run += v[j];
   }
-  if (tid == kEpiBlock - 1) block_sum[blockIdx.x] = s[tid];
-}
-
-// One CTA: exclusive scan of the block sums in place, sequential chunks.
-__global__ void __launch_bounds__(kEpiBlock)
-scan_sums_kernel(uint32_t *__restrict__ block_sum, int nb) {
-  pdl_wait();
-  __shared__ uint32_t s[kEpiBlock];
-  __shared__ uint32_t carry;
-  const int tid = threadIdx.x;
-  if (tid == 0) carry = 0u;
-  __syncthreads();
-  for (int c0 = 0; c0 < nb; c0 += kEpiBlock) {
-    const uint32_t v = c0 + tid < nb ? block_sum[c0 + tid] : 0u;
-    s[tid] = v;
-    __syncthreads();
-    for (int o = 1; o < kEpiBlock; o <<= 1) {
-      const uint32_t add = tid >= o ? s[tid - o] : 0u;
-      __syncthreads();
-      s[tid] += add;
-      __syncthreads();
-    }
-    if (c0 + tid < nb) block_sum[c0 + tid] = carry + s[tid] - v;
-    __syncthreads();
-    if (tid == kEpiBlock - 1) carry += s[tid];
-    __syncthreads();
-  }
-}
-
-__global__ void __launch_bounds__(kEpiBlock)
-scan_add_kernel(uint32_t *__restrict__ off, int64_t n, const uint32_t *__restrict__ block_sum) {
-  pdl_wait();
-  const int64_t i = (int64_t)blockIdx.x * kEpiBlock + threadIdx.x;
-  if (i < n) off[i] += block_sum[i / kScanTile];
 }
 
 __global__ void __launch_bounds__(kEpiBlock)
@@ -206,8 +181,6 @@ epi_median_kernel(const uint32_t *__restrict__ count, const uint32_t *__restrict
 
 }  // namespace
 
-int64_t epi_scan_blocks(int64_t n) { return (n + kScanTile - 1) / kScanTile; }
-
 cudaError_t launch_epipolar(const Raster &r, const double *pose_1, const double *pose_2, const float2 *p1,
                             const float2 *p2, const int32_t *gid, int64_t m, float4 *gauss, int64_t n,
                             uint8_t *labels, float eps, float m_static, float *dist, float *dbar, const EpiBuffers &b,
@@ -216,21 +189,15 @@ cudaError_t launch_epipolar(const Raster &r, const double *pose_1, const double 
   if (e != cudaSuccess) return e;
   const unsigned gm = (unsigned)((m + kEpiBlock - 1) / kEpiBlock);
   const unsigned gn = (unsigned)((n + kEpiBlock - 1) / kEpiBlock);
-  const int nb = (int)epi_scan_blocks(n);
   // programmatic launches after the first: each kernel waits for its
   // predecessor's memory before its first access, and its launch overlaps
   // the predecessor's last wave
   if (m > 0) {
-    epi_F_kernel<<<1, 32, 0, s>>>(r, pose_1, pose_2, b.F);
-    e = launch_pdl(epi_dist_kernel, dim3(gm), dim3(kEpiBlock), 0, s, (const double *)b.F, p1, p2, gid, m, n, dist,
-                   b.count, b.rank, status);
-  }
-  if (n > 0 && e == cudaSuccess) {
-    e = launch_pdl(scan_tiles_kernel, dim3((unsigned)nb), dim3(kEpiBlock), 0, s, (const uint32_t *)b.count, n, b.off,
-                   b.block_sum);
-    if (e == cudaSuccess) e = launch_pdl(scan_sums_kernel, dim3(1), dim3(kEpiBlock), 0, s, b.block_sum, nb);
-    if (e == cudaSuccess)
-      e = launch_pdl(scan_add_kernel, dim3(gn), dim3(kEpiBlock), 0, s, b.off, n, (const uint32_t *)b.block_sum);
+    epi_dist_kernel<<<gm, kEpiBlock, 0, s>>>(r, pose_1, pose_2, p1, p2, gid, m, n, dist, b.count, b.rank, b.cursor,
+                                             status);
+    if (n > 0)
+      e = launch_pdl(epi_offsets_kernel, dim3((unsigned)((n + kScanTile - 1) / kScanTile)), dim3(kEpiBlock), 0, s,
+                     (const uint32_t *)b.count, n, b.off, b.cursor);
   }
   if (m > 0 && e == cudaSuccess)
     e = launch_pdl(epi_scatter_kernel, dim3(gm), dim3(kEpiBlock), 0, s, gid, (const uint32_t *)b.rank,

@@ -15,8 +15,8 @@
 // MP-guided edge-warp regulariser (Sec. IV-D, Eqs. (25), (26)): one thread
 // per pixel u of frame i. An edge pixel (a valid 4-neighbour differs by more
 // than edge_rel times its depth) is back-projected with its observed depth, moved by
-// T_ji = T_jW T_iW^-1 (formed once in FP64 by a one-thread kernel) and projected into frame
-// j; D_j and w^j are sampled bilinearly at u', r = w^j (D_j - z_ref) enters
+// T_ji = T_jW T_iW^-1 (formed in FP64 by twelve threads of each CTA) and
+// projected into frame j; D_j and w^j are sampled bilinearly at u', r = w^j (D_j - z_ref) enters
 // the Huber kernel, and the gradients with respect to both poses' left
 // twists follow by the chain rule through the bilinear cell, the projection
 // and the rigid motion. The 13 sums go per CTA in FP32 (warp shuffles, then
@@ -97,26 +97,23 @@ mp_consistency_kernel(const float4 *__restrict__ gauss, const float4 *__restrict
   }
 }
 
-// T_ji = T_jW T_iW^-1 (R = Rj Ri^T, t = tj - R ti) of two world-to-camera
-// poses, or pose_j itself when pose_i is NULL, in FP64 by one thread, rounded
-// to FP32 for the per-element kernels.
-__global__ void rel_pose_kernel(const double *__restrict__ pose_i, const double *__restrict__ pose_j,
-                                float *__restrict__ out) {
-  if (threadIdx.x != 0) return;
-  if (!pose_i) {
-    for (int k = 0; k < 12; ++k) out[k] = (float)pose_j[k];
-    return;
-  }
-  double R[9];
-  for (int a = 0; a < 3; ++a)
-    for (int b = 0; b < 3; ++b)
-      R[3 * a + b] = pose_j[4 * a] * pose_i[4 * b] + pose_j[4 * a + 1] * pose_i[4 * b + 1] +
-                     pose_j[4 * a + 2] * pose_i[4 * b + 2];
-  for (int a = 0; a < 3; ++a) {
-    for (int b = 0; b < 3; ++b) out[4 * a + b] = (float)R[3 * a + b];
-    out[4 * a + 3] =
-        (float)(pose_j[4 * a + 3] - (R[3 * a] * pose_i[3] + R[3 * a + 1] * pose_i[7] + R[3 * a + 2] * pose_i[11]));
-  }
+// Entry k of T_ji = T_jW T_iW^-1 (R = Rj Ri^T, t = tj - R ti) of two
+// world-to-camera poses, in FP64, rounded to FP32 for the per-element kernels.
+__device__ __forceinline__ float rel_pose_entry(const double *__restrict__ pose_i, const double *__restrict__ pose_j,
+                                                int k) {
+  const int a = k >> 2, b = k & 3;
+  double R[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+    R[j] = pose_j[4 * a] * pose_i[4 * j] + pose_j[4 * a + 1] * pose_i[4 * j + 1] +
+           pose_j[4 * a + 2] * pose_i[4 * j + 2];
+  if (b < 3) return (float)(b == 0 ? R[0] : b == 1 ? R[1] : R[2]);
+  return (float)(pose_j[4 * a + 3] - (R[0] * pose_i[3] + R[1] * pose_i[7] + R[2] * pose_i[11]));
+}
+
+// A pose rounded to FP32.
+__global__ void pose32_kernel(const double *__restrict__ pose, float *__restrict__ out) {
+  if (threadIdx.x < 12) out[threadIdx.x] = (float)pose[threadIdx.x];
 }
 
 constexpr int kEdgeBlock = 256;
@@ -124,20 +121,22 @@ constexpr int kEdgeOut = 13;     // lambda L_edge, d/d xi_i (6), d/d xi_j (6)
 
 __global__ void __launch_bounds__(kEdgeBlock)
 edge_warp_kernel(Raster r, const float *__restrict__ Di, const float *__restrict__ Dj,
-                 const float *__restrict__ wj, const float *__restrict__ Tji, dags_edge_cfg c, float lam,
-                 double *__restrict__ partial, uint32_t *__restrict__ done, double *__restrict__ out) {
-  pdl_wait();
+                 const float *__restrict__ wj, const double *__restrict__ pose_i, const double *__restrict__ pose_j,
+                 dags_edge_cfg c, float lam, double *__restrict__ partial, uint32_t *__restrict__ done,
+                 double *__restrict__ out) {
   __shared__ float s_T[12];
   __shared__ float s_red[kEdgeBlock / 32][kEdgeOut];
   __shared__ int s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid < 12) s_T[tid] = Tji[tid];
+  // T_ji per CTA: a launch of its own for these few FP64 operations costs more
+  if (tid < 12) s_T[tid] = rel_pose_entry(pose_i, pose_j, tid);
   __syncthreads();
   const int W = r.W, H = r.H;
   const int p = blockIdx.x * kEdgeBlock + tid;
   float v[kEdgeOut];
 #pragma unroll
   for (int k = 0; k < kEdgeOut; ++k) v[k] = 0.f;
+  bool hit = false;
   if (p < W * H) {
     const int y = p / W, x = p - y * W;
     const float d = Di[p];
@@ -187,6 +186,7 @@ edge_warp_kernel(Raster r, const float *__restrict__ Di, const float *__restrict
             float g2 = -(dru * r.fx * Y0 + drv * r.fy * Y1) * iz * iz;
             if (!c.literal) g2 -= ws;
             g0 *= drho; g1 *= drho; g2 *= drho;
+            hit = true;
             v[0] = rho;
             // pose j: rho_j += gY, phi_j += Y x gY
             v[7] = g0; v[8] = g1; v[9] = g2;
@@ -202,10 +202,15 @@ edge_warp_kernel(Raster r, const float *__restrict__ Di, const float *__restrict
       }
     }
   }
+  // few warps hold an edge: the others' sums are the zeros that they would add up
+  if (__any_sync(0xffffffffu, hit)) {
 #pragma unroll
-  for (int k = 0; k < kEdgeOut; ++k) {
-    const float sw = warp_sum(v[k]);
-    if (lane == 0) s_red[warp][k] = sw;
+    for (int k = 0; k < kEdgeOut; ++k) {
+      const float sw = warp_sum(v[k]);
+      if (lane == 0) s_red[warp][k] = sw;
+    }
+  } else if (lane < kEdgeOut) {
+    s_red[warp][lane] = 0.f;
   }
   __syncthreads();
   if (tid < kEdgeOut) {
@@ -227,9 +232,16 @@ edge_warp_kernel(Raster r, const float *__restrict__ Di, const float *__restrict
   __shared__ double s_col[kEdgeOut * 16];
   if (tid < kEdgeOut * 16) {
     const int c = tid >> 4, part = tid & 15;
+    // the loads of twelve partials side by side, added in order
     double a[4] = {0.0, 0.0, 0.0, 0.0};
-    int j = 0;
-    for (int b = part; b < (int)gridDim.x; b += 16, ++j) a[j & 3] += __ldcg(partial + (size_t)b * kEdgeOut + c);
+    const int n = (int)gridDim.x;
+    for (int b = part; b < n; b += 16 * 12) {
+      double x[12];
+#pragma unroll
+      for (int j = 0; j < 12; ++j) x[j] = b + 16 * j < n ? __ldcg(partial + (size_t)(b + 16 * j) * kEdgeOut + c) : 0.0;
+#pragma unroll
+      for (int j = 0; j < 12; ++j) a[j & 3] += x[j];
+    }
     s_col[tid] = (a[0] + a[1]) + (a[2] + a[3]);
   }
   __syncthreads();
@@ -249,13 +261,9 @@ int64_t edge_warp_blocks(int64_t pixels) { return (pixels + kEdgeBlock - 1) / kE
 
 cudaError_t launch_edge_warp(const Raster &r, const float *Di, const float *Dj, const float *wj, const double *pose_i,
                              const double *pose_j, const dags_edge_cfg &c, float lam, double *partial, uint32_t *done,
-                             double *out, float *tji, cudaStream_t s) {
-  rel_pose_kernel<<<1, 32, 0, s>>>(pose_i, pose_j, tji);
-  // a programmatic launch: the warp's launch overlaps the one-thread kernel
-  const cudaError_t e = launch_pdl(edge_warp_kernel, dim3((unsigned)edge_warp_blocks((int64_t)r.W * r.H)),
-                                   dim3(kEdgeBlock), 0, s, r, Di, Dj, wj, (const float *)tji, c, lam, partial, done,
-                                   out);
-  if (e != cudaSuccess) return e;
+                             double *out, cudaStream_t s) {
+  edge_warp_kernel<<<(unsigned)edge_warp_blocks((int64_t)r.W * r.H), kEdgeBlock, 0, s>>>(
+      r, Di, Dj, wj, pose_i, pose_j, c, lam, partial, done, out);
   return cudaGetLastError();
 }
 
@@ -268,7 +276,7 @@ cudaError_t launch_mp_consistency(const float4 *gauss, const float4 *prev, int64
     if (loss) return cudaMemsetAsync(loss, 0, sizeof(double), s);
     return cudaSuccess;
   }
-  if (rel) rel_pose_kernel<<<1, 32, 0, s>>>(nullptr, rel, rel32);
+  if (rel) pose32_kernel<<<1, 32, 0, s>>>(rel, rel32);
   const cudaError_t e = launch_pdl(mp_consistency_kernel, dim3((unsigned)mp_consistency_blocks(n)), dim3(kRegBlock), 0, s,
                                    gauss, prev, n, (const float *)(rel ? rel32 : nullptr), lam, grad, partial, done, loss);
   if (e != cudaSuccess) return e;
