@@ -60,3 +60,38 @@ def test_association_radii(dags, r_s, scales):
     d = mp_scene(30_000, 31, 253, 189, seed=8)
     gpu, ref = run_both(dags, d, {"r_s": r_s, "scales": scales})
     check(gpu, ref, d["table"].shape[0])
+
+
+def test_update_replays_from_a_graph(dags):
+    # the cooperative launch is captured like the others: a replay gives the
+    # medians and labels of a plain call on the same records
+    d = mp_scene(20_000, 31, 160, 120, seed=9)
+    cam = dags.Camera(*d["cam"].as_tuple())
+    P = cam.width * cam.height
+    image = torch.zeros((8, P), dtype=torch.float32)
+    image[0:3] = torch.from_numpy(d["rend"][:, 0:3].T.copy())
+    image[3] = torch.from_numpy(d["rend"][:, 3].copy())
+    image = image.cuda()
+    rec = torch.from_numpy(d["rec"].copy()).cuda()
+    tg, inst, table, lab0 = (torch.from_numpy(d[k].copy()).cuda() for k in ("obs", "inst", "table", "labels0"))
+    pose = torch.from_numpy(np.ascontiguousarray(d["pose"])).cuda()
+    ctx = dags.Context(rec.shape[0], cam.width, cam.height, 1)
+    cfg = dags.default_mp_cfg()
+    gauss, labels = rec.clone(), lab0.clone()
+    stats = ctx.mp_update(gauss, cam, pose, tg, image, inst, table, labels, cfg, True)
+    torch.cuda.synchronize()
+    want = gauss[:, 11].clone(), labels.clone(), stats.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ctx.mp_update(gauss, cam, pose, tg, image, inst, table, labels, cfg, True, stats=stats)
+    for _ in range(2):
+        gauss.copy_(rec)
+        labels.copy_(lab0)
+        stats.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        ctx.check()
+        # the region sums' float atomics may round differently between runs
+        assert (gauss[:, 11] - want[0]).abs().max().item() <= 1e-6
+        assert (labels != want[1]).sum().item() <= 2
+        assert stats[5].item() == want[2][5].item()
