@@ -382,7 +382,7 @@ def learned_mp_section(args, ctx, dags, synth, image, targets, inst, table, cam,
     return {"workload": f"{B} frames of {cam.width}x{cam.height} x 8 BF16 features per launch",
             "infer_us": round(t_inf, 2), "infer_frames_per_s": round(B / (t_inf * 1e-6), 1),
             "infer_tflops": round(flop / (t_inf * 1e-6) / 1e12, 2), "alg_flop_per_launch": flop,
-            "train_step_us": round(t_tr, 2), "gpu_launches_infer": 1, "gpu_launches_train": 6}
+            "train_step_us": round(t_tr, 2), "gpu_launches_infer": 1, "gpu_launches_train": 5}
 
 
 def mp_section(ctx, dags, gauss, cam, poses, targets, image, inst, table, labels, mp_stats, flush, stream):
@@ -553,8 +553,8 @@ def edge_section(ctx, dags, gauss, cam, tg_all, pose_all, flush, stream):
 def epipolar_section(dags, flush, stream):
     """Epipolar verification and static recovery (Eqs. (18), (19)) on the
     synthetic matches of frames 11 and 16 (300k-Gaussian map, 20k Gaussians
-    with 4 matches each, 0.3 px noise): CUDA events around the call (seven
-    launches: distances, three scan kernels, scatter, medians; one memset),
+    with 4 matches each, 0.3 px noise): CUDA events around the call (four
+    launches: distances, group offsets, scatter, medians; one memset),
     L2 flushed before each; and what the recovery does."""
     import torch
     from paper_2602_21644_gb300 import synth
@@ -586,7 +586,7 @@ def epipolar_section(dags, flush, stream):
     moving = d["moving"]
     return {"workload": f"{len(d['gid'])} matches of {len(np.unique(d['gid']))} Gaussians, frames 11 -> 16, "
                         f"{n} Gaussians",
-            "us": round(1e3 * float(np.median(ts)), 3), "gpu_launches": 7,
+            "us": round(1e3 * float(np.median(ts)), 3), "gpu_launches": 4,
             "restored_static": int((restored & ~moving).sum()), "restored_moving": int((restored & moving).sum()),
             "suppressed_static": int(((d["labels"] == 1) & ~moving).sum())}
 
@@ -983,7 +983,7 @@ def run_ours(args):
     # the forward, the adjoint and the pose chain (pose step fused); per frame
     # the culling and the MP update's 9 kernels (pixel sum, pixel var, pixel map, gauss,
     # apply, 2 select levels, labels, region stats)
-    gpu_launches = args.steps * (args.iters * 4 + 9 + 1)   # + the frame's culling
+    gpu_launches = args.steps * (args.iters * 4 + 5 + 1)   # + the frame's culling
     line = {"metric": METRIC, "value": round(value, 2), "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": round(t_ms / args.steps, 4), "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
