@@ -683,7 +683,7 @@ int track_iteration(dags_ctx *ctx, const float *gauss, int64_t n, const dags_cam
   if (w.bucket_cap == 0) return DAGS_E_INVAL;
   const float4 *g4 = reinterpret_cast<const float4 *>(gauss);
   KernelTimer &tm = ctx->timer;
-  // the pose path accumulates 2D-gradient words G2_U .. G2_Z: two float4
+  // the pose path accumulates 2D-gradient words G2_E .. G2_Z: two float4
   int ev = tm.begin(DAGS_K_PREPROCESS, s);
   // after an iteration, the candidate list is three launches old and the
   // preprocess may load it before waiting for the pose step; after the

@@ -36,14 +36,18 @@ __device__ __forceinline__ bool dags_in_bounds(bool ok, uint32_t *status) {
 #define DAGS_IN_BOUNDS(cond, status) true
 #endif
 
-// 2D gradient slots per (view, Gaussian), sums over the pixels it covers.
-// With g = alpha dL/dalpha (0 where alpha is clamped) and d = centre - pixel:
-//   moments      words 0-4: g dx, g dy, g dx^2, g dx dy, g dy^2, of which the
-//                gradients of centre and conic are linear combinations
+// 2D gradient slots per (view, Gaussian), sums over the pixels it covers. With
+// g = alpha dL/dalpha (0 where alpha is clamped), (dx, dy) = centre - pixel and
+// e = dx + k dy for the conic's shear k = b / a:
+//   moments      words 0-4: g e, g dy, g e^2, g e dy, g dy^2
 //   otherwise    words 0-4: the gradients of the centre (u, v) and of the conic
 //                (a, b, c) themselves
-// and in both the gradient of depth, the sum of g, and those of the colour.
-enum { G2_U = 0, G2_V, G2_A, G2_B, G2_C, G2_Z, G2_S0, G2_R, G2_G, G2_BL };
+// and in both the gradient of depth, the sum of g, and those of the colour. The
+// moments are taken over e because the conic times the offset, of which the
+// gradients of centre and covariance are made, is then a sum of two terms that
+// do not cancel; for a long splat off the axes a dx and b dy nearly do, and sums
+// over dx lose what is left to the rounding of FP32 atomics.
+enum { G2_E = 0, G2_Y, G2_EE, G2_EY, G2_YY, G2_Z, G2_S0, G2_R, G2_G, G2_BL };
 
 // Counters in the workspace's counter array.
 enum {
@@ -391,6 +395,13 @@ __device__ __forceinline__ float hw_rcp(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+
+// The shear k = b / a of the conic (a, b, c) from its entries in log2 units (a',
+// b', see the projected record): approximate, but the same bits wherever it is
+// formed. 0 where a underflows.
+__device__ __forceinline__ float conic_shear(float a2, float b2) {
+  return fabsf(a2) > 1e-30f ? __fmul_rn(__fmul_rn(0.5f, b2), hw_rcp(a2)) : 0.f;
 }
 
 // Two FP32 values in a register pair and the packed operations of sm_100-class

@@ -25,17 +25,16 @@ namespace {
 
 constexpr int kMaxViewsSmem = 64;
 // the pose path's words are the first two float4 (the preprocess zeroes only those)
-static_assert(G2_U == 0 && G2_C == 4 && G2_Z == 5 && G2_BL == 9 && kGradWords >= 10, "2D-gradient word order");
+static_assert(G2_E == 0 && G2_YY == 4 && G2_Z == 5 && G2_BL == 9 && kGradWords >= 10, "2D-gradient word order");
 
 // Warp sums of an entry's moments over the warp's 8 x 4 pixels (lane = 8 row +
-// column). dx depends on the column only and dy on the row only, so m0, m1, m2
-// = g, g dx, g dx^2 and the depth and colour terms are first reduce-scattered
-// over each row's 8 lanes, and the y factors are applied to the row sums: 7 + 2
-// shuffles for the ten words and 4 + 2 for the pose path's six (a
-// reduce-scatter of all words over 32 lanes takes 12 and 8, and needs every
-// word formed per pixel). The terms are given as x = (m1, m2, z, r, g, b, m0),
-// or (m1, m2, z, m0) for the pose path; after the row stage lane l8 = lane & 7
-// holds
+// column). dy depends on the row only, so m0, m1, m2 = g, g e, g e^2 and the
+// depth and colour terms are first reduce-scattered over each row's 8 lanes, and
+// the y factors are applied to the row sums: 7 + 2 shuffles for the ten words
+// and 4 + 2 for the pose path's six (a reduce-scatter of all words over 32 lanes
+// takes 12 and 8, and needs every word formed per pixel). The terms are given as
+// x = (m1, m2, z, r, g, b, m0), or (m1, m2, z, m0) for the pose path; after the
+// row stage lane l8 = lane & 7 holds
 //   FULL:      m1, m2, z, m0, r, g, b, m0
 //   pose only: m1, m1, m2, m2, z, z, m0, m0
 // and the rows are summed as is by the lanes below 16, weighted with dy by the
@@ -45,11 +44,11 @@ template <bool FULL>
 __device__ __forceinline__ int moment_word(int lane) {
   const int l8 = lane & 7;
   if (lane & 8) return -1;
-  if (lane & 16) return l8 == 0 ? G2_B : (l8 == (FULL ? 3 : 6) ? G2_V : -1);
-  if (l8 == 0) return G2_U;
-  if (l8 == 7) return G2_C;
-  if (FULL) return l8 == 1 ? G2_A : l8 == 2 ? G2_Z : l8 == 3 ? G2_S0 : l8 == 4 ? G2_R : l8 == 5 ? G2_G : G2_BL;
-  return l8 == 2 ? G2_A : l8 == 4 ? G2_Z : -1;
+  if (lane & 16) return l8 == 0 ? G2_EY : (l8 == (FULL ? 3 : 6) ? G2_Y : -1);
+  if (l8 == 0) return G2_E;
+  if (l8 == 7) return G2_YY;
+  if (FULL) return l8 == 1 ? G2_EE : l8 == 2 ? G2_Z : l8 == 3 ? G2_S0 : l8 == 4 ? G2_R : l8 == 5 ? G2_G : G2_BL;
+  return l8 == 2 ? G2_EE : l8 == 4 ? G2_Z : -1;
 }
 
 template <int K>
@@ -65,7 +64,7 @@ __device__ __forceinline__ float moment_sums(const float (&x)[K], float dy, int 
 }
 
 // FULL: every parameter's 2D gradients (else the pose path's six words);
-// MOMENTS: words 0-4 as moments (see G2_U), else as gradients formed per pixel;
+// MOMENTS: words 0-4 as moments (see G2_E), else as gradients formed per pixel;
 // MASKS: visit only the entries the forward recorded as taken by the warp
 // (ws.warp_masks); COUNT: count evaluations and contributions (ws.evals).
 // One warp, and one CTA, per 8 x 4 pixel block: no barrier joins the blocks of a
@@ -225,19 +224,18 @@ render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ tar
     // alpha does not move with the exponent)
     const float dpw = contrib && ag <= r.alpha_max ? dal * alpha : 0.f;
     const float gz = g3 * wk;
-    const float tx = dpw * dx;
     Sg = fmaf(gcv, wk, Sg);
     id = __float_as_uint(d.w);
-    if constexpr (MOMENTS && FULL) {
-      x[0] = tx; x[1] = tx * dx; x[2] = gz; x[3] = g0 * wk; x[4] = g1 * wk; x[5] = g2 * wk; x[6] = dpw;
-    } else if constexpr (MOMENTS) {
-      x[0] = tx; x[1] = tx * dx; x[2] = gz; x[3] = dpw;
+    if constexpr (MOMENTS) {
+      const float e = fmaf(d.y, dy, dx), te = dpw * e;
+      x[0] = te; x[1] = te * e; x[2] = gz; x[kTerms - 1] = dpw;
+      if constexpr (FULL) { x[3] = g0 * wk; x[4] = g1 * wk; x[5] = g2 * wk; }
     } else {
       // the exponent in log2 units is p, so d/dx of the natural exponent is
       // ln2 dp/dx: d p / d(u, v) = (2 a' dx + b' dy, b' dx + 2 c' dy) from the
       // exponent's products; d(natural exponent) / d(conic) = -(dx^2 / 2,
       // dx dy, dy^2 / 2)
-      const float hl = dpw * kLn2, ty = dpw * dy;
+      const float hl = dpw * kLn2, tx = dpw * dx, ty = dpw * dy;
       x[0] = hl * fmaf(2.f, bxdx, b.y * dy); x[1] = hl * fmaf(2.f, bzdy, bydx); x[2] = -0.5f * (tx * dx);
       x[3] = -(tx * dy); x[4] = -0.5f * (ty * dy); x[5] = gz; x[6] = dpw; x[7] = g0 * wk; x[8] = g1 * wk;
       x[9] = g2 * wk;
@@ -267,18 +265,19 @@ render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ tar
     mask_next = 0u;
     if (g > 1) group(g - 2, id_next, mask_next);
     asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncwarp();
+    // the lane's own entry: whether its box meets the block, and the conic's
+    // shear in place of the box's half width
     const float4(*const rec)[32] = s_rec[cur];
     const bool recorded = MASKS && g < kMaskGroups;
-    if (!recorded) {
-      // later groups, or no record: the entries whose box meets the block
-      bool hit = false;
-      if ((mask >> lane) & 1u) {
-        const float4 a = rec[0][lane], d = rec[3][lane];
-        hit = fabsf(a.x - bcx) <= d.y + 3.5f && fabsf(a.y - bcy) <= d.z + 1.5f;
-      }
-      mask = __ballot_sync(FULLM, hit);
+    bool hit = false;
+    if ((mask >> lane) & 1u) {
+      const float4 a = rec[0][lane], b = rec[1][lane], d = rec[3][lane];
+      hit = fabsf(a.x - bcx) <= d.y + 3.5f && fabsf(a.y - bcy) <= d.z + 1.5f;
+      if (MOMENTS) s_rec[cur][3][lane].y = conic_shear(b.x, b.y);
     }
+    // without a record (later groups, or none): the entries that passed
+    if (!recorded) mask = __ballot_sync(FULLM, hit);
+    __syncwarp();
     // two entries at a time: the second's arithmetic and reduction fill the
     // latencies of the first's
     while (mask) {
@@ -307,36 +306,57 @@ render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ tar
   if (ws.bucket_cap && warp == 0 && lane == 0) ws.tile_count[tile] = 0u;
 }
 
+// A projection with what the chain makes of its conic. The exponent is
+// -(d^T Q d) / 2 over the offset d = (dx, dy) with the conic Q = [[a, b], [b, c]],
+// and Q d = (a e + h dy, b e + s dy) with e = dx + k dy: k is b / a up to its
+// rounding, so h = b - a k is that rounding's remainder and s = c - b k is 1 / C,
+// the inverse of a covariance entry. Neither is formed as a difference of conic
+// entries, which cancels as the square of the splat's aspect ratio.
+struct ChainProj : Proj {
+  float h, s;
+};
+__device__ __forceinline__ void chain_factors(ChainProj &q) {
+  const float k = conic_shear(__fmul_rn(-0.5f * kLog2e, q.ca), __fmul_rn(-kLog2e, q.cb));
+  const float rem = fmaf(-k, q.C, -q.B);
+  q.h = rem * __fdiv_rn(1.f, q.det);
+  q.s = fmaf(q.cb, rem, 1.f) / q.C;
+}
+
 // Chains the 2D gradients of the Gaussian projected as q in view slot `slot`
 // (pose Pm) to the pose twist (pg, added) and, FULL, to the record's
 // parameters (acc, added).
 template <bool FULL, bool MOMENTS>
-__device__ __forceinline__ void chain_proj(const Workspace &ws, const Raster &r, const Proj &q, const float *Pm,
+__device__ __forceinline__ void chain_proj(const Workspace &ws, const Raster &r, const ChainProj &q, const float *Pm,
                                            size_t slot, float *pg, float *acc) {
   const float *gd = ws.grad2d + slot * kGradWords;
   const float4 ga4 = *reinterpret_cast<const float4 *>(gd);
   const float4 gb4 = *reinterpret_cast<const float4 *>(gd + 4);
-  float gu = ga4.x, gv = ga4.y, gA = ga4.z, gB = ga4.w, gC = gb4.x;
   const float gzz = gb4.y;
+  float gu, gv, d00, d01, d11;   // gradients of the centre and of the 2D covariance
   if constexpr (MOMENTS) {
-    // the natural exponent is -(a dx^2 / 2 + b dx dy + c dy^2 / 2) for the
-    // conic (a, b, c): d/du = -(a Sx + b Sy), d/d(a, b, c) = -(Sxx / 2, Sxy,
-    // Syy / 2)
-    gu = -fmaf(q.ca, ga4.x, q.cb * ga4.y);
-    gv = -fmaf(q.cc, ga4.y, q.cb * ga4.x);
-    gA *= -0.5f;
-    gB = -gB;
-    gC *= -0.5f;
+    // d/d(u, v) = -sum g Q d
+    gu = -fmaf(q.ca, ga4.x, q.h * ga4.y);
+    gv = -fmaf(q.cb, ga4.x, q.s * ga4.y);
+    // dS = sum g (Q d)(Q d)^T / 2: the sums of g (Q d)_u (e, dy) and of g (Q d)_v (e, dy)
+    const float t0e = q.ca * ga4.z + q.h * ga4.w, t0y = q.ca * ga4.w + q.h * gb4.x;
+    const float t1e = q.cb * ga4.z + q.s * ga4.w, t1y = q.cb * ga4.w + q.s * gb4.x;
+    d00 = 0.5f * (t0e * q.ca + t0y * q.h);
+    d01 = 0.5f * (t0e * q.cb + t0y * q.s);
+    d11 = 0.5f * (t1e * q.cb + t1y * q.s);
+  } else {
+    gu = ga4.x;
+    gv = ga4.y;
+    // conic -> 2D covariance: dS = -Q Gq Q with Gq the symmetric-matrix form of
+    // the conic gradient (the off-diagonal appears twice in the quadratic form)
+    const float gA = ga4.z, gB = ga4.w, gC = gb4.x;
+    const float qa = q.ca, qb = q.cb, qc = q.cc;
+    const float h = 0.5f * gB;
+    const float t00 = qa * gA + qb * h, t01 = qa * h + qb * gC;
+    const float t10 = qb * gA + qc * h, t11 = qb * h + qc * gC;
+    d00 = -(t00 * qa + t01 * qb);
+    d01 = -(t00 * qb + t01 * qc);
+    d11 = -(t10 * qb + t11 * qc);
   }
-  // conic -> 2D covariance: dS = -Q Gq Q with Gq the symmetric-matrix form of
-  // the conic gradient (the off-diagonal appears twice in the quadratic form)
-  const float qa = q.ca, qb = q.cb, qc = q.cc;
-  const float h = 0.5f * gB;
-  const float t00 = qa * gA + qb * h, t01 = qa * h + qb * gC;
-  const float t10 = qb * gA + qc * h, t11 = qb * h + qc * gC;
-  const float d00 = -(t00 * qa + t01 * qb);
-  const float d01 = -(t00 * qb + t01 * qc);
-  const float d11 = -(t10 * qb + t11 * qc);
   // Sigma' = M2 M2^T + d I with M2 = J K: dM2 = 2 dS M2
   float dm0[3], dm1[3];
 #pragma unroll
@@ -425,19 +445,22 @@ __device__ __forceinline__ void chain_proj(const Workspace &ws, const Raster &r,
 
 // Whether the Gaussian of view slot `slot` has a non-empty tile range, and if
 // so its projection.
+template <bool MOMENTS>
 __device__ __forceinline__ bool visible_proj(const Workspace &ws, const Raster &r, const float4 &g0,
                                              const float4 &g1, const float4 &g2, const float *Pm, size_t slot,
-                                             Proj &q) {
+                                             ChainProj &q) {
   const uint2 rc = ws.rect[slot];
-  return (rc.x >> 16) > (rc.x & 0xFFFF) && project_gaussian(g0, g1, g2, Pm, r, q);
+  if ((rc.x >> 16) <= (rc.x & 0xFFFF) || !project_gaussian(g0, g1, g2, Pm, r, q)) return false;
+  if (MOMENTS) chain_factors(q);
+  return true;
 }
 
 // chain_proj of Gaussian (g0, g1, g2) when it is visible.
 template <bool FULL, bool MOMENTS>
 __device__ __forceinline__ void chain_one(const Workspace &ws, const Raster &r, const float4 &g0, const float4 &g1,
                                           const float4 &g2, const float *Pm, size_t slot, float *pg, float *acc) {
-  Proj q;
-  if (visible_proj(ws, r, g0, g1, g2, Pm, slot, q)) chain_proj<FULL, MOMENTS>(ws, r, q, Pm, slot, pg, acc);
+  ChainProj q;
+  if (visible_proj<MOMENTS>(ws, r, g0, g1, g2, Pm, slot, q)) chain_proj<FULL, MOMENTS>(ws, r, q, Pm, slot, pg, acc);
 }
 
 // Compensated (double-FP32) addition: (h, l) += (bh, bl) through two-sum,
@@ -475,8 +498,12 @@ __device__ __forceinline__ void store_pose_partial(const Workspace &ws, float *p
 // !FULL (pose only): a fixed grid strides over the Gaussians of each view.
 // The last CTA sums the pose partials in a fixed order in FP64 (one warp per
 // twist component) and, if ps.poses is set, applies the pose step.
+// The pose-only form keeps to 96 registers, five CTAs per SM: its grid of four
+// per SM and the ranking CTA are then one wave (at 104 registers and four CTAs
+// per SM the ranking CTA pushes one out, and an iteration of the tracking loop
+// takes 3 us more).
 template <bool FULL, bool MOMENTS>
-__global__ void __launch_bounds__(kBwdPrepBlock)
+__global__ void __launch_bounds__(kBwdPrepBlock, FULL ? 1 : 5)
 preprocess_bwd_kernel(Workspace ws, const float4 *__restrict__ gauss, int64_t n, int views, Raster r,
                       float *__restrict__ grad_gauss, double *__restrict__ grad_pose, PoseStep ps) {
   // pose only, tracking loop: the grid's first CTA (dispatched first, so
@@ -500,7 +527,7 @@ preprocess_bwd_kernel(Workspace ws, const float4 *__restrict__ gauss, int64_t n,
   // and the FP32 pose were written two or more launches before this one, so
   // each thread projects its first visible Gaussian before waiting for the
   // adjoint, whose 2D gradients it reads after the wait
-  Proj q0;
+  ChainProj q0;
   bool pre = false, pre_vis = false;
   // the pose step's bias corrections depend only on the Adam step count,
   // written by the previous iteration's step (three launches back): every
@@ -523,7 +550,7 @@ preprocess_bwd_kernel(Workspace ws, const float4 *__restrict__ gauss, int64_t n,
       if (DAGS_IN_BOUNDS(i >= 0 && i < n, ws.counters + CNT_STATUS)) {
         pre_slot = (size_t)i;
         const float4 g0 = __ldg(gauss + 4 * i + 0), g1 = __ldg(gauss + 4 * i + 1), g2 = __ldg(gauss + 4 * i + 2);
-        pre_vis = visible_proj(ws, r, g0, g1, g2, sp, pre_slot, q0);
+        pre_vis = visible_proj<MOMENTS>(ws, r, g0, g1, g2, sp, pre_slot, q0);
       }
     }
   }
@@ -652,14 +679,16 @@ preprocess_bwd_kernel(Workspace ws, const float4 *__restrict__ gauss, int64_t n,
 
 }  // namespace
 
-// Whether the 2D gradients are accumulated as moments. They are, except where
-// the Gaussian and the twist gradients are both asked for: the twist gradient
-// cancels by two to three digits over the map, and a caller that takes it in
-// FP64 beside the map's gradients gets it with the rounding of the per-pixel
-// form (either form is about 3e-7 from 64 bits on the 2,000-Gaussian scene).
-// Gradients of 200k Gaussians over 8 views of 640x480: the adjoint takes 333 us
-// with moments over the entries the forward recorded, 421 us per pixel over
-// every entry whose box meets the warp's block.
+// Whether the 2D gradients are accumulated as moments: not where the Gaussian
+// and the twist gradients are both asked for. Moments are the faster form (the
+// adjoint of one frame, 300k Gaussians, 640x480, all gradients over recorded
+// entries: 59 against 66 us) and no less exact: against 64 bits the twist of
+// 2,000 Gaussians is 2.5e-7 off from moments and 2.9e-7 from words per pixel
+// (means of six scenes), that of discs seen edge-on with a standard deviation
+// of 2 to 110 px 1e-6 .. 1e-5 and 1e-6 .. 5e-4. But the two differ by what
+// either is off, 3e-7 there and 4e-8 on the 300k frame, three times what the
+// order of the atomics does, and a caller of both takes the twist as FP64:
+// those results stay as they were.
 static bool backward_moments(bool full, bool pose) { return !(full && pose); }
 
 cudaError_t launch_render_bwd(const Workspace &ws, int views, int64_t n, const Raster &r, const Loss &l,
