@@ -209,12 +209,13 @@ render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ tar
     const bool contrib = k < lastp && p >= r.log2_alpha_min;
     if (COUNT) { n_eval += k < lastp ? 1u : 0u; n_contrib += contrib ? 1u : 0u; }
     const float ag = hw_exp2(p);
-    // zero for a lane that does not take the entry: 1 / (1 - alpha) is
-    // then exactly 1, T is kept, and the weight and the suffix update
-    // vanish without a select
+    // zero for a lane that does not take the entry: the weight and the suffix
+    // update vanish without a select
     const float alpha = contrib ? fminf(r.alpha_max, ag) : 0.f;
     const float inv = hw_rcp(1.f - alpha);
-    T *= inv;                            // transmittance in front of this Gaussian
+    // transmittance in front of this Gaussian; kept, whatever the approximate
+    // reciprocal makes of 1, by a lane that does not take it
+    if (contrib) T *= inv;
     const float wk = alpha * T;
     const float4 c = rec[2][j], d = rec[3][j];
     // dL/dalpha = sum_ch g_ch (c_ch T - S_ch / (1 - alpha))
