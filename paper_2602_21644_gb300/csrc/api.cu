@@ -814,6 +814,9 @@ int splat_track(dags_ctx *ctx, const float *gauss, int64_t n, const dags_camera 
     g.key_len = kl;
   }
   ctx->last_stream = s;
+  // a replay leaves the workspace as an enqueued iteration does: without the
+  // last forward's lists, records and masks
+  if (iters > 0) ctx->fwd_image = nullptr;
   int left = iters;
   for (; left >= kTrackUnroll; left -= kTrackUnroll)
     if (cudaGraphLaunch(g.exec_chunk, s) != cudaSuccess) return DAGS_E_CUDA;
@@ -1042,6 +1045,9 @@ int splat_track_lm(dags_ctx *ctx, const float *gauss, int64_t n, const dags_came
     g.key_len = kl;
   }
   ctx->last_stream = s;
+  // a replay leaves the workspace as an enqueued iteration does: without the
+  // last forward's lists, records and masks
+  if (iters > 0) ctx->fwd_image = nullptr;
   int left = iters;
   for (; left >= kTrackUnroll; left -= kTrackUnroll)
     if (cudaGraphLaunch(g.exec_chunk, s) != cudaSuccess) return DAGS_E_CUDA;
