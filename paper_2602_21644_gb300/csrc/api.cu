@@ -843,9 +843,14 @@ int ensure_lm(dags_ctx *ctx) {
   A(alloc(&b.done, tiles + groups + 1));
   A(alloc(&b.normal, (size_t)DAGS_LM_NORMAL));
   A(alloc(&b.pose_try, (size_t)12));
-  // (synchronous: the first call's kernels may be on any stream)
-  if (e == cudaSuccess) e = cudaMemset(b.done, 0, (tiles + groups + 1) * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  // zeroed before the call returns, whatever stream the next call is on, but on
+  // a stream of its own: a device-wide wait would wait for the caller's other
+  // work, and end any stream capture under way in another thread
+  cudaStream_t z = nullptr;
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&z, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b.done, 0, (tiles + groups + 1) * sizeof(uint32_t), z);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(z);
+  if (z) cudaStreamDestroy(z);
   if (e != cudaSuccess) {
     cudaGetLastError();
     free_lm(b);
