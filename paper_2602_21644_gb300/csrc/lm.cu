@@ -274,7 +274,7 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
 // sorts its bucket, scalar (93M warp instructions) or packed (77M, the same
 // time: the tile's CTAs wait on one another); 129 us with a warp per block and
 // the sort beside the tangents (60M); 125 with the sums and the step spread
-// over warps and lanes; 121 without branches, the next entry read ahead.
+// over warps and lanes; 121 with the next entry read ahead.
 __global__ void __launch_bounds__(32, 20)
 render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__restrict__ targets,
                   const float4 *__restrict__ tan, LmBuffers buf, double *__restrict__ normal,
@@ -384,10 +384,9 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
     for (int j = 0; mask; ++j) {
       const int bit = __ffs((int)mask) - 1;
       mask &= mask - 1;
-      // evaluated by every lane, without branches: a lane that is done, or
-      // whose alpha is below alpha_min, or that would stop here carries zero
-      // weights (x + 0 * c == x), so each pixel's sums are those of the
-      // branching form, operation for operation
+      // alpha is evaluated by every lane; a lane that is done, or whose alpha
+      // is below alpha_min, or that would stop here leaves the sums alone (a
+      // zero weight would not: a Gaussian's colour may be infinite)
       const float dx = (a.x - fpx) + a.z, dy = (a.y - fpy) + a.w;
       const float p = fmaf(b.x * dx, dx, fmaf(b.y * dx, dy, fmaf(b.z * dy, dy, b.w)));
       const bool live = !done && p >= r.log2_alpha_min;
@@ -403,37 +402,38 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
       // of the staging buffer that nothing uses)
       a = rec[0][j + 1];
       b = rec[1][j + 1];
-      if (!__any_sync(FULL, contrib)) continue;
-      const float w = contrib ? alpha * T : 0.f;
-      const float4 c = rec[2][j];
-      const float blue = rec[3][j].x;
-      cr += c.z * w; cg += c.w * w; cb += blue * w;
-      dd += c.x * w; oo += w; rm += c.y * w;
-      // tangents: p' = da' dx^2 + db' dx dy + dc' dy^2 + dp/du du + dp/dv dv,
-      // alpha' = alpha ln2 p' (0 where clamped), weight' = alpha' T + alpha T';
-      // the next entry's T = T - weight, so its T' = T' - weight'
-      const f32x2 gx = dup2(gxs), gy = dup2(gys);
-      const f32x2 pdx = dup2(dx), pdy = dup2(dy);
-      const f32x2 dx2 = mul2(pdx, pdx), dxy = mul2(pdx, pdy), dy2 = mul2(pdy, pdy);
-      const f32x2 aln = dup2(contrib && !clamped ? alpha * kLn2 : 0.f), al2 = dup2(contrib ? alpha : 0.f);
-      const f32x2 T2 = dup2(T), w2 = dup2(w);
-      const f32x2 cz2 = dup2(c.x), cr2 = dup2(c.z), cg2 = dup2(c.w), cb2 = dup2(blue);
+      if (contrib) {
+        const float w = alpha * T;
+        const float4 c = rec[2][j];
+        const float blue = rec[3][j].x;
+        cr += c.z * w; cg += c.w * w; cb += blue * w;
+        dd += c.x * w; oo += w; rm += c.y * w;
+        // tangents: p' = da' dx^2 + db' dx dy + dc' dy^2 + dp/du du + dp/dv dv,
+        // alpha' = alpha ln2 p' (0 where clamped), weight' = alpha' T + alpha T';
+        // the next entry's T = T - weight, so its T' = T' - weight'
+        const f32x2 gx = dup2(gxs), gy = dup2(gys);
+        const f32x2 pdx = dup2(dx), pdy = dup2(dy);
+        const f32x2 dx2 = mul2(pdx, pdx), dxy = mul2(pdx, pdy), dy2 = mul2(pdy, pdy);
+        const f32x2 aln = dup2(clamped ? 0.f : alpha * kLn2), al2 = dup2(alpha);
+        const f32x2 T2 = dup2(T), w2 = dup2(w);
+        const f32x2 cz2 = dup2(c.x), cr2 = dup2(c.z), cg2 = dup2(c.w), cb2 = dup2(blue);
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const ulonglong2 uv = *reinterpret_cast<const ulonglong2 *>(&rec[4 + 3 * k][j]);
-        const ulonglong2 ab = *reinterpret_cast<const ulonglong2 *>(&rec[5 + 3 * k][j]);
-        const ulonglong2 cz = *reinterpret_cast<const ulonglong2 *>(&rec[6 + 3 * k][j]);
-        const f32x2 dp = fma2(ab.x, dx2, fma2(ab.y, dxy, fma2(cz.x, dy2, fma2(gx, uv.x, mul2(gy, uv.y)))));
-        const f32x2 da = mul2(aln, dp);
-        const f32x2 dw = fma2(da, T2, mul2(al2, dT2[k]));
-        jr2[k] = fma2(cr2, dw, jr2[k]);
-        jg2[k] = fma2(cg2, dw, jg2[k]);
-        jb2[k] = fma2(cb2, dw, jb2[k]);
-        jd2[k] = fma2(cz2, dw, fma2(w2, cz.y, jd2[k]));
-        dT2[k] = fma2(dw, minus1, dT2[k]);
+        for (int k = 0; k < 3; ++k) {
+          const ulonglong2 uv = *reinterpret_cast<const ulonglong2 *>(&rec[4 + 3 * k][j]);
+          const ulonglong2 ab = *reinterpret_cast<const ulonglong2 *>(&rec[5 + 3 * k][j]);
+          const ulonglong2 cz = *reinterpret_cast<const ulonglong2 *>(&rec[6 + 3 * k][j]);
+          const f32x2 dp = fma2(ab.x, dx2, fma2(ab.y, dxy, fma2(cz.x, dy2, fma2(gx, uv.x, mul2(gy, uv.y)))));
+          const f32x2 da = mul2(aln, dp);
+          const f32x2 dw = fma2(da, T2, mul2(al2, dT2[k]));
+          jr2[k] = fma2(cr2, dw, jr2[k]);
+          jg2[k] = fma2(cg2, dw, jg2[k]);
+          jb2[k] = fma2(cb2, dw, jb2[k]);
+          jd2[k] = fma2(cz2, dw, fma2(w2, cz.y, jd2[k]));
+          dT2[k] = fma2(dw, minus1, dT2[k]);
+        }
+        T = tt;
+        lastk = kbase + bit;
       }
-      T = contrib ? tt : T;
-      lastk = contrib ? kbase + bit : lastk;
     }
     __syncwarp();   // the chunk's buffer is staged again in the next round
     if (__all_sync(FULL, done)) break;
