@@ -256,6 +256,7 @@ __device__ __forceinline__ bool arrive_last(uint32_t *counter, uint32_t count) {
       __threadfence();
     }
   }
+  __syncwarp();   // the fence orders lane 0's view; this passes it on to the other lanes
   return __shfl_sync(0xffffffffu, t, 0) == count - 1u;
 }
 
