@@ -281,8 +281,9 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
                   const float4 *__restrict__ tan, LmBuffers buf, double *__restrict__ normal,
                   float *__restrict__ jac, float *__restrict__ image, int32_t *__restrict__ last, LmFuse fuse) {
   pdl_wait();
-  // records and tangent records of a chunk's entries, double-buffered
-  __shared__ float4 s_rec[2][4 + kTan4][kJacChunk];
+  // records and tangent records of a chunk's entries, double-buffered: word w of
+  // entry j at w * kJacChunk + j
+  __shared__ float4 s_rec[2][(4 + kTan4) * kJacChunk];
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x;
   const int warp = (int)(blockIdx.x % kBlocks);   // the tile's pixel block
@@ -364,9 +365,9 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
     if (take) {
       const float4 *rec = ws.rec2d + (size_t)pid * 4, *tg = tan + (size_t)pid * kTan4;
 #pragma unroll
-      for (int w = 0; w < 4; ++w) cp_async16(&s_rec[b][w][rank], rec + w);
+      for (int w = 0; w < 4; ++w) cp_async16(&s_rec[b][w * kJacChunk + rank], rec + w);
 #pragma unroll
-      for (int w = 0; w < kTan4; ++w) cp_async16(&s_rec[b][4 + w][rank], tg + w);
+      for (int w = 0; w < kTan4; ++w) cp_async16(&s_rec[b][(4 + w) * kJacChunk + rank], tg + w);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
     const unsigned chunk = __ballot_sync(FULL, take);
@@ -380,8 +381,8 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
     mask_next = stage(cur ^ 1);
     asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncwarp();
-    const float4(*const rec)[kJacChunk] = s_rec[cur];
-    float4 a = rec[0][0], b = rec[1][0];
+    const float4 *const rec = s_rec[cur];
+    float4 a = rec[0], b = rec[kJacChunk];
     for (int j = 0; mask; ++j) {
       const int bit = __ffs((int)mask) - 1;
       mask &= mask - 1;
@@ -399,14 +400,14 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
       const bool contrib = live && !stop;
       done = done || stop;
       const float gxs = fmaf(2.f * b.x, dx, b.y * dy), gys = fmaf(b.y, dx, 2.f * b.z * dy);
-      // the next entry's centre and conic (past the chunk's last, stale values
-      // of the staging buffer that nothing uses)
-      a = rec[0][j + 1];
-      b = rec[1][j + 1];
+      // the next entry's centre and conic (past the chunk's last, the buffer's
+      // following word, which nothing uses)
+      a = rec[j + 1];
+      b = rec[kJacChunk + j + 1];
       if (contrib) {
         const float w = alpha * T;
-        const float4 c = rec[2][j];
-        const float blue = rec[3][j].x;
+        const float4 c = rec[2 * kJacChunk + j];
+        const float blue = rec[3 * kJacChunk + j].x;
         cr += c.z * w; cg += c.w * w; cb += blue * w;
         dd += c.x * w; oo += w; rm += c.y * w;
         // tangents: p' = da' dx^2 + db' dx dy + dc' dy^2 + dp/du du + dp/dv dv,
@@ -420,9 +421,9 @@ render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__r
         const f32x2 cz2 = dup2(c.x), cr2 = dup2(c.z), cg2 = dup2(c.w), cb2 = dup2(blue);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          const ulonglong2 uv = *reinterpret_cast<const ulonglong2 *>(&rec[4 + 3 * k][j]);
-          const ulonglong2 ab = *reinterpret_cast<const ulonglong2 *>(&rec[5 + 3 * k][j]);
-          const ulonglong2 cz = *reinterpret_cast<const ulonglong2 *>(&rec[6 + 3 * k][j]);
+          const ulonglong2 uv = *reinterpret_cast<const ulonglong2 *>(&rec[(4 + 3 * k) * kJacChunk + j]);
+          const ulonglong2 ab = *reinterpret_cast<const ulonglong2 *>(&rec[(5 + 3 * k) * kJacChunk + j]);
+          const ulonglong2 cz = *reinterpret_cast<const ulonglong2 *>(&rec[(6 + 3 * k) * kJacChunk + j]);
           const f32x2 dp = fma2(ab.x, dx2, fma2(ab.y, dxy, fma2(cz.x, dy2, fma2(gx, uv.x, mul2(gy, uv.y)))));
           const f32x2 da = mul2(aln, dp);
           const f32x2 dw = fma2(da, T2, mul2(al2, dT2[k]));
