@@ -368,6 +368,9 @@ void dags_default_mp_cfg(dags_mp_cfg *cfg);
  *           residual terms and region statistics are the frame's own.
  * mp_pixel  device out, H*W floats, or NULL: the fused M_p of Eq. (7) per
  *           pixel (the method's own map, e.g. a training target).
+ * The update ends in a cooperative launch whose CTAs wait for one another,
+ * within a bound; if that runs out (DAGS_E_TIMEOUT) the records' MP words may
+ * have been updated, labels and stats have not.
  * Needs a ctx created with max_views >= 1 and images at least H x W. */
 int mp_update(dags_ctx *ctx, float *gauss, int64_t n, const dags_camera *cam, const double *pose,
               const float *targets, const float *image, const uint8_t *inst, const float *table,
@@ -619,9 +622,10 @@ int mpnet_train_step(dags_ctx *ctx, void *weights, float *master, float *adam_m,
 
 /* Failure-path self-test (no paper counterpart): one device thread waits,
  * for `spins` bounded iterations, on an mbarrier phase that nothing
- * completes - the same bounded wait the tensor-core kernels use - and records
- * DAGS_E_TIMEOUT in the ctx's status word, which the next dags_sync_status
- * returns and clears. Nothing hangs or faults; the ctx stays usable.
+ * completes - the same bounded wait the tensor-core kernels use - and then a
+ * CTA as long for an arrival at mp_update's grid barrier that nothing makes.
+ * Where both give up, DAGS_E_TIMEOUT is recorded in the ctx's status word,
+ * which the next dags_sync_status returns and clears. Nothing hangs or faults; the ctx stays usable.
  * 0 <= spins <= 2^24, else DAGS_E_INVAL. */
 int dags_selftest_timeout(dags_ctx *ctx, int64_t spins, void *stream);
 

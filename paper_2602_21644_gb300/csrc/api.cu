@@ -1329,7 +1329,11 @@ int dags_selftest_timeout(dags_ctx *ctx, int64_t spins, void *stream) {
   if (!ctx || spins < 0 || spins > (1ll << 24)) return DAGS_E_INVAL;
   cudaStream_t s = (cudaStream_t)stream;
   ctx->last_stream = s;
-  return cuda_status(launch_selftest_wait(ctx->ws.counters + CNT_STATUS, (long long)spins, s));
+  uint32_t *scratch = ctx->mp.sel + 4;
+  cudaError_t e = cudaMemsetAsync(scratch, 0, 3 * sizeof(uint32_t), s);
+  if (e == cudaSuccess) e = launch_selftest_wait(scratch + 1, (long long)spins, s);
+  if (e == cudaSuccess) e = launch_selftest_barrier(scratch, (int)spins, ctx->ws.counters + CNT_STATUS, s);
+  return cuda_status(e);
 }
 
 int dags_timing_enable(dags_ctx *ctx, int enable) {

@@ -289,6 +289,7 @@ inline long long mpnet_plane_size(int batch, int W, int H) {
   return (long long)batch * H * 4 * ((long long)(W + kMpnetStrip - 1) / kMpnetStrip * kMpnetStrip + 2);
 }
 cudaError_t launch_selftest_wait(uint32_t *status, long long limit, cudaStream_t s);
+cudaError_t launch_selftest_barrier(uint32_t *scratch, int spins, uint32_t *status, cudaStream_t s);
 cudaError_t launch_mpnet_train(void *weights, float *master, float *adam_m, float *adam_v, int step,
                                const uint16_t *feats, const float *target, int batch, int W, int H, float lr,
                                double *loss, const MpnetScratch &sc, uint32_t *status, int num_sms, cudaStream_t s);
@@ -309,7 +310,7 @@ struct MpBuffers {
   float *mhat = nullptr, *sige = nullptr, *U = nullptr, *Mt = nullptr, *Ut = nullptr;  // [max_n]
   uint32_t *idx = nullptr;            // [max_n]
   uint32_t *hist = nullptr;           // [3 * 2 * 2048]
-  uint32_t *sel = nullptr;            // [8]
+  uint32_t *sel = nullptr;            // [8]: four of the update, four of the self-test
 };
 cudaError_t launch_semantic_trigger(const double *stats, const dags_sched_cfg &cfg, int seg_refreshed,
                                     int32_t *state, double *score, cudaStream_t s);

@@ -428,15 +428,15 @@ constexpr int kApplyHeld = 8;      // list entries that a thread keeps in regist
 constexpr int kBarrierSpins = 1 << 22;
 
 // All CTAs of the grid (a cooperative launch) have arrived `round` times;
-// false if one did not within the spin limit.
-__device__ bool grid_barrier(uint32_t *arrivals, uint32_t round, uint32_t *status) {
+// false, with the timeout recorded, if one did not within `spins` iterations.
+__device__ bool grid_barrier(uint32_t *arrivals, uint32_t round, int spins, uint32_t *status) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(arrivals, 1u);
     bool ok = false;
-    for (int it = 0; it < kBarrierSpins && !ok; ++it) {
+    for (int it = 0; it < spins && !ok; ++it) {
       uint32_t v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(arrivals) : "memory");
       ok = v >= round * gridDim.x;
@@ -447,6 +447,16 @@ __device__ bool grid_barrier(uint32_t *arrivals, uint32_t round, uint32_t *statu
   }
   __syncthreads();
   return s_ok != 0;
+}
+
+// Failure-path self-test: the one CTA waits for a second arrival that nothing
+// makes. scratch[0] counts arrivals, [1] is the status that an earlier wait
+// recorded its timeout in, [2] this one's; the ctx's status gets the timeout if
+// both did.
+__global__ void selftest_barrier_kernel(uint32_t *scratch, int spins, uint32_t *status) {
+  const bool ok = grid_barrier(scratch, 2u, spins, scratch + 2);
+  if (threadIdx.x == 0 && !ok && (__ldcg(scratch + 1) & __ldcg(scratch + 2) & kStatusTimeout))
+    atomicOr(status, kStatusTimeout);
 }
 
 // Radix-select level l of the floats' bits: 31-21, 20-10, 9-0.
@@ -565,7 +575,7 @@ mp_apply_kernel(MpWs m, float *__restrict__ gauss, uint8_t *__restrict__ labels,
     uint32_t *hist = m.hist + level * 2 * kSelBins;
     for (int k = threadIdx.x; k < 2 * kSelBins; k += kApplyBlock)
       if (s_h[k]) atomicAdd(&hist[k], s_h[k]);
-    if (!grid_barrier(m.sel + 3, (uint32_t)level + 1u, m.status)) return;
+    if (!grid_barrier(m.sel + 3, (uint32_t)level + 1u, kBarrierSpins, m.status)) return;
     uint32_t bin[2];
     find_bins(hist, rank, bin);
     prefix[0] |= bin[0] << shift;
@@ -609,6 +619,11 @@ __global__ void semantic_trigger_kernel(const double *__restrict__ stats, double
 }
 
 }  // namespace
+
+cudaError_t launch_selftest_barrier(uint32_t *scratch, int spins, uint32_t *status, cudaStream_t s) {
+  selftest_barrier_kernel<<<1, 32, 0, s>>>(scratch, spins < kBarrierSpins ? spins : kBarrierSpins, status);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_mp_update(const MpBuffers &b, float *gauss, int64_t n, const double *pose, const Raster &r,
                              const float4 *targets, const float *image, const uint8_t *inst, const float *table,

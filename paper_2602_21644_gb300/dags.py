@@ -702,7 +702,7 @@ class Context:
         return loss
 
     def selftest_timeout(self, spins: int = 1000):
-        """Run the failure-path self-test (a bounded wait that runs out); the
+        """Run the failure-path self-test (bounded waits that run out); the
         next check() raises with DAGS_E_TIMEOUT."""
         _check(self.lib.dags_selftest_timeout(self.h, int(spins), _stream()), "dags_selftest_timeout")
 
