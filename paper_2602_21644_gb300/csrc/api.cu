@@ -529,8 +529,9 @@ int splat_backward(dags_ctx *ctx, const float *gauss, int64_t n, const dags_came
   const bool full = (grad_flags & DAGS_GRAD_GAUSS) != 0;
   KernelTimer &tm = ctx->timer;
   int ev = tm.begin(DAGS_K_RENDER_BWD, s);
-  cudaError_t e = launch_render_bwd(backward_workspace(ctx, r), n_views, n, r, l, reinterpret_cast<const float4 *>(targets),
-                                    image, last, full, (grad_flags & DAGS_GRAD_POSE) != 0, s);
+  cudaError_t e = launch_render_bwd(backward_workspace(ctx, r), n_views, n, r, l,
+                                    reinterpret_cast<const float4 *>(targets), image, last, full,
+                                    (grad_flags & DAGS_GRAD_POSE) != 0, s);
   tm.end(ev, s);
   if (e == cudaSuccess) {
     ev = tm.begin(DAGS_K_PREPROCESS_BWD, s);
@@ -565,7 +566,8 @@ int splat_backward_upstream(dags_ctx *ctx, const float *gauss, int64_t n, const 
   const bool full = (grad_flags & DAGS_GRAD_GAUSS) != 0;
   KernelTimer &tm = ctx->timer;
   int ev = tm.begin(DAGS_K_RENDER_BWD, s);
-  cudaError_t e = launch_render_bwd(backward_workspace(ctx, r), n_views, n, r, l, nullptr, image, last, full, (grad_flags & DAGS_GRAD_POSE) != 0, s, grad_image);
+  cudaError_t e = launch_render_bwd(backward_workspace(ctx, r), n_views, n, r, l, nullptr, image, last, full,
+                                    (grad_flags & DAGS_GRAD_POSE) != 0, s, grad_image);
   tm.end(ev, s);
   if (e == cudaSuccess) {
     ev = tm.begin(DAGS_K_PREPROCESS_BWD, s);

@@ -260,11 +260,6 @@ __device__ __forceinline__ bool arrive_last(uint32_t *counter, uint32_t count) {
   return __shfl_sync(0xffffffffu, t, 0) == count - 1u;
 }
 
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-
 // One warp, and one CTA, per 8 x 4 pixel block, as in the adjoint of the
 // first-order loop: bound by the latency of a warp's own chain (59% of the
 // issue slots used, FP32 pipe next) and by the number of warps that 30 tangent

@@ -78,11 +78,6 @@ __device__ __forceinline__ float moment_sums(const float (&x)[K], float dy, int 
 // gradients: 74 -> 66 us; 2,000 Gaussians, 160x120: 60 -> 42 us.
 constexpr int kBlocks = kTilePix / 32;   // pixel blocks per tile
 
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-
 template <bool FULL, bool MOMENTS, bool MASKS, bool COUNT>
 __global__ void __launch_bounds__(32, 32)
 render_bwd_kernel(Workspace ws, Raster r, Loss l, const float4 *__restrict__ targets,
