@@ -118,7 +118,9 @@ void dags_default_pose_cfg(dags_pose_cfg *cfg);
  * larger of 16 * max_gaussians * max_views and min(max_gaussians, 4096) *
  * tiles * max_views, so that splat_track's fixed-capacity tile buckets hold
  * at least min(max_gaussians, 4096) entries each). Allocates device memory
- * (cudaMalloc).
+ * (cudaMalloc), among it, per view, 124 bytes per Gaussian (projected record
+ * 64, 2D gradients 48, tile range 8, visible id 4) and 1 KB per 16x16 tile
+ * (which list entries the last forward's pixels took, for its adjoint).
  * Returns DAGS_E_INVAL / DAGS_E_NOMEM / DAGS_E_CUDA on failure (*out = NULL). */
 int dags_create(dags_ctx **out, int64_t max_gaussians, int32_t max_width, int32_t max_height,
                 int32_t max_views, int64_t max_pairs);
@@ -289,9 +291,10 @@ int gauss_adam_step(dags_ctx *ctx, float *gauss, int64_t n, float *colour, float
  * iterations); (re)capturing synchronises `stream` first. A tile whose list
  * exceeds its bucket is reported by dags_sync_status as DAGS_E_CAPACITY with
  * the max_pairs that would hold every bucket (the longest list times the
- * tiles); the iteration's outputs are then undefined. A splat_backward or
- * dags_copy_bins after splat_track returns DAGS_E_ORDER (no forward of its
- * own precedes it). */
+ * tiles); the iteration's outputs are then undefined. The loop takes the place
+ * of the ctx's last forward, whether it is enqueued or replayed (unless iters
+ * is 0): a splat_backward after it returns DAGS_E_ORDER, a dags_copy_bins
+ * DAGS_E_INVAL. */
 int splat_track(dags_ctx *ctx, const float *gauss, int64_t n, const dags_camera *cam, double *pose,
                 const float *targets, const dags_raster_cfg *rcfg, const dags_loss_cfg *lcfg,
                 const dags_pose_cfg *pcfg, int32_t iters, double *adam_state, float *image, int32_t *last,
@@ -611,9 +614,11 @@ int mpnet_infer(dags_ctx *ctx, const void *weights, const uint16_t *feats, int32
  * feats as for mpnet_infer; target device float [batch][height][width],
  * negative = pixel excluded; loss device double (written: the loss at the
  * weights before the step); grad_out device float [DAGS_MPNET_PARAMS] or
- * NULL. Scratch of 2 + 2 * 96 + 2 * 32 bytes per pixel is owned by the ctx
- * and grows on demand (synchronising the stream); the call is not
- * capturable when it grows. lr >= 0. Errors: DAGS_E_INVAL for NULL or
+ * NULL. Scratch is owned by the ctx and grows on demand (synchronising the
+ * stream); the call is not capturable when it grows. It takes 4 bytes per pixel
+ * and 256 bytes per pixel of rows padded to a multiple of 128 pixels plus two:
+ * 261 bytes per pixel at 640 wide, 417 at 160, 512 at 130, and 4 + 33,280 /
+ * width below 128. lr >= 0. Errors: DAGS_E_INVAL for NULL or
  * unaligned buffers or bad sizes, DAGS_E_NOMEM, DAGS_E_CUDA. */
 #define DAGS_MPNET_PARAMS 10881
 int mpnet_train_step(dags_ctx *ctx, void *weights, float *master, float *adam_m, float *adam_v, int32_t step,

@@ -12,7 +12,7 @@ namespace dags {
 constexpr int kTile = 16;               // tile edge in pixels
 constexpr int kTilePix = kTile * kTile; // pixels (= threads) per render CTA
 constexpr int kGradWords = 12;          // per (view, Gaussian) 2D gradient slots
-constexpr int kSortSmallCap = 1024;     // tile lists up to this length are sorted by the render CTA
+constexpr int kSortSmallCap = 1024;     // tile lists up to this length are sorted in shared memory
 constexpr int kPrepBlock = 128;         // threads per preprocess / emit CTA
 constexpr int kBwdPrepBlock = 128;      // threads per preprocess-backward CTA
 constexpr int kMaskGroups = 32;         // list groups of 32 entries with a recorded forward mask (1024 entries)

@@ -20,12 +20,11 @@
 //                         pixel the loss and W J J^T, W r J; summed per block
 //                         and tile in FP32 and over tiles in FP64, each in a
 //                         fixed order, into (L, H, g)
-//   LM step               FP64, one thread on shared-memory copies: accept the
-//                         linearisation point if its loss is lower, adapt the
-//                         damping, solve the damped 6x6 system by Cholesky and
-//                         step the pose; inside the tracking loop it runs in
-//                         the last warp of render_jac_kernel, on its own as
-//                         lm_step_kernel
+//   LM step               FP64, one warp: accept the linearisation point if its
+//                         loss is lower, adapt the damping, solve the damped
+//                         6x6 system by Cholesky and step the pose, spread over
+//                         the lanes; inside the tracking loop it is the last
+//                         warp of render_jac_kernel, on its own lm_step_kernel
 //
 // The kernels use programmatic dependent launch like the other splatting
 // kernels: each waits for its predecessor's memory before its first access.
@@ -266,11 +265,10 @@ __device__ __forceinline__ bool arrive_last(uint32_t *counter, uint32_t count) {
 // accumulators per pixel leave room for (20 per SM at 96 registers; 24 spill
 // and are slower, as are 16 and 18). The six twist directions run in pairs on
 // the packed FP32 operations, so a pair's 84 operations issue as 42. 300k
-// Gaussians, 640x480, per launch: 146 us with a CTA of 8 warps per tile that
-// sorts its bucket, scalar (93M warp instructions) or packed (77M, the same
-// time: the tile's CTAs wait on one another); 129 us with a warp per block and
-// the sort beside the tangents (60M); 125 with the sums and the step spread
-// over warps and lanes; 121 with the next entry read ahead.
+// Gaussians, 640x480, per launch: 122 us and 64M warp instructions; 146 us with
+// a CTA of 8 warps per tile that sorts its bucket, scalar (93M) or packed (77M:
+// its warps wait on one another). The sort went beside the tangents, the sums
+// and the step over warps and lanes, and the next entry is read ahead.
 __global__ void __launch_bounds__(32, 20)
 render_jac_kernel(Workspace ws, Raster r, Loss l, float delta, const float4 *__restrict__ targets,
                   const float4 *__restrict__ tan, LmBuffers buf, double *__restrict__ normal,

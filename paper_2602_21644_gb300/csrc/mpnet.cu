@@ -169,8 +169,8 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 //     s mod 3: a2 into its buffer).
 // The product runs on the tensor core while epilogues 1 and 3 run, the next
 // step's z1 while epilogues 3 and 2 do, so a step begins with its z1 done (it
-// had waited 1,200 of its 3,700 cycles; 16 x 640 x 480: 169 -> 152 us with the
-// even split of the rows). Every buffer is rewritten only after the barrier that follows its last reader:
+// had waited 1,200 of its 3,700 cycles). Every buffer is rewritten only after
+// the barrier that follows its last reader:
 // the a1 buffer s mod 2 was last read by the product of step s - 1, which
 // the commits of step s cover; the a2 buffer by the z3 of step s; a slot
 // is re-biased one step after epilogue 2 read it. Out-of-image rows and
@@ -243,9 +243,10 @@ struct FwdUnits {
 };
 
 // kSave: the activations are kept, pixel-major for a caller (acts) or in
-// planes for the training step (a warp stores 512 contiguous bytes per chunk;
-// 16 x 640 x 480 with 192-byte rows per pixel: 341 us, with planes 255 us, of
-// which 153 us are the bytes' time). Without: 137 us.
+// planes for the training step (a warp stores 512 contiguous bytes per chunk).
+// 16 x 640 x 480: 137 us without (169 with z1 ahead of each step, uneven rows
+// and the stores' code in the way), 255 with planes, of which 153 are the
+// bytes' time (341 with 192-byte rows per pixel).
 template <bool kSave>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 mpnet_fwd_kernel(const __grid_constant__ CUtensorMap in_map, const uint8_t *__restrict__ weights, int batch, int W,

@@ -681,7 +681,7 @@ preprocess_bwd_kernel(Workspace ws, const float4 *__restrict__ gauss, int64_t n,
 // entries: 59 against 66 us) and no less exact: against 64 bits the twist of
 // 2,000 Gaussians is 2.5e-7 off from moments and 2.9e-7 from words per pixel
 // (means of six scenes), that of discs seen edge-on with a standard deviation
-// of 2 to 110 px 1e-6 .. 1e-5 and 1e-6 .. 5e-4. But the two differ by what
+// of 2 to 110 px 1e-6 .. 1e-5 and 1e-6 .. 7e-4. But the two differ by what
 // either is off, 3e-7 there and 4e-8 on the 300k frame, three times what the
 // order of the atomics does, and a caller of both takes the twist as FP64:
 // those results stay as they were.
