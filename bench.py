@@ -260,10 +260,11 @@ def kernel_bytes(n, nv, K, P):
 # (alpha >= alpha_min): forward alpha, its clamp, 1 - alpha, the new T and its
 # test, the weight and six accumulations (12); backward alpha, its clamp,
 # 1/(1 - alpha), the transmittance recovery, the weight, dL/dalpha over six
-# channels with its suffix term, the chain to centre, conic and depth, the
-# suffix update and the warp sums of the six gradient words (39). The
-# evaluation and contribution counts are counted by the kernels themselves.
-OPS_EVAL, OPS_FWD_CONTRIB, OPS_BWD_CONTRIB = 9, 12, 39
+# channels with its suffix term, the four terms g, g e, g e^2 and the depth's
+# (the conic's shear included), the suffix update and the warp sums of the four
+# (27; the factors of y are applied to the sums of rows). The evaluation and
+# contribution counts are counted by the kernels themselves.
+OPS_EVAL, OPS_FWD_CONTRIB, OPS_BWD_CONTRIB = 9, 12, 27
 # special-function operations per contribution: forward exp2; backward exp2
 # and the reciprocal of 1 - alpha
 SFU_FWD_CONTRIB, SFU_BWD_CONTRIB = 1, 2
@@ -981,8 +982,8 @@ def run_ours(args):
     iter_us = 1e3 * t_ms / (args.iters * args.steps)
     # kernels per step: per iteration the preprocess (with direct binning),
     # the forward, the adjoint and the pose chain (pose step fused); per frame
-    # the culling and the MP update's 9 kernels (pixel sum, pixel var, pixel map, gauss,
-    # apply, 2 select levels, labels, region stats)
+    # the culling and the MP update's 5 kernels (pixel sum, pixel var, pixel map,
+    # gauss, apply)
     gpu_launches = args.steps * (args.iters * 4 + 5 + 1)   # + the frame's culling
     line = {"metric": METRIC, "value": round(value, 2), "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": round(t_ms / args.steps, 4), "higher_is_better": True,
